@@ -189,8 +189,8 @@ int fa_apply_A(fa_ctx* ctx, const double* in, double* out, int dagger, int preci
  * a CUDA graph under global stream-capture mode (where cudaMalloc is refused)
  * or code whose device memory is owned by a framework allocator or a fixed
  * budget.  The paper has no counterpart; this is a library convenience.
- * The two working spinors live in one static device array sized for at most
- * 8192 sites (3 MiB, resident on every GPU that loads the library until the
+ * The working spinor lives in one static device array sized for at most
+ * 8192 sites (1.5 MiB, resident on every GPU that loads the library until the
  * process exits); larger lattices return FA_EINVAL.  The first call on a
  * device looks up that array's device address (make it before any stream
  * capture); the context's device must be current.  All calls share the array,

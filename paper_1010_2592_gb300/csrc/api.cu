@@ -323,19 +323,17 @@ static int apply_op(fa_ctx* c, const double* in, double* out, int dagger, int pr
     const bool dg = dagger != 0;
     if (precision == FA_F64) {
         const size_t b = (size_t)12 * V * sizeof(double2);
-        CUDA_OR(c->io64a.ensure(b), "alloc");
-        CUDA_OR(c->io64b.ensure(b), "alloc");
-        double2 *a = c->io64a.as<double2>(), *o = c->io64b.as<double2>();
-        TRY(launch_pack_spinor_f64(c->g, in, a, st));
+        // the FP64 sweeps read and write the canonical layout themselves: they are bound
+        // by the FP64 pipe, which hides the strided loads
         if (is_A) {
             CUDA_OR(c->tmp64.ensure(b), "alloc");
-            double2* t = c->tmp64.as<double2>();
-            TRY(hop_f64(c, a, t, 1.0, false, true, dg, nullptr, nullptr, nullptr));
-            TRY(hop_f64(c, t, o, c->scale_c, false, true, dg, nullptr, nullptr, nullptr));
+            const View64 t = internal64(c->tmp64.as<double2>(), V);
+            TRY(hop_f64(c, canonical64(in), t, 1.0, false, true, dg));
+            TRY(hop_f64(c, t, canonical64(out), c->scale_c, false, true, dg));
         } else {
-            TRY(hop_f64(c, a, o, 1.0, dg, dg, dg, nullptr, nullptr, nullptr));
+            TRY(hop_f64(c, canonical64(in), canonical64(out), 1.0, dg, dg, dg));
         }
-        TRY(launch_unpack_spinor_f64(c->g, o, out, st));
+        return FA_OK;
     } else if (precision == FA_F32) {
         const size_t b = (size_t)6 * V * sizeof(float4);
         CUDA_OR(c->io32a.ensure(b), "alloc");

@@ -14,6 +14,7 @@
 // left to L1/L2 (the 126 MB L2 holds several time slices of every field even
 // on 32^3 x 64).  Memory traffic floor per site and sweep: one spinor in, one
 // out, four links (FP32: 96 + 96 + 4 * 48 = 384 B).
+#include "hop64.cuh"
 #include "hop_device.cuh"
 
 namespace fa {
@@ -69,49 +70,36 @@ hop_rows_kernel(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cd
     if (DOT) block_reduce_store<1, R, kRowThreads>(dres, partials, 0, blockIdx.x);
 }
 
-template <typename R, typename LP, typename SP>
-static int launch_hop_t(const Geom& g, const LP* links, const SP* in, SP* out, double diag, double ef,
-                        double eb, double t_bc, double scale, bool g5in, bool g5out, const SP* dot_with,
-                        double2* partials, const int* done, cudaStream_t st, int shape = 0) {
-    LinkView<R> U{links, g.V};
-    SpinorView<R> vin{const_cast<SP*>(in), g.V};
-    SpinorView<R> vout{out, g.V};
-    SpinorView<R> vd{const_cast<SP*>(dot_with), g.V};
-    const R cdiag = (R)(scale * diag), chop = (R)(-0.5 * scale);
-    const R ref = (R)ef, reb = (R)eb, rbc = (R)t_bc;
-    const bool dot = dot_with != nullptr;
-    if constexpr (std::is_same<R, float>::value) {
-      if (hop_use_narrow(shape, g.V)) {
-        constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks;
-        const int nb = (g.V + NT - 1) / NT;
-#define FA_HOPN(A, B, C) hop_kernel<R, A, B, C, NT, MB><<<nb, NT, 0, st>>>(g, U, vin, vout, cdiag, chop, ref, reb, rbc, vd, partials, done)
-        if (!g5in && !g5out && !dot) FA_HOPN(false, false, false);
-        else if (!g5in && g5out && !dot) FA_HOPN(false, true, false);
-        else if (!g5in && g5out && dot) FA_HOPN(false, true, true);
-        else if (g5in && g5out && !dot) FA_HOPN(true, true, false);
-        else if (!g5in && !g5out && dot) FA_HOPN(false, false, true);
-        else return FA_EINVAL;
-#undef FA_HOPN
-        return launch_status("hop kernel");
-      }
-    }
-    const int nb = nblocks(g.V);
-#define FA_HOP(A, B, C) hop_kernel<R, A, B, C><<<nb, kThreads, 0, st>>>(g, U, vin, vout, cdiag, chop, ref, reb, rbc, vd, partials, done)
-    if (!g5in && !g5out && !dot) FA_HOP(false, false, false);
-    else if (!g5in && g5out && !dot) FA_HOP(false, true, false);
-    else if (!g5in && g5out && dot) FA_HOP(false, true, true);
-    else if (g5in && g5out && !dot) FA_HOP(true, true, false);
-    else if (!g5in && !g5out && dot) FA_HOP(false, false, true);
-    else return FA_EINVAL;
-#undef FA_HOP
-    return launch_status("hop kernel");
+// FP64: a tile of 32 sites per block or cluster (hop64.cuh).  CANON: canonical
+// output, staged in shared memory (a thread of phase 2 holds one real number of
+// every 192-byte record, so direct stores would write 8 bytes per 32-byte sector).
+template <int C, bool CANON>
+__global__ void __launch_bounds__(hop64_threads<C>(), hop64_min_blocks<C>())
+hop64_kernel(Geom g, const double2* __restrict__ U, View64 in, View64 out, Op64 op, const int* done) {
+    if (done != nullptr && *done) return;
+    __shared__ Smem64<C> sm;
+    const int tile = blockIdx.x / C, rank = blockIdx.x % C;
+    hop64_tile<C, !CANON, CANON>(g, U, in, out, op, tile, rank, sm);
+    if (CANON && rank == 0) store_canonical<C>(out.p, g.V, tile, sm);
 }
 
-int launch_hop_f64(const Geom& g, const double2* links, const double2* in, double2* out, double diag,
-                   double ef, double eb, double t_bc, double scale, bool g5in, bool g5out,
-                   const double2* dot_with, double2* partials, const int* done, cudaStream_t st) {
-    return launch_hop_t<double>(g, links, in, out, diag, ef, eb, t_bc, scale, g5in, g5out, dot_with,
-                                partials, done, st);
+template <int C>
+static int launch_hop64(const Geom& g, const double2* links, const View64& in, const View64& out, const Op64& op,
+                        const int* done, cudaStream_t st) {
+    const dim3 grid(tiles64(g.V) * C);
+    if (out.ks == 1) launch_ex(false, C, hop64_kernel<C, true>, grid, hop64_threads<C>(), st, g, links, in, out, op, done);
+    else launch_ex(false, C, hop64_kernel<C, false>, grid, hop64_threads<C>(), st, g, links, in, out, op, done);
+    return launch_status("FP64 hop kernel");
+}
+
+int launch_hop_f64(const Geom& g, const double2* links, const View64& in, const View64& out, double diag, double ef,
+                   double eb, double t_bc, double scale, bool g5in, bool g5out, const int* done, cudaStream_t st) {
+    const Op64 op{scale * diag, -0.5 * scale, ef, eb, t_bc, g5in ? 1 : 0, g5out ? 1 : 0};
+    switch (hop64_split(g.V, sm_count())) {
+        case 1: return launch_hop64<1>(g, links, in, out, op, done, st);
+        case 2: return launch_hop64<2>(g, links, in, out, op, done, st);
+        default: return launch_hop64<4>(g, links, in, out, op, done, st);
+    }
 }
 
 int launch_hop_df(const Geom& g, const float4* links, const float4* in, float4* out, double diag, double ef,
@@ -139,8 +127,29 @@ int launch_hop_df(const Geom& g, const float4* links, const float4* in, float4* 
 int launch_hop_f32(const Geom& g, const float4* links, const float4* in, float4* out, double diag,
                    double ef, double eb, double t_bc, double scale, bool g5in, bool g5out,
                    const float4* dot_with, double2* partials, const int* done, cudaStream_t st, int shape) {
-    return launch_hop_t<float>(g, links, in, out, diag, ef, eb, t_bc, scale, g5in, g5out, dot_with,
-                               partials, done, st, shape);
+    LinkView<float> U{links, g.V};
+    SpinorView<float> vin{const_cast<float4*>(in), g.V};
+    SpinorView<float> vout{out, g.V};
+    SpinorView<float> vd{const_cast<float4*>(dot_with), g.V};
+    const float cdiag = (float)(scale * diag), chop = (float)(-0.5 * scale);
+    const float ref = (float)ef, reb = (float)eb, rbc = (float)t_bc;
+    const bool dot = dot_with != nullptr;
+    const bool narrow = hop_use_narrow(shape, g.V);
+    const int nt = narrow ? kHopNarrowThreads : kThreads;
+    const int nb = (g.V + nt - 1) / nt;
+#define FA_HOPS(A, B, C)                                                                                              \
+    (narrow ? hop_kernel<float, A, B, C, kHopNarrowThreads, kHopNarrowBlocks><<<nb, nt, 0, st>>>(                     \
+                  g, U, vin, vout, cdiag, chop, ref, reb, rbc, vd, partials, done)                                    \
+            : hop_kernel<float, A, B, C><<<nb, nt, 0, st>>>(g, U, vin, vout, cdiag, chop, ref, reb, rbc, vd, partials, \
+                                                            done))
+    if (!g5in && !g5out && !dot) FA_HOPS(false, false, false);
+    else if (!g5in && g5out && !dot) FA_HOPS(false, true, false);
+    else if (!g5in && g5out && dot) FA_HOPS(false, true, true);
+    else if (g5in && g5out && !dot) FA_HOPS(true, true, false);
+    else if (!g5in && !g5out && dot) FA_HOPS(false, false, true);
+    else return FA_EINVAL;
+#undef FA_HOPS
+    return launch_status("hop kernel");
 }
 
 // ------------------------------------------------------------------ link force (adjoint)

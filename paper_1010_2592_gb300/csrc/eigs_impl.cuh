@@ -219,31 +219,15 @@ int lincomb(Dev& D, const double2* V, int k, const std::vector<zc>& coef, const 
 
 }  // namespace
 
-static int ok_alloc(fa_ctx* c, size_t sb);
-
 // w = T v = c H A^{-1} v at chemical potential `mu` (canonical spinors); y is scratch
 static int apply_T(fa_ctx* c, double mu, const double* v, double* w, double* y, const fa_solver_params* ps) {
     const double mu0 = c->mu;
     c->mu = mu;
     fa_solver_stats st{};
     int rc = solve(c, v, y, nullptr, ps, &st);   // A^{-1} v (poles: omega = 1, sigma = 0)
-    if (rc == FA_OK) {
-        const size_t sb = (size_t)12 * c->g.V * sizeof(double2);
-        rc = ok_alloc(c, sb);
-        if (rc == FA_OK) rc = launch_pack_spinor_f64(c->g, y, c->io64a.as<double2>(), c->stream);
-        if (rc == FA_OK)
-            rc = hop_f64(c, c->io64a.as<double2>(), c->io64b.as<double2>(), c->scale_c, false, true, false, nullptr,
-                         nullptr, nullptr);
-        if (rc == FA_OK) rc = launch_unpack_spinor_f64(c->g, c->io64b.as<double2>(), w, c->stream);
-    }
+    if (rc == FA_OK) rc = hop_f64(c, canonical64(y), canonical64(w), c->scale_c, false, true, false);
     c->mu = mu0;
     return rc;
-}
-
-static int ok_alloc(fa_ctx* c, size_t sb) {
-    cudaError_t e = c->io64a.ensure(sb);
-    if (e == cudaSuccess) e = c->io64b.ensure(sb);
-    return e == cudaSuccess ? FA_OK : cuda_fail(e, "alloc");
 }
 
 // Krylov-Schur on T at chemical potential mu: the k eigenvalues of T largest in

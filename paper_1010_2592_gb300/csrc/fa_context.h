@@ -5,7 +5,7 @@
 #include <vector>
 #include <string>
 
-#include "fa_internal.cuh"
+#include "hop64.cuh"
 
 struct fa_ctx;
 
@@ -123,8 +123,7 @@ inline const float4* linksdf_of(const fa_ctx* c) {
     return c->links_owner ? c->links_owner->linksdf.as<float4>() : c->linksdf.as<float4>();
 }
 // operator application on internal layouts (used by the C-ABI and the solver)
-int hop_f64(fa_ctx* c, const double2* in, double2* out, double scale, bool g5in, bool g5out, bool dagger_mu,
-            const double2* dot_with, double2* partials, const int* done);
+int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g5in, bool g5out, bool dagger_mu);
 int hop_f32(fa_ctx* c, const float4* in, float4* out, double scale, bool g5in, bool g5out, bool dagger_mu,
             const float4* dot_with, double2* partials, const int* done);
 int hop_df(fa_ctx* c, const float4* in, float4* out, double scale, bool g5in, bool g5out, bool dagger_mu,

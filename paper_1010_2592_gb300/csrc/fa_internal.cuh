@@ -396,13 +396,10 @@ inline int launch_status(const char* what) {
 }
 
 // Hop (one D_w sweep): out = scale * G5OUT * (diag*in' - 1/2 sum hops(in')),
-// in' = G5IN ? gamma_5 in : in, time weights from `mu_sign` * mu.
+// in' = G5IN ? gamma_5 in : in, time weights from `mu_sign` * mu (the FP64
+// sweep, launch_hop_f64, is declared in hop64.cuh).
 // When dot_with != nullptr, per-block partials of <dot_with, out> are written
 // to partials[blockIdx] (nblk = ceil(V/kThreads) of them).
-int launch_hop_f64(const Geom& g, const double2* links, const double2* in, double2* out,
-                   double diag, double ef, double eb, double t_bc, double scale,
-                   bool g5in, bool g5out, const double2* dot_with, double2* partials,
-                   const int* done, cudaStream_t st);
 // shape: 0 narrow when the lattice fits one wave of it, 1 wide (kThreads x
 // FA_HOP_MINB per SM), 2 narrow (kHopNarrowThreads x kHopNarrowBlocks per SM)
 int launch_hop_f32(const Geom& g, const float4* links, const float4* in, float4* out,

@@ -7,12 +7,12 @@
 // framework's caching allocator or a fixed budget wants no hidden
 // cudaMalloc/cudaFree that could fail or fragment that budget.  fa_apply_A
 // grows per-context scratch buffers on first use; this variant instead keeps
-// its two working spinors in one file-scope device array whose size is fixed
-// when the library is loaded.
+// its working spinor in one file-scope device array whose size is fixed when
+// the library is loaded.
 //
 // Limits: lattices up to kNoAllocMaxSites = 8192 sites (8^3 x 16); larger
 // ones are rejected with FA_EINVAL before any device work.  The array
-// (2 x 12 x 8192 complex doubles = 3 MiB) is resident on every GPU that loads
+// (12 x 8192 complex doubles = 1.5 MiB) is resident on every GPU that loads
 // the library until the process exits.  All calls share it: calls that
 // overlap on a GPU (other streams, other contexts on the same device) race
 // on it and must be serialised by the caller.  Nothing in it needs clearing
@@ -27,8 +27,8 @@ namespace fa {
 constexpr int kNoAllocMaxSites = 8192;
 constexpr int kNoAllocMaxDevices = 64;
 
-// two internal-layout FP64 spinors: [2][12][kNoAllocMaxSites] double2
-static __device__ __align__(256) double2 g_noalloc_scratch[2 * 12 * kNoAllocMaxSites];
+// an internal-layout FP64 spinor: [12][kNoAllocMaxSites] double2
+static __device__ __align__(256) double2 g_noalloc_scratch[12 * kNoAllocMaxSites];
 
 // Device address of g_noalloc_scratch per device, resolved once per device
 // with that device current.  In host code the symbol itself is only a
@@ -76,21 +76,17 @@ extern "C" int fa_apply_A_noalloc(fa_ctx* c, const double* in, double* out, int 
     double2* scratch = nullptr;
     int rc = scratch_address(dev, &scratch);
     if (rc != FA_OK) return rc;
-    double2* a = scratch;                                   // packed input, later the packed result
-    double2* t = scratch + (size_t)12 * kNoAllocMaxSites;   // g5 D in
+    const View64 t = internal64(scratch, c->g.V);   // g5 D in
     // A = c g5 D g5 D; A^H = A(-mu).  The hop kernels are launched directly,
     // so the call leaves the context's solver state and timing untouched.
     const double mu = dagger != 0 ? -c->mu : c->mu;
     const double ef = std::exp(mu), eb = std::exp(-mu), diag = 4.0 + c->mass;
-    rc = launch_pack_spinor_f64(c->g, in, a, c->stream);
+    rc = launch_hop_f64(c->g, links64_of(c), canonical64(in), t, diag, ef, eb, c->t_bc, 1.0, false, true, nullptr,
+                        c->stream);
     if (rc == FA_OK)
-        rc = launch_hop_f64(c->g, links64_of(c), a, t, diag, ef, eb, c->t_bc, 1.0, false, true, nullptr, nullptr,
+        rc = launch_hop_f64(c->g, links64_of(c), t, canonical64(out), diag, ef, eb, c->t_bc, c->scale_c, false, true,
                             nullptr, c->stream);
-    if (rc == FA_OK)
-        rc = launch_hop_f64(c->g, links64_of(c), t, a, diag, ef, eb, c->t_bc, c->scale_c, false, true, nullptr,
-                            nullptr, nullptr, c->stream);
-    if (rc == FA_OK) rc = launch_unpack_spinor_f64(c->g, a, out, c->stream);
     if (rc != FA_OK) return rc;   // the launch error is recorded for fa_last_error
-    c->launches += 4;
+    c->launches += 2;
     return FA_OK;
 }

@@ -68,12 +68,11 @@ static void hop_timing_collect(fa_ctx* c, int m_run = 1 << 30) {
     c->hop_ev_used = 0;
 }
 
-int hop_f64(fa_ctx* c, const double2* in, double2* out, double scale, bool g5in, bool g5out, bool dagger_mu,
-            const double2* dot_with, double2* partials, const int* done) {
+int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g5in, bool g5out, bool dagger_mu) {
     const double mu = dagger_mu ? -c->mu : c->mu;
-    hop_timing_begin(c, 0 + (dot_with ? 3 : 0));
-    int rc = launch_hop_f64(c->g, links64_of(c), in, out, 4.0 + c->mass, std::exp(mu), std::exp(-mu),
-                            c->t_bc, scale, g5in, g5out, dot_with, partials, done, c->stream);
+    hop_timing_begin(c, 0);
+    int rc = launch_hop_f64(c->g, links64_of(c), in, out, 4.0 + c->mass, std::exp(mu), std::exp(-mu), c->t_bc, scale,
+                            g5in, g5out, nullptr, c->stream);
     hop_timing_end(c);
     c->launches++;
     return rc;
@@ -101,11 +100,11 @@ int hop_df(fa_ctx* c, const float4* in, float4* out, double scale, bool g5in, bo
     return rc;
 }
 
-// A v = c g5 D g5 D v through the scratch spinor tmp; optional <dot_with, A v> partials.
-static int apply_A_64(fa_ctx* c, const double2* in, double2* out, double2* tmp, const double2* dot_with,
-                      double2* partials, const int* done, double scale) {
-    FA_TRY(hop_f64(c, in, tmp, 1.0, false, true, false, nullptr, nullptr, done));
-    return hop_f64(c, tmp, out, scale, false, true, false, dot_with, partials, done);
+// A v = c g5 D g5 D v through the scratch spinor tmp
+static int apply_A_64(fa_ctx* c, const double2* in, double2* out, double2* tmp, double scale) {
+    const int V = c->g.V;
+    FA_TRY(hop_f64(c, internal64(in, V), internal64(tmp, V), 1.0, false, true, false));
+    return hop_f64(c, internal64(tmp, V), internal64(out, V), scale, false, true, false);
 }
 // ------------------------------------------------------------------ small FP64 kernels
 __global__ void k_sc_invnorm(const double2* part, int nblk, double* out) {
@@ -202,7 +201,7 @@ static int ensure_workspace(fa_ctx* c, const Layout& Lo) {
     // the Gram epilogue of the FP32 sweep writes n_gram(l) partials per block
     const size_t hop_blk = (size_t)std::max(nblocks(V), (V + kHopNarrowThreads - 1) / kHopNarrowThreads) + 1;
     FA_CUDA(c->partials.ensure(std::max({(size_t)std::max({Lo.nblk, Lo.red_grid, Lo.vgrid + 1}) * Lo.part_slots,
-                                         (size_t)row_blocks(V), hop_blk * (size_t)Lo.part_slots}) *
+                                         (size_t)row_blocks(V), (size_t)tiles64(V), hop_blk * (size_t)Lo.part_slots}) *
                                sizeof(double2)),
             "alloc partials");
     FA_CUDA(c->state.ensure(sizeof(DevState)), "alloc state");
@@ -329,23 +328,12 @@ struct Batch {
 };
 
 
-// Kernel launch, with programmatic stream serialization when `pdl` is set: the
-// kernel may then be placed on the SMs while its predecessor (a kernel) finishes,
-// and it waits in dep_sync() before its first memory access.  Used only for
-// kernels that call dep_sync() first and follow another kernel in the stream.
+// Launch inside an outer iteration: with `pdl`, programmatic stream
+// serialization (only for kernels that call dep_sync() first and follow
+// another kernel in the stream).
 template <typename... KArgs, typename... Args>
 static void launch(bool pdl, void (*k)(KArgs...), dim3 grid, int block, cudaStream_t st, Args... args) {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl ? 1 : 0;
-    (void)cudaLaunchKernelEx(&cfg, k, args...);   // errors surface through cudaGetLastError
+    launch_ex(pdl, 1, k, grid, block, st, args...);
 }
 
 static int upload(Batch& B) {
@@ -370,7 +358,7 @@ template <typename R> constexpr int rp_of() {
 template <typename R, int L>
 static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reliable) {
     fa_ctx* c = B.c0;
-    const int n = B.n, nb = B.Lo.nblk, rg = B.Lo.red_grid, vg = B.Lo.vgrid;
+    const int n = B.n, rg = B.Lo.red_grid, vg = B.Lo.vgrid;
     const int p2 = pass2 ? 1 : 0;
     // The vector kernels run vg blocks (one site per thread while the lattice
     // fits one wave); their XS variants add the shift block, which finishes
@@ -378,7 +366,7 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     // sites for 256 threads, a second pass for one thread of every block).
     // k_gram / k_mr use vg where their register budget gives kVecBlocks
     // resident blocks per SM, else the reduction grid.
-    dim3 gs(nb, n), gv(vg, n), gvx(vg + 1, n);
+    dim3 gv(vg, n), gvx(vg + 1, n);
     const bool gram_vec = gram_min_blocks<R, L>() >= kVecBlocks, mr_vec = mr_min_blocks<R, L>() >= kVecBlocks;
     dim3 gg(gram_vec ? vg : rg, n);
     const int mg = mr_vec ? vg : rg;
@@ -436,22 +424,33 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
                 else
                     launch(pdl, k_hop1_rows<R, false>, nbh, kRowThreads, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
                                                                         vdot, nullptr, done, ds, none);
+            } else if constexpr (rp_of<R>() == RP64) {
+                const Op64 op{cdiag, chop, ef, eb, bc, 0, 1};
+                auto go = [&](auto split) {
+                    constexpr int C = decltype(split)::value;
+                    const dim3 gh(tiles64(V) * C);
+                    if (dot)
+                        launch_ex(pdl, C, k_hop64<C, true>, gh, hop64_threads<C>(), st, h0.g, h0.links64, vin.p, vout.p, op,
+                                  (const double2*)rt, h0.part, done, ds, step);
+                    else
+                        launch_ex(pdl, C, k_hop64<C, false>, gh, hop64_threads<C>(), st, h0.g, h0.links64, vin.p, vout.p, op,
+                                  (const double2*)nullptr, (double2*)nullptr, done, ds, none);
+                };
+                const int split = hop64_split(V, sms());
+                if (split == 1) go(std::integral_constant<int, 1>{});
+                else if (split == 2) go(std::integral_constant<int, 2>{});
+                else go(std::integral_constant<int, 4>{});
             } else {
-                bool narrow = false;
-                if constexpr (rp_of<R>() == RP32) {
-                    if (hop_use_narrow(c->hop_shape, V)) {
-                        narrow = true;
-                        constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks;
-                        const int nbh = (V + NT - 1) / NT;
-                        if (dot)
-                            launch(pdl, k_hop1<R, true, NT, MB>, nbh, NT, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
-                                                                        vdot, h0.part, done, ds, step);
-                        else
-                            launch(pdl, k_hop1<R, false, NT, MB>, nbh, NT, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
-                                                                         vdot, nullptr, done, ds, none);
-                    }
-                }
-                if (!narrow) {
+                if (hop_use_narrow(c->hop_shape, V)) {
+                    constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks;
+                    const int nbh = (V + NT - 1) / NT;
+                    if (dot)
+                        launch(pdl, k_hop1<R, true, NT, MB>, nbh, NT, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
+                                                                    vdot, h0.part, done, ds, step);
+                    else
+                        launch(pdl, k_hop1<R, false, NT, MB>, nbh, NT, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
+                                                                     vdot, nullptr, done, ds, none);
+                } else {
                     const int nbh = nblocks(V);
                     if (dot)
                         launch(pdl, k_hop1<R, true>, nbh, kThreads, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc, vdot,
@@ -497,16 +496,17 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
                             step, tw);
             else launch(pdl, k_hop_sys_rows<R, false>, gw, kRowThreads, st, ds, in_sel, in_j, out_sel, out_j, second, p2,
                         none, tw);
-        } else {
+        } else if constexpr (rp_of<R>() == RP64) {
+            dim3 gh(tiles64(h0.V), n);
             const int4* th = nullptr;
             if (B.tables) {
-                gs = dim3(B.tab_n[TB_HOP]);
+                gh = dim3(B.tab_n[TB_HOP]);
                 th = B.tab[TB_HOP];
             }
-            if (dot) launch(pdl, k_hop_sys<R, true>, gs, kThreads, st, ds, in_sel, in_j, out_sel, out_j, second, p2, step,
-                            th);
-            else launch(pdl, k_hop_sys<R, false>, gs, kThreads, st, ds, in_sel, in_j, out_sel, out_j, second, p2, none,
-                        th);
+            if (dot) launch(pdl, k_hop64_sys<true>, gh, hop64_threads<1>(), st, ds, in_sel, in_j, out_sel, out_j, second,
+                            p2, step, th);
+            else launch(pdl, k_hop64_sys<false>, gh, hop64_threads<1>(), st, ds, in_sel, in_j, out_sel, out_j, second, p2,
+                        none, th);
         }
         if (timing) hop_timing_end(c);
         FA_LAUNCHED(c, "k_hop_sys");
@@ -590,11 +590,12 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
         double2* t1 = c->io64a.as<double2>();
         double2* t2 = c->io64b.as<double2>();
         const int* done = pass2 ? nullptr : &h0.st->done;
-        int rc = launch_hop_f64(h0.g, h0.links64, h0.x64, t1, h0.diag, h0.ef, h0.eb, h0.bc, 1.0, false, true,
-                                nullptr, nullptr, done, st);
+        const int V = h0.V;
+        int rc = launch_hop_f64(h0.g, h0.links64, internal64(h0.x64, V), internal64(t1, V), h0.diag, h0.ef, h0.eb, h0.bc,
+                                1.0, false, true, done, st);
         if (rc == FA_OK)
-            rc = launch_hop_f64(h0.g, h0.links64, t1, t2, h0.diag, h0.ef, h0.eb, h0.bc, h0.scale, false, true,
-                                nullptr, nullptr, done, st);
+            rc = launch_hop_f64(h0.g, h0.links64, internal64(t1, V), internal64(t2, V), h0.diag, h0.ef, h0.eb, h0.bc,
+                                h0.scale, false, true, done, st);
         c->launches += 2;
         if (rc != FA_OK) return rc;
         k_reliable<R><<<gv, kThreads, 0, st>>>(ds, t2, p2, conv);
@@ -813,7 +814,7 @@ static int build_tables(Batch& B) {
         blocks(t[TB_VECX], i, lo.vgrid, true);
         blocks(t[TB_RG], i, lo.red_grid, false);
         blocks(t[TB_RGX], i, lo.red_grid, true);
-        blocks(t[TB_HOP], i, lo.nblk, false);
+        blocks(t[TB_HOP], i, tiles64(lo.V), false);
         blocks(t[TB_ROWS], i, row_blocks(lo.V), false);
     }
     // lattice groups for the FP32 multi-RHS sweep: systems sharing the packed
@@ -1413,23 +1414,15 @@ int apply_sign(fa_ctx* c, const double* b, double* out, const fa_solver_params* 
                bool overlap) {
     const int rc = solve(c, b, out, nullptr, p, stats);   // out holds y for now
     if (rc != FA_OK) return rc;
-    const int V = c->g.V;
-    const size_t s64 = (size_t)12 * V * sizeof(double2);
+    const int n = 12 * c->g.V;
     cudaStream_t st = c->stream;
-    FA_CUDA(c->io64b.ensure(s64), "alloc");
-    double2* o = c->io64b.as<double2>();
-    FA_TRY(hop_f64(c, c->y64.as<double2>(), o, std::sqrt(c->scale_c), false, !overlap, false, nullptr, nullptr,
-                   nullptr));
+    FA_TRY(hop_f64(c, internal64(c->y64.as<double2>(), c->g.V), canonical64(out), std::sqrt(c->scale_c), false, !overlap,
+                   false));
     if (overlap) {
-        FA_CUDA(c->io64a.ensure(s64), "alloc");
-        double2* bp = c->io64a.as<double2>();
-        FA_TRY(launch_pack_spinor_f64(c->g, b, bp, st));
-        k_add_f64<<<(12 * V + kThreads - 1) / kThreads, kThreads, 0, st>>>(12 * V, bp, o);
-        c->launches++;
+        k_add_f64<<<(n + kThreads - 1) / kThreads, kThreads, 0, st>>>(n, reinterpret_cast<const double2*>(b),
+                                                                      reinterpret_cast<double2*>(out));
         FA_LAUNCHED(c, "k_add_f64");
     }
-    FA_TRY(launch_unpack_spinor_f64(c->g, o, out, st));
-    c->launches++;
     FA_CUDA(cudaStreamSynchronize(st), "sync sign");
     return FA_OK;
 }
@@ -1552,8 +1545,8 @@ int grad(fa_ctx* c, const double* b, const double* eta, double* dLdU, double* dL
         for (int i = 0; i < k && rc == FA_OK; ++i) {
             const double2* xs = gxs + i * vs;
             const double2* ls = lam + i * vs;
-            rc = hop_f64(c, xs, t1, 1.0, false, true, false, nullptr, nullptr, nullptr);   // g5 D x
-            if (rc == FA_OK) rc = hop_f64(c, ls, t2, 1.0, false, false, true, nullptr, nullptr, nullptr);   // D(-mu) lambda
+            rc = hop_f64(c, internal64(xs, V), internal64(t1, V), 1.0, false, true, false);   // g5 D x
+            if (rc == FA_OK) rc = hop_f64(c, internal64(ls, V), internal64(t2, V), 1.0, false, false, true);   // D(-mu) lambda
             if (rc == FA_OK)
                 rc = launch_force(c->g, links64_of(c), ls, t1, t2, xs, dLdU, -c->scale_c * om_all[s0 + i],
                                   std::exp(c->mu), std::exp(-c->mu), c->t_bc, part + (size_t)i * nb, st);
@@ -1639,11 +1632,11 @@ int estimate_scale(fa_ctx* c, const double* v0, int iters, double* scale_out) {
     };
     FA_TRY(normalise(v));
     for (int it = 0; it < iters; ++it) {
-        FA_TRY(apply_A_64(c, v, w, c->tmp64.as<double2>(), nullptr, nullptr, nullptr, 1.0));
+        FA_TRY(apply_A_64(c, v, w, c->tmp64.as<double2>(), 1.0));
         FA_TRY(normalise(w));
         std::swap(v, w);
     }
-    FA_TRY(apply_A_64(c, v, w, c->tmp64.as<double2>(), nullptr, nullptr, nullptr, 1.0));
+    FA_TRY(apply_A_64(c, v, w, c->tmp64.as<double2>(), 1.0));
     k_dot2<double><<<rg, kThreads, 0, st>>>(V, w, w, c->partials.as<double2>());
     FA_LAUNCHED(c, "k_dot2");
     k_sc_invnorm<<<1, kScalarThreads, 0, st>>>(c->partials.as<double2>(), rg, sc);

@@ -22,6 +22,7 @@
 // arithmetic (explicit fma intrinsics, no contraction by the compiler).
 #pragma once
 
+#include "hop64.cuh"
 #include "hop_device.cuh"
 #include "trace.cuh"
 
@@ -391,14 +392,33 @@ __device__ __forceinline__ void recip2(double p, double q, double& ip, double& i
 // otherwise FP64 values summed in FP64.
 template <typename R> constexpr bool dfp_of() { return !std::is_same<R, double>::value; }
 
+// TILES (FP64): the partials are those of 32-site tiles, nblk of them; eight at
+// a time are first added in the order of a warp shuffle tree over eight lanes,
+// and the sums of those 256-site groups are what is split into quarters.
+//
 // dry: warp 0 runs the code of one quarter once, every load predicated off
 // (the sums are 0); the other warps only meet the barriers.
-template <int NSMAX, bool DFP>
+__device__ __forceinline__ double2 tile_group(const double2* pd, int i, int n) {
+    double2 v[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) v[t] = 8 * i + t < n ? __ldcg(pd + 8 * i + t) : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int t = 0; t < o; ++t) {
+            v[t].x = __dadd_rn(v[t].x, v[t + o].x);
+            v[t].y = __dadd_rn(v[t].y, v[t + o].y);
+        }
+    return v[0];
+}
+template <int NSMAX, bool DFP, bool TILES = false>
 __device__ __forceinline__ void reduce_slots(const double2* part, int nblk, int ns, dcx* out, bool dry = false) {
+    static_assert(!(DFP && TILES), "tile partials are FP64");
     __shared__ double2 qs[4 * NSMAX];
     __shared__ float4 qf[4 * NSMAX];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int per = (nblk + 3) >> 2;
+    const int npart = TILES ? (nblk + 7) >> 3 : nblk;
+    const int per = (npart + 3) >> 2;
     const int ntask = dry ? 1 : 4 * ns;
     if (dry && (int)threadIdx.x < 4 * ns) {   // the quarters a dry run leaves out
         qs[threadIdx.x] = make_double2(0.0, 0.0);
@@ -452,7 +472,7 @@ __device__ __forceinline__ void reduce_slots(const double2* part, int nblk, int 
     }
     for (int u = u_first; u < ntask; u += nw) {
         const int k = u >> 2;
-        const int i0 = (u & 3) * per, i1 = dry ? i0 : min(nblk, i0 + per);
+        const int i0 = (u & 3) * per, i1 = dry ? i0 : min(npart, i0 + per);
         const int iend = dry ? i0 + 32 : i1;
         if constexpr (DFP) {
             const float4* pf = reinterpret_cast<const float4*>(part) + (size_t)k * nblk;
@@ -481,19 +501,27 @@ __device__ __forceinline__ void reduce_slots(const double2* part, int nblk, int 
         } else {
             const double2* pd = part + (size_t)k * nblk;
             double a = 0.0, b = 0.0;
-            for (int ib = i0 + lane; ib < iend; ib += 32 * 8) {
-                double2 v[8];
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const int i = ib + 32 * t;
-                    v[t] = i < i1 ? __ldcg(pd + i) : make_double2(0.0, 0.0);
+            if constexpr (TILES) {
+                for (int i = i0 + lane; i < i1; i += 32) {
+                    const double2 v = tile_group(pd, i, nblk);
+                    a = __dadd_rn(a, v.x);
+                    b = __dadd_rn(b, v.y);
                 }
-                const int nt = min(8, (max(i1, ib + 1) - ib + 31) >> 5);   // loads that hit (FP64 adds are scarce)
+            } else {
+                for (int ib = i0 + lane; ib < iend; ib += 32 * 8) {
+                    double2 v[8];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    if (t < nt) {
-                        a = __dadd_rn(a, v[t].x);
-                        b = __dadd_rn(b, v[t].y);
+                    for (int t = 0; t < 8; ++t) {
+                        const int i = ib + 32 * t;
+                        v[t] = i < i1 ? __ldcg(pd + i) : make_double2(0.0, 0.0);
+                    }
+                    const int nt = min(8, (max(i1, ib + 1) - ib + 31) >> 5);   // loads that hit (FP64 adds are scarce)
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) {
+                        if (t < nt) {
+                            a = __dadd_rn(a, v[t].x);
+                            b = __dadd_rn(b, v[t].y);
+                        }
                     }
                 }
             }
@@ -575,7 +603,7 @@ __device__ __noinline__ void sc_beta(const SolverDev& d, int j, int nblk, bool d
     const int done = S->done, m = S->m;
     const dcx rho0 = ld(S->rho0), alpha = ld(S->alpha);
     __shared__ dcx red[1];
-    reduce_slots<1, DFP>(d.part, nblk, 1, red, dry);
+    reduce_slots<1, DFP, !DFP>(d.part, nblk, 1, red, dry);   // (FP64 sweeps leave tile partials)
     if (done) return;
     if (threadIdx.x == 0) {
         const dcx rho1 = red[0];
@@ -595,7 +623,7 @@ __device__ __noinline__ void sc_alpha_seed(const SolverDev& d, int j, int nblk, 
     const int done = S->done, m = S->m;
     const dcx rho0 = ld(S->rho0);
     __shared__ dcx red[1];
-    reduce_slots<1, DFP>(d.part, nblk, 1, red, dry);
+    reduce_slots<1, DFP, !DFP>(d.part, nblk, 1, red, dry);   // (FP64 sweeps leave tile partials)
     if (done) return;
     if (threadIdx.x == 0) {
         const dcx den = dry ? mk(1.0) : red[0];
@@ -1265,38 +1293,43 @@ __device__ __forceinline__ typename Ch<R>::T* select_vec(const SolverDev& d, int
     return base + (size_t)j * vstride<R>(d);
 }
 
-template <typename R, bool DOT>
-__global__ void __launch_bounds__(kThreads, hop_min_blocks<R>())
-k_hop_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel, int out_j, int second, int pass2,
-          ScalarStep step, const int4* tab) {
+// FP64, one system, pointers as kernel parameters: C blocks per tile (hop64.cuh)
+template <int C, bool DOT>
+__global__ void __launch_bounds__(hop64_threads<C>(), hop64_min_blocks<C>())
+k_hop64(Geom g, const double2* __restrict__ U, const double2* in, double2* out, Op64 op, const double2* dotv,
+        double2* partials, const int* done, const SolverDev* __restrict__ ds, ScalarStep step) {
     dep_sync();
-    const TraceScope trace_(trace_kind<R>(FA_TK_HOP_SYS, DOT));
+    const TraceScope trace_(trace_kind<double>(FA_TK_HOP1, DOT));
+    if (done != nullptr && *done) return;
+    __shared__ Smem64<C> sm;
+    const int tile = blockIdx.x / C, rank = blockIdx.x % C;
+    hop64_tile<C, true, DOT>(g, U, internal64(in, g.V), internal64(out, g.V), op, tile, rank, sm);
+    if (DOT && rank == 0) {
+        const double2 v = dot64_tile<C>(internal64(dotv, g.V), g.V, tile, sm);
+        if (threadIdx.x == 0) partials[tile] = v;
+        run_step<false>(ds[0], step, gridDim.x / C, gridDim.x / C);
+    }
+}
+
+// FP64, a batch: one tile of one system per block
+template <bool DOT>
+__global__ void __launch_bounds__(hop64_threads<1>(), hop64_min_blocks<1>())
+k_hop64_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel, int out_j, int second, int pass2,
+            ScalarStep step, const int4* tab) {
+    dep_sync();
+    const TraceScope trace_(trace_kind<double>(FA_TK_HOP_SYS, DOT));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, pass2)) return;
-    const int s = w.bx * kThreads + threadIdx.x;
-    cx<R> dres[1] = {czero<R>()};
-    if (s < d.V) {
-        const double sc = second ? d.scale : 1.0;
-        SpinorView<R> in{select_vec<R>(d, in_sel, in_j), d.V};
-        SpinorView<R> out{select_vec<R>(d, out_sel, out_j), d.V};
-        cx<R> p[12];
-        hop_site<R, false, true>(d.g, Vec<R>::links(d), in, s, fromdbl<R>(sc * d.diag), fromdbl<R>(-0.5 * sc),
-                                 fromdbl<R>(d.ef), fromdbl<R>(d.eb), fromdbl<R>(d.bc), p);
-        out.store(s, p);
-        if (DOT) {
-            SpinorView<R> rt{Vec<R>::rt(d), d.V};
-            cx<R> q[12];
-            rt.load(s, q);
-            cx<R> a = czero<R>();
-#pragma unroll
-            for (int k = 0; k < 12; ++k) a = cjfma(q[k], p[k], a);
-            dres[0] = a;
-        }
-    }
+    __shared__ Smem64<1> sm;
+    const double sc = second ? d.scale : 1.0;
+    const Op64 op{sc * d.diag, -0.5 * sc, d.ef, d.eb, d.bc, 0, 1};
+    hop64_tile<1, true, DOT>(d.g, d.links64, internal64(select_vec<double>(d, in_sel, in_j), d.V),
+                             internal64(select_vec<double>(d, out_sel, out_j), d.V), op, w.bx, 0, sm);
     if (DOT) {
-        block_reduce_store<1, R>(dres, d.part, 0, w.bx);
-        run_step<dfp_of<R>()>(d, step, w.nbx, w.ntk);
+        const double2 v = dot64_tile<1>(internal64(d.rt64, d.V), d.V, w.bx, sm);
+        if (threadIdx.x == 0) d.part[w.bx] = v;
+        run_step<false>(d, step, w.nbx, w.ntk);
     }
 }
 
