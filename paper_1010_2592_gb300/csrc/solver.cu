@@ -16,6 +16,7 @@
 
 #include "fa_context.h"
 #include "fused_sweep.cuh"
+#include "vec64.cuh"
 
 namespace fa {
 
@@ -183,6 +184,7 @@ __global__ void __launch_bounds__(kThreads) k_lincomb_canon(int n, int k, const 
 struct Layout {
     int L, ns, max_outer, V;
     bool need64, need32, single;
+    bool fp64;                 // FP64 outer iterations (the whole solve or its head)
     bool gram_hop;             // FP32 pass 1: the Gram matrix in the last sweep's epilogue (one system, l <= 4)
     size_t vs64, vs32;         // one spinor in elements of double2 / float4
     int nblk, red_grid, part_slots;
@@ -200,7 +202,8 @@ static int ensure_workspace(fa_ctx* c, const Layout& Lo) {
     const size_t s64 = (size_t)12 * V * sizeof(double2), s32 = (size_t)6 * V * sizeof(float4);
     // the Gram epilogue of the FP32 sweep writes n_gram(l) partials per block
     const size_t hop_blk = (size_t)std::max(nblocks(V), (V + kHopNarrowThreads - 1) / kHopNarrowThreads) + 1;
-    FA_CUDA(c->partials.ensure(std::max({(size_t)std::max({Lo.nblk, Lo.red_grid, Lo.vgrid + 1}) * Lo.part_slots,
+    // (FP64 reductions leave a partial per warp: 8 per block of the reduction grid)
+    FA_CUDA(c->partials.ensure(std::max({(size_t)std::max({Lo.nblk, 8 * Lo.red_grid, 8 * Lo.vgrid}) * Lo.part_slots,
                                          (size_t)row_blocks(V), (size_t)tiles64(V), hop_blk * (size_t)Lo.part_slots}) *
                                sizeof(double2)),
             "alloc partials");
@@ -300,7 +303,11 @@ static SolverDev make_dev(fa_ctx* c, const Layout& Lo) {
 
 // Work tables of a batch launch (see `where` in solver_kernels.cuh): per kernel
 // kind, one entry (system, block, vector blocks, tickets) per block of the launch.
-enum TabKind { TB_VEC = 0, TB_VECX, TB_RG, TB_RGX, TB_HOP, TB_ROWS, TB_KINDS };
+// FP64 kernels: tiles of the sweep, pairs of the elementwise updates (and 32 at a
+// time for the shift vectors), tiles of the vector and reduction grids.
+enum TabKind {
+    TB_VEC = 0, TB_VECX, TB_RG, TB_RGX, TB_ROWS, TB_HOP, TB_FLAT, TB_FLATX, TB_FLATS, TB_TV, TB_TR, TB_TRX, TB_KINDS
+};
 
 // A batch: systems whose kernels share each launch.  One system, or systems of
 // one lattice shape without work tables (grid.y = systems), or systems of any
@@ -367,7 +374,7 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     // k_gram / k_mr use vg where their register budget gives kVecBlocks
     // resident blocks per SM, else the reduction grid.
     dim3 gv(vg, n), gvx(vg + 1, n);
-    const bool gram_vec = gram_min_blocks<R, L>() >= kVecBlocks, mr_vec = mr_min_blocks<R, L>() >= kVecBlocks;
+    const bool gram_vec = gram_min_blocks<L>() >= kVecBlocks, mr_vec = mr_min_blocks<L>() >= kVecBlocks;
     dim3 gg(gram_vec ? vg : rg, n);
     const int mg = mr_vec ? vg : rg;
     dim3 gm(mg, n), gmx(mg + 1, n);
@@ -386,6 +393,11 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     }
     const SolverDev* ds = B.dev;
     cudaStream_t st = c->stream;
+    // FP64 kernels (vec64.cuh)
+    auto grid64 = [&](int k, int blocks, const int4*& t) {
+        t = B.tables ? B.tab[k] : nullptr;
+        return B.tables ? dim3(B.tab_n[k]) : dim3(blocks, n);
+    };
     constexpr int kind = rp_of<R>() == RP64 ? 0 : (rp_of<R>() == RP32 ? 1 : 2);
     const bool timing = c->hop_timing && !B.use_graph;
     const bool pdl = B.pdl && !timing;
@@ -546,19 +558,37 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     // after <rt, r_{j+1}>, the MR coefficients after the Gram matrix,
     // convergence after |r_0|^2); the shift parts in block 0 of the next
     // vector kernel (double-pass forms) or with the seed part (single pass).
+    const int V0 = B.Lo.V;
     for (int j = 0; j < L; ++j) {
-        launch(j > 0 && pdl, k_update_u<R>, gv, kThreads, st, ds, j, p2, tv);
+        if constexpr (rp_of<R>() == RP64) {
+            const int4* t;
+            const dim3 g = grid64(TB_FLAT, flat_blocks(V0, kFlat), t);
+            launch(j > 0 && pdl, k_update_u64, g, kFlat, st, ds, j, p2, t);
+        } else {
+            launch(j > 0 && pdl, k_update_u<R>, gv, kThreads, st, ds, j, p2, tv);
+        }
         FA_LAUNCHED(c, "k_update_u");
         FA_TRY(hop(0, j, 2, 0, 0, false, none));                                   // tmp = g5 D u_j
         const ScalarStep alpha{single ? STEP_ALPHA_ALL : STEP_ALPHA, j};
         FA_TRY(hop(2, 0, 0, j + 1, 1, !pass2, pass2 ? none : alpha));              // u_{j+1}
-        if (pass2) {
-            launch(pdl, k_update_r<R, true, false>, gv, kThreads, st, ds, j, p2, tv);
-        } else if (single) {
-            if constexpr (rp_of<R>() == RP64) launch(pdl, k_update_r<R, false, true>, gv, kThreads, st, ds, j, p2, tv);
+        // pass 1 of the double-pass forms: block 0 runs the shift part of sub-step j
+        // beside the vector blocks
+        if constexpr (rp_of<R>() == RP64) {
+            const int4* t;
+            if (pass2) {
+                const dim3 g = grid64(TB_FLAT, flat_blocks(V0, kFlat), t);
+                launch(pdl, k_update_r64<true, false, false>, g, kFlat, st, ds, j, p2, t);
+            } else if (single) {
+                const dim3 g = grid64(TB_FLATS, flat_blocks(V0, kFlatShift), t);
+                launch(pdl, k_update_r64<false, true, false>, g, kFlat, st, ds, j, p2, t);
+            } else {
+                const dim3 g = grid64(TB_FLATX, flat_blocks(V0, kFlat) + 1, t);
+                launch(pdl, k_update_r64<false, false, true>, g, kFlat, st, ds, j, p2, t);
+            }
+        } else if (pass2) {
+            launch(pdl, k_update_r<R, true>, gv, kThreads, st, ds, j, p2, tv);
         } else {
-            // block 0: shift part of sub-step j beside the vector blocks
-            launch(pdl, k_update_r<R, false, false, true>, gvx, kThreads, st, ds, j, p2, tvx);
+            launch(pdl, k_update_r<R, false, true>, gvx, kThreads, st, ds, j, p2, tvx);
         }
         FA_LAUNCHED(c, "k_update_r");
         FA_TRY(hop(1, j, 2, 0, 0, false, none));                                   // tmp = g5 D r_j
@@ -569,19 +599,39 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
             FA_TRY(hop(2, 0, 1, j + 1, 1, next_beta, next_beta ? ScalarStep{STEP_BETA, j + 1} : none));   // r_{j+1}
         }
     }
-    if (!pass2 && !gram_hop) {
-        launch(pdl, k_gram<R, L>, gg, kThreads, st, ds, single ? 1 : 0, tg);
-        FA_LAUNCHED(c, "k_gram");
-    }
     const ScalarStep conv = pass2 ? none : ScalarStep{STEP_CONV, head ? 1 : 0};
-    if (pass2) {
-        launch(pdl, k_mr<R, L, true, false, false>, gm, kThreads, st, ds, p2, none, tm);
-    } else if (single) {
-        if constexpr (rp_of<R>() == RP64)
-            launch(pdl, k_mr<R, L, false, true, true>, gm, kThreads, st, ds, p2, reliable ? none : conv, tm);
+    const ScalarStep mr_step = reliable ? none : conv;
+    if constexpr (rp_of<R>() == RP64) {
+        const int4* t;
+        if (!pass2) {
+            // l <= 2: the tiles of the vector grid, else of the reduction grid
+            const dim3 g = grid64(L <= 2 ? TB_TV : TB_TR, 8 * (L <= 2 ? vg : rg), t);
+            launch(pdl, k_gram64<L>, g, 32 * gram64_warps<L>(), st, ds, single ? 1 : 0, t);
+            FA_LAUNCHED(c, "k_gram");
+        }
+        if (pass2) {
+            const dim3 g = grid64(TB_TR, 8 * rg, t);
+            launch(pdl, k_mr64<L, true, false, false, false, 1>, g, kMrThreads, st, ds, p2, none, t);
+        } else if (single) {
+            // shift vectors: clusters where each of their blocks gets an SM of its own
+            const int C = (B.tables || n > 1) ? 1 : 64 * rg <= sms() ? 8 : 32 * rg <= sms() ? 4 : 16 * rg <= sms() ? 2 : 1;
+            const dim3 g = grid64(TB_TR, 8 * rg * C, t);
+            if (C == 8) launch_ex(pdl, 8, k_mr64<L, false, true, true, false, 8>, g, kMrThreads, st, ds, p2, mr_step, t);
+            else if (C == 4) launch_ex(pdl, 4, k_mr64<L, false, true, true, false, 4>, g, kMrThreads, st, ds, p2, mr_step, t);
+            else if (C == 2) launch_ex(pdl, 2, k_mr64<L, false, true, true, false, 2>, g, kMrThreads, st, ds, p2, mr_step, t);
+            else launch_ex(pdl, 1, k_mr64<L, false, true, true, false, 1>, g, kMrThreads, st, ds, p2, mr_step, t);
+        } else {
+            const dim3 g = grid64(TB_TRX, 8 * rg + 1, t);
+            launch(pdl, k_mr64<L, false, false, true, true, 1>, g, kMrThreads, st, ds, p2, mr_step, t);
+        }
     } else {
-        // block 0: shift part of the MR step beside the vector blocks
-        launch(pdl, k_mr<R, L, false, false, true, true>, gmx, kThreads, st, ds, p2, reliable ? none : conv, tmx);
+        if (!pass2 && !gram_hop) {
+            launch(pdl, k_gram<R, L>, gg, kThreads, st, ds, tg);
+            FA_LAUNCHED(c, "k_gram");
+        }
+        // pass 1: block 0 runs the shift part of the MR step beside the vector blocks
+        if (pass2) launch(pdl, k_mr<R, L, true, false>, gm, kThreads, st, ds, p2, none, tm);
+        else launch(pdl, k_mr<R, L, false, true, true>, gmx, kThreads, st, ds, p2, mr_step, tmx);
     }
     FA_LAUNCHED(c, "k_mr");
     if (reliable) {
@@ -807,6 +857,10 @@ static int build_tables(Batch& B) {
     for (int i = 0; i < n; ++i) {
         t[TB_VECX].push_back(make_int4(i, -1, B.lo[i].vgrid, B.lo[i].vgrid + 1));
         t[TB_RGX].push_back(make_int4(i, -1, B.lo[i].red_grid, B.lo[i].red_grid + 1));
+        if (!B.lo[i].fp64) continue;
+        const int nf = flat_blocks(B.lo[i].V, kFlat), nt = 8 * B.lo[i].red_grid;
+        t[TB_FLATX].push_back(make_int4(i, -1, nf, nf + 1));
+        t[TB_TRX].push_back(make_int4(i, -1, nt, nt + 1));
     }
     for (int i = 0; i < n; ++i) {
         const Layout& lo = B.lo[i];
@@ -814,7 +868,15 @@ static int build_tables(Batch& B) {
         blocks(t[TB_VECX], i, lo.vgrid, true);
         blocks(t[TB_RG], i, lo.red_grid, false);
         blocks(t[TB_RGX], i, lo.red_grid, true);
-        blocks(t[TB_HOP], i, tiles64(lo.V), false);
+        if (lo.fp64) {
+            blocks(t[TB_HOP], i, tiles64(lo.V), false);
+            blocks(t[TB_FLAT], i, flat_blocks(lo.V, kFlat), false);
+            blocks(t[TB_FLATX], i, flat_blocks(lo.V, kFlat), true);
+            if (lo.single) blocks(t[TB_FLATS], i, flat_blocks(lo.V, kFlatShift), false);
+            blocks(t[TB_TV], i, 8 * lo.vgrid, false);
+            blocks(t[TB_TR], i, 8 * lo.red_grid, false);
+            blocks(t[TB_TRX], i, 8 * lo.red_grid, true);
+        }
         blocks(t[TB_ROWS], i, row_blocks(lo.V), false);
     }
     // lattice groups for the FP32 multi-RHS sweep: systems sharing the packed
@@ -930,6 +992,7 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
         Lo.V = c->g.V;
         Lo.single = single;
         Lo.need64 = prec != FA_F32;
+        Lo.fp64 = prec == FA_F64 || prec == FA_MIXED;
         Lo.need32 = prec != FA_F64;
         Lo.vs64 = (size_t)12 * Lo.V;
         Lo.vs32 = (size_t)6 * Lo.V;
@@ -1509,7 +1572,7 @@ int grad(fa_ctx* c, const double* b, const double* eta, double* dLdU, double* dL
     FA_CUDA(c->tmp64.ensure(sb), "alloc");
     // mu-derivative partials of one chunk (summed on the host chunk by chunk, in
     // shift order) and the partials of <eta, y>
-    FA_CUDA(c->gpart.ensure(((size_t)chunk * nb + 2 * (size_t)rg) * sizeof(double2)), "alloc");
+    FA_CUDA(c->gpart.ensure(((size_t)chunk * nb + 2 * (size_t)n_partials<double>(rg)) * sizeof(double2)), "alloc");
     FA_CUDA(c->defl.ensure(2 * sb), "alloc");             // y and dL/db accumulators
     double2* yacc = c->defl.as<double2>();
     double2* bacc = yacc + vs;
@@ -1585,11 +1648,14 @@ int grad(fa_ctx* c, const double* b, const double* eta, double* dLdU, double* dL
     k_dot2<double><<<rg, kThreads, 0, st>>>(V, t1, yacc, part);
     FA_LAUNCHED(c, "k_dot2");
     if (dLdb) FA_TRY(launch_unpack_spinor_f64(c->g, bacc, dLdb, st));
-    std::vector<double2> h((size_t)rg);
+    std::vector<double2> h((size_t)n_partials<double>(rg));
     FA_CUDA(cudaMemcpyAsync(h.data(), part, h.size() * sizeof(double2), cudaMemcpyDeviceToHost, st), "read partials");
     FA_CUDA(cudaStreamSynchronize(st), "sync gradient");
     double lre = 0.0;
-    for (int k = 0; k < rg; ++k) lre += h[k].x;
+    for (int k = 0; k < rg; ++k) {   // the eight warps of a block in a shuffle tree's order
+        const double2* p = h.data() + 8 * k;
+        lre += ((p[0].x + p[4].x) + (p[2].x + p[6].x)) + ((p[1].x + p[5].x) + (p[3].x + p[7].x));
+    }
     *dLdmu = dmu;
     *L = lre;
     if (stats) {
@@ -1613,7 +1679,7 @@ int estimate_scale(fa_ctx* c, const double* v0, int iters, double* scale_out) {
     FA_CUDA(c->io64a.ensure(s64), "alloc");
     FA_CUDA(c->io64b.ensure(s64), "alloc");
     FA_CUDA(c->tmp64.ensure(s64), "alloc");
-    FA_CUDA(c->partials.ensure((size_t)std::max(nblocks(V), rg) * 2 * sizeof(double2)), "alloc");
+    FA_CUDA(c->partials.ensure((size_t)n_partials<double>(rg) * 2 * sizeof(double2)), "alloc");
     FA_CUDA(c->state.ensure(sizeof(DevState)), "alloc");
     double2* v = c->io64a.as<double2>();
     double2* w = c->io64b.as<double2>();
@@ -1624,7 +1690,7 @@ int estimate_scale(fa_ctx* c, const double* v0, int iters, double* scale_out) {
     auto normalise = [&](double2* x) -> int {
         k_dot2<double><<<rg, kThreads, 0, st>>>(V, x, x, c->partials.as<double2>());
         FA_LAUNCHED(c, "k_dot2");
-        k_sc_invnorm<<<1, kScalarThreads, 0, st>>>(c->partials.as<double2>(), rg, sc);
+        k_sc_invnorm<<<1, kScalarThreads, 0, st>>>(c->partials.as<double2>(), n_partials<double>(rg), sc);
         FA_LAUNCHED(c, "k_sc_invnorm");
         k_scale_f64<<<g, kThreads, 0, st>>>(n, x, sc);
         FA_LAUNCHED(c, "k_scale_f64");
@@ -1639,7 +1705,7 @@ int estimate_scale(fa_ctx* c, const double* v0, int iters, double* scale_out) {
     FA_TRY(apply_A_64(c, v, w, c->tmp64.as<double2>(), 1.0));
     k_dot2<double><<<rg, kThreads, 0, st>>>(V, w, w, c->partials.as<double2>());
     FA_LAUNCHED(c, "k_dot2");
-    k_sc_invnorm<<<1, kScalarThreads, 0, st>>>(c->partials.as<double2>(), rg, sc);
+    k_sc_invnorm<<<1, kScalarThreads, 0, st>>>(c->partials.as<double2>(), n_partials<double>(rg), sc);
     FA_LAUNCHED(c, "k_sc_invnorm");
     double h[2];
     FA_CUDA(cudaMemcpyAsync(h, sc, sizeof(h), cudaMemcpyDeviceToHost, st), "read norm");

@@ -281,6 +281,16 @@ __device__ __forceinline__ void acc_x(double2* x, int q, int V, int s, double2 a
     }
 }
 
+// x (FP64) += a v for one complex number
+__device__ __forceinline__ void acc_x1(double2* x, double2 a, cx<double> v) {
+    double2 t = *x;
+    t.x = __fma_rn(a.x, v.r, t.x);
+    t.x = __fma_rn(-a.y, v.i, t.x);
+    t.y = __fma_rn(a.x, v.i, t.y);
+    t.y = __fma_rn(a.y, v.r, t.y);
+    *x = t;
+}
+
 // ------------------------------------------------------------------ scalar steps
 // The scalar steps of the recurrence run inside the vector kernels, in two
 // parts.  The seed part (beta, alpha, the MR coefficients gamma, convergence)
@@ -324,8 +334,8 @@ __device__ __forceinline__ int last_block(DevState* S, int ntickets) {
     __shared__ int is_last;
     __syncthreads();
     if (threadIdx.x == 0) {
-        // thread 0 stored the block's partials; the fence is cumulative over
-        // what the barrier ordered before it (release), and the one after the
+        // one or several threads stored the block's partials; the fence is cumulative
+        // over what the barrier ordered before it (release), and the one after the
         // last ticket orders the reads that follow (acquire; the other threads
         // read the partials after the barrier, from L2)
         __threadfence();
@@ -392,8 +402,8 @@ __device__ __forceinline__ void recip2(double p, double q, double& ip, double& i
 // otherwise FP64 values summed in FP64.
 template <typename R> constexpr bool dfp_of() { return !std::is_same<R, double>::value; }
 
-// TILES (FP64): the partials are those of 32-site tiles, nblk of them; eight at
-// a time are first added in the order of a warp shuffle tree over eight lanes,
+// FP64 partials are those of warps (32-site tiles), nblk of them; eight at a
+// time are first added in the order of a warp shuffle tree over eight lanes,
 // and the sums of those 256-site groups are what is split into quarters.
 //
 // dry: warp 0 runs the code of one quarter once, every load predicated off
@@ -411,13 +421,12 @@ __device__ __forceinline__ double2 tile_group(const double2* pd, int i, int n) {
         }
     return v[0];
 }
-template <int NSMAX, bool DFP, bool TILES = false>
+template <int NSMAX, bool DFP>
 __device__ __forceinline__ void reduce_slots(const double2* part, int nblk, int ns, dcx* out, bool dry = false) {
-    static_assert(!(DFP && TILES), "tile partials are FP64");
     __shared__ double2 qs[4 * NSMAX];
     __shared__ float4 qf[4 * NSMAX];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int npart = TILES ? (nblk + 7) >> 3 : nblk;
+    const int npart = DFP ? nblk : (nblk + 7) >> 3;
     const int per = (npart + 3) >> 2;
     const int ntask = dry ? 1 : 4 * ns;
     if (dry && (int)threadIdx.x < 4 * ns) {   // the quarters a dry run leaves out
@@ -473,8 +482,8 @@ __device__ __forceinline__ void reduce_slots(const double2* part, int nblk, int 
     for (int u = u_first; u < ntask; u += nw) {
         const int k = u >> 2;
         const int i0 = (u & 3) * per, i1 = dry ? i0 : min(npart, i0 + per);
-        const int iend = dry ? i0 + 32 : i1;
         if constexpr (DFP) {
+            const int iend = dry ? i0 + 32 : i1;
             const float4* pf = reinterpret_cast<const float4*>(part) + (size_t)k * nblk;
             df a(0.0f), b(0.0f);
             // eight loads in flight per lane before the adds (zero padding
@@ -501,29 +510,10 @@ __device__ __forceinline__ void reduce_slots(const double2* part, int nblk, int 
         } else {
             const double2* pd = part + (size_t)k * nblk;
             double a = 0.0, b = 0.0;
-            if constexpr (TILES) {
-                for (int i = i0 + lane; i < i1; i += 32) {
-                    const double2 v = tile_group(pd, i, nblk);
-                    a = __dadd_rn(a, v.x);
-                    b = __dadd_rn(b, v.y);
-                }
-            } else {
-                for (int ib = i0 + lane; ib < iend; ib += 32 * 8) {
-                    double2 v[8];
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        const int i = ib + 32 * t;
-                        v[t] = i < i1 ? __ldcg(pd + i) : make_double2(0.0, 0.0);
-                    }
-                    const int nt = min(8, (max(i1, ib + 1) - ib + 31) >> 5);   // loads that hit (FP64 adds are scarce)
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        if (t < nt) {
-                            a = __dadd_rn(a, v[t].x);
-                            b = __dadd_rn(b, v[t].y);
-                        }
-                    }
-                }
+            for (int i = i0 + lane; i < i1; i += 32) {
+                const double2 v = tile_group(pd, i, nblk);
+                a = __dadd_rn(a, v.x);
+                b = __dadd_rn(b, v.y);
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -603,7 +593,7 @@ __device__ __noinline__ void sc_beta(const SolverDev& d, int j, int nblk, bool d
     const int done = S->done, m = S->m;
     const dcx rho0 = ld(S->rho0), alpha = ld(S->alpha);
     __shared__ dcx red[1];
-    reduce_slots<1, DFP, !DFP>(d.part, nblk, 1, red, dry);   // (FP64 sweeps leave tile partials)
+    reduce_slots<1, DFP>(d.part, nblk, 1, red, dry);
     if (done) return;
     if (threadIdx.x == 0) {
         const dcx rho1 = red[0];
@@ -623,7 +613,7 @@ __device__ __noinline__ void sc_alpha_seed(const SolverDev& d, int j, int nblk, 
     const int done = S->done, m = S->m;
     const dcx rho0 = ld(S->rho0);
     __shared__ dcx red[1];
-    reduce_slots<1, DFP, !DFP>(d.part, nblk, 1, red, dry);   // (FP64 sweeps leave tile partials)
+    reduce_slots<1, DFP>(d.part, nblk, 1, red, dry);
     if (done) return;
     if (threadIdx.x == 0) {
         const dcx den = dry ? mk(1.0) : red[0];
@@ -933,6 +923,30 @@ __device__ __forceinline__ void site_range(int V, unsigned bx, unsigned nbx, int
     s1 = (int)(((long long)V * (bx + 1)) / nbx);
 }
 
+// Partials of a kThreads-block reduction: one per block, FP64 one per warp
+// (the order that reduce_slots takes them in), K slots of n_partials(nbx) each.
+template <typename R> __host__ __device__ constexpr int n_partials(int nbx) {
+    return std::is_same<R, double>::value ? nbx * (kThreads / 32) : nbx;
+}
+template <int K, typename R>
+__device__ __forceinline__ void reduce_store(cx<R> (&v)[K], double2* out, int nbx, int bx) {
+    if constexpr (std::is_same<R, double>::value) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            double a = v[k].r, b = v[k].i;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a = __dadd_rn(a, __shfl_down_sync(0xffffffffu, a, o));
+                b = __dadd_rn(b, __shfl_down_sync(0xffffffffu, b, o));
+            }
+            if ((threadIdx.x & 31) == 0)
+                out[(size_t)k * n_partials<R>(nbx) + n_partials<R>(bx) + (threadIdx.x >> 5)] = make_double2(a, b);
+        }
+    } else {
+        block_reduce_store<K, R>(v, out, nbx, bx);
+    }
+}
+
 // ------------------------------------------------------------------ BiCG sub-step kernels
 // u_i <- r_i - beta u_i, i = 0..j (r, u: l+1 spinors each, contiguous, stride vs)
 template <typename R>
@@ -967,11 +981,11 @@ k_update_u(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) 
 
 // r_i <- r_i - alpha u_{i+1}, i = 0..j.
 // ACC (pass 2): y += sum_i coef[m][slot_old(j,i)] r_i(before the update).
-// SHIFTS (single-pass, FP64): the shift-vector updates of the BiCG sub-step,
-// reading each seed vector once for all active shifts.
 // XS (pass 1 of the double-pass forms): block 0 runs the shift part of sub-step
 // j (sc_alpha_shifts) beside the vector blocks 1..nblk.
-template <typename R, bool ACC, bool SHIFTS, bool XS = false>
+// (FP32 and double-float; FP64, with the shift vectors of single-pass solves:
+// k_update_r64.)
+template <typename R, bool ACC, bool XS = false>
 __global__ void __launch_bounds__(kThreads, kVecBlocks)
 k_update_r(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) {
     dep_sync();
@@ -989,10 +1003,6 @@ k_update_r(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) 
     typename Ch<R>::T* r = Vec<R>::r(d);
     const typename Ch<R>::T* u = Vec<R>::u(d);
     const size_t vs = vstride<R>(d);
-    double2* y = d.y;
-    double2* xs = d.xs;
-    double2* us = d.us;
-    const size_t svs = (size_t)12 * d.V;
     typename Ch<R>::T* store = pass2 ? nullptr : store_at<R>(d, m);
     const int L = d.L;
     const cx<R> na = negcx<R>(d.rec_alpha[m * L + j]);
@@ -1012,52 +1022,12 @@ k_update_r(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) 
 #pragma unroll
                 for (int w = 0; w < Ch<R>::W; ++w) t[w] = cfma(c, a.c[w], t[w]);
             }
-            if (SHIFTS) {
-                // u^s_i <- r_old_i/zeta - beta_s u^s_i   (FP64 only)
-                for (int sh = 0; sh < d.ns; ++sh) {
-                    if (!d.active[sh]) continue;
-                    const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * j;
-                    const cx<R> bs = negcx<R>(P[1]), iz = tocx<R>(P[2]);
-                    double2* usi = us + ((size_t)sh * (L + 1) + i) * svs;
-                    Ch<R> v = Ch<R>::ld((const typename Ch<R>::T*)usi, q, d.V, s);
-#pragma unroll
-                    for (int w = 0; w < Ch<R>::W; ++w) v.c[w] = cfma(bs, v.c[w], cmul(iz, a.c[w]));
-                    v.stv((typename Ch<R>::T*)usi, q, d.V, s);
-                }
-            }
             Ch<R> n;
 #pragma unroll
             for (int w = 0; w < Ch<R>::W; ++w) n.c[w] = cfma(na, b.c[w], a.c[w]);
             n.stv(ri, q, d.V, s);
-            if (SHIFTS && i == j) {
-                // u^s_{j+1} <- r_old_j/(alpha_s zeta) - r_j/(alpha_s zeta_new) - sigma u^s_j;
-                // x_s <- x_s + alpha_s u^s_0
-                for (int sh = 0; sh < d.ns; ++sh) {
-                    if (!d.active[sh]) continue;
-                    const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * j;
-                    const cx<R> as = tocx<R>(P[0]), iaz = tocx<R>(P[3]), niazn = negcx<R>(P[4]);
-                    const R nsig = (R)(-d.sigma[sh]);
-                    double2* usj = us + ((size_t)sh * (L + 1) + j) * svs;
-                    double2* usj1 = us + ((size_t)sh * (L + 1) + j + 1) * svs;
-                    double2* us0 = us + ((size_t)sh * (L + 1)) * svs;
-                    double2* xsh = xs + (size_t)sh * svs;
-                    Ch<R> vj = Ch<R>::ld((const typename Ch<R>::T*)usj, q, d.V, s);
-                    Ch<R> v0 = Ch<R>::ld((const typename Ch<R>::T*)us0, q, d.V, s);
-                    Ch<R> xv = Ch<R>::ld((const typename Ch<R>::T*)xsh, q, d.V, s);
-                    Ch<R> nv;
-#pragma unroll
-                    for (int w = 0; w < Ch<R>::W; ++w) {
-                        cx<R> e = cmul(iaz, a.c[w]);
-                        e = cfma(niazn, n.c[w], e);
-                        nv.c[w] = crfma(nsig, vj.c[w], e);
-                        xv.c[w] = cfma(as, v0.c[w], xv.c[w]);
-                    }
-                    nv.stv((typename Ch<R>::T*)usj1, q, d.V, s);
-                    xv.stv((typename Ch<R>::T*)xsh, q, d.V, s);
-                }
-            }
         }
-        if (ACC) acc_y<R>(y, q, d.V, s, t);
+        if (ACC) acc_y<R>(d.y, q, d.V, s, t);
         if (d.x64 != nullptr) acc_x<R>(d.x64, q, d.V, s, d.rec_alpha[m * L + j], Ch<R>::ld(u, q, d.V, s));
     }
     }
@@ -1065,13 +1035,13 @@ k_update_r(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) 
 
 // ------------------------------------------------------------------ MR part
 // Gram matrix <r_i, r_k>, 0 <= i <= k <= L, grid-stride, per-block partials.
-// Last block: the MR coefficients (sc_mr_seed) and, for single-pass solves
-// (shifts != 0), their shift part.
+// Last block: the MR coefficients (sc_mr_seed).  (FP32 and double-float; FP64:
+// k_gram64.)
 // l <= 2: registers capped for 4 blocks/SM (one wave of 512 blocks)
-template <typename R, int L> constexpr int gram_min_blocks() { return L <= 2 ? 4 : 1; }
+template <int L> constexpr int gram_min_blocks() { return L <= 2 ? 4 : 1; }
 template <typename R, int L>
-__global__ void __launch_bounds__(kThreads, gram_min_blocks<R, L>())
-k_gram(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
+__global__ void __launch_bounds__(kThreads, gram_min_blocks<L>())
+k_gram(const SolverDev* __restrict__ ds, const int4* tab) {
     dep_sync();
     const TraceScope trace_(trace_kind<R>(FA_TK_GRAM));
     const Where w = where<false>(tab);
@@ -1105,18 +1075,11 @@ k_gram(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
     }
     block_reduce_store<NG, R>(acc, partials, w.nbx, w.bx);
     const int lb = last_block(d.st, w.ntk);
-    if (lb == LB_LAST || (lb == LB_WARM && dfp_of<R>())) {
-        sc_mr_seed<L, dfp_of<R>()>(d, w.nbx, lb == LB_WARM);
-        if (shifts && lb == LB_LAST) {
-            __syncthreads();
-            sc_mr_shifts<L>(d);
-        }
-    }
+    if (lb != LB_NONE) sc_mr_seed<L, true>(d, w.nbx, lb == LB_WARM);
 }
 
 // MR update: r_0 -= sum gamma_j r_j, u_0 -= sum gamma_j u_j.
 // ACC: y += sum_k coef[m][slot_mr(k)] r_k (before the update).
-// SHIFTS: x_s += sum_k c_k/(zeta p_s) r_k, u^s_0 <- (u^s_0 - sum gamma_j u^s_j)/p_s.
 // DOT: per-block partials of <rt, r_0> (slot 0) and |r_0|^2 (slot 1), grid-stride,
 // then `step` (convergence) in the last block.
 // XS (pass 1 of the double-pass forms): block 0 runs the shift part of the MR
@@ -1125,11 +1088,10 @@ k_gram(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
 // FP32 and double-float, l <= 3: registers capped for 4 blocks/SM (64; some
 // bytes spilled), so that a 16^3 x 32 lattice (512 blocks) runs in one wave
 // instead of 1.12 (left alone, the compiler takes up to 167 registers here)
-template <typename R, int L> constexpr int mr_min_blocks() {
-    return (!std::is_same<R, double>::value && L <= 3) ? 4 : 1;
-}
-template <typename R, int L, bool ACC, bool SHIFTS, bool DOT, bool XS = false>
-__global__ void __launch_bounds__(kThreads, mr_min_blocks<R, L>())
+// (FP64, with the shift vectors of single-pass solves: k_mr64.)
+template <int L> constexpr int mr_min_blocks() { return L <= 3 ? 4 : 1; }
+template <typename R, int L, bool ACC, bool DOT, bool XS = false>
+__global__ void __launch_bounds__(kThreads, mr_min_blocks<L>())
 k_mr(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const int4* tab) {
     dep_sync();
     const TraceScope trace_(trace_kind<R>(FA_TK_MR, XS));
@@ -1149,9 +1111,6 @@ k_mr(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const int4* t
     const typename Ch<R>::T* rt = Vec<R>::rt(d);
     const size_t vs = vstride<R>(d);
     double2* y = d.y;
-    double2* xs = d.xs;
-    double2* us = d.us;
-    const size_t svs = (size_t)12 * d.V;
     typename Ch<R>::T* store = pass2 ? nullptr : store_at<R>(d, m);
     double2* partials = d.part;
     cx<R> ng[L + 1];
@@ -1183,33 +1142,6 @@ k_mr(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const int4* t
                     for (int w = 0; w < Ch<R>::W; ++w) t[w] = cfma(c, rv[k].c[w], t[w]);
                 }
                 acc_y<R>(y, q, d.V, s, t);
-            }
-            if (SHIFTS) {
-                for (int sh = 0; sh < d.ns; ++sh) {
-                    if (!d.active[sh]) continue;
-                    const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * L;
-                    const cx<R> ips = tocx<R>(P[0]);
-                    double2* xsh = xs + (size_t)sh * svs;
-                    Ch<R> xv = Ch<R>::ld((const typename Ch<R>::T*)xsh, q, d.V, s);
-                    Ch<R> u0 = Ch<R>::ld((const typename Ch<R>::T*)(us + (size_t)sh * (L + 1) * svs), q, d.V, s);
-#pragma unroll
-                    for (int k = 0; k < L; ++k) {
-                        const cx<R> c = tocx<R>(P[1 + k]);
-#pragma unroll
-                        for (int w = 0; w < Ch<R>::W; ++w) xv.c[w] = cfma(c, rv[k].c[w], xv.c[w]);
-                    }
-#pragma unroll
-                    for (int j = 1; j <= L; ++j) {
-                        Ch<R> uj = Ch<R>::ld((const typename Ch<R>::T*)(us + ((size_t)sh * (L + 1) + j) * svs),
-                                             q, d.V, s);
-#pragma unroll
-                        for (int w = 0; w < Ch<R>::W; ++w) u0.c[w] = cfma(ng[j], uj.c[w], u0.c[w]);
-                    }
-#pragma unroll
-                    for (int w = 0; w < Ch<R>::W; ++w) u0.c[w] = cmul(ips, u0.c[w]);
-                    xv.stv((typename Ch<R>::T*)xsh, q, d.V, s);
-                    u0.stv((typename Ch<R>::T*)(us + (size_t)sh * (L + 1) * svs), q, d.V, s);
-                }
             }
             if (d.x64 != nullptr) {
 #pragma unroll
@@ -1264,7 +1196,7 @@ __device__ __forceinline__ void k_dot2_body(int V, const typename Ch<R>::T* rt, 
             }
         }
     }
-    block_reduce_store<2, R>(dots, partials, nbx, bx);
+    reduce_store<2, R>(dots, partials, nbx, bx);
 }
 
 template <typename R>
@@ -1280,7 +1212,7 @@ k_dot2_sys(const SolverDev* __restrict__ ds, double tol, double theta, const int
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     k_dot2_body<R>(d.V, Vec<R>::rt(d), Vec<R>::r(d), d.part, w.bx, w.nbx);
-    if (last_block(d.st, w.ntk) == LB_LAST) sc_init<dfp_of<R>()>(d, w.nbx, tol, theta);
+    if (last_block(d.st, w.ntk) == LB_LAST) sc_init<dfp_of<R>()>(d, n_partials<R>(w.nbx), tol, theta);
 }
 
 // A application inside the solver: out = scale * g5 D in on the system's own
@@ -1495,8 +1427,8 @@ k_reliable(const SolverDev* __restrict__ ds, const double2* ax, int pass2, Scala
             }
         }
     }
-    block_reduce_store<2, R>(dots, d.part, gridDim.x);
-    run_step<dfp_of<R>()>(d, step, gridDim.x, gridDim.x);
+    reduce_store<2, R>(dots, d.part, gridDim.x, blockIdx.x);
+    run_step<dfp_of<R>()>(d, step, n_partials<R>(gridDim.x), gridDim.x);
 }
 
 // ------------------------------------------------------------------ pseudo-double-pass gather
