@@ -34,10 +34,19 @@ struct Geom {
 // returns, which happens once the predecessor grid has completed and its writes
 // are visible.  `launch_dependents` then lets the successor start its own launch.
 // For an ordinary launch both instructions return at once.  Every kernel that
-// the solver may launch this way calls this first.
+// the solver may launch this way calls one of these first.
+//
+// The FP64 kernels let their successor launch only once their main work is done
+// (dep_launch; leaving the kernel counts too): blocks that arrive earlier are
+// placed on the SMs that have room, several on one SM while others still run
+// their predecessor, and blocks that share an SM share its FP64 pipe.  Measured
+// on 8^4, 16 outer iterations of FP64 double pass: 6.98 ms with the successor
+// launched at once, 5.59 ms without programmatic launch.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dep_sync() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    dep_wait();
+    dep_launch();
 }
 
 // ------------------------------------------------------------------ complex

@@ -241,17 +241,28 @@ __device__ __forceinline__ void store_canonical(double2* out, int V, int tile, c
     for (int e = threadIdx.x; e < n; e += hop64_threads<C>()) o[e] = sm.out[e % 12][e / 12];
 }
 
-// Blocks per tile: clusters only where every block still gets an SM of its own.
-// A tile is 912 FP64 warp instructions, 228 per sub-partition with one block;
-// with idle SMs, C blocks on C SMs cut that time, past that point the cluster's
-// barriers and remote reads only cost.  Measured on GB300, one fa_apply_dw with
-// C = 1 / 2 / 4: 512 sites (16 tiles) 12.4 / 10.3 / 8.2 us, 2160 sites (68) 12.4 /
-// 10.3 / 10.3, 4096 sites (128) 13.0 / 14.4 / 15.0, 8192 sites 22.4 / 22.8 / 22.6,
-// 16^3 x 32 234 / 239 / 246 us (its FP64 issue floor; one thread per site: 270).
+// Blocks per tile.  A tile is 912 FP64 warp instructions, 228 per sub-partition
+// with one block on an SM; the busiest SM takes ceil(tiles C / SMs) / C of that,
+// which C = 2 or 4 lowers for few tiles and evens out for a few per SM; 8 % per
+// doubling is charged for the cluster's barriers and remote reads.  Measured on
+// GB300, 16 outer iterations of FP64 double pass from graphs, ms with C = 1 / 2 /
+// 4: 512 sites 4.5 / 3.7 / 3.3, 2160 sites 4.6 / 3.7 / 3.8, 3456 sites 4.7 / 4.9 /
+// 4.4, 4096 sites 4.6 / 4.9 / 4.9, 6144 sites 6.9 / 6.3 / 6.3, 16000 sites 12.1 /
+// 11.7 / 11.7, 41472 sites 25.2 / 26.4 / 26.2; one sweep on 16^3 x 32 234 / 239 /
+// 246 us (its FP64 issue floor; one thread per site: 270).
 inline int hop64_split(int V, int nsm) {
     if (nsm < 1) nsm = 152;
-    const int t = tiles64(V);
-    return 4 * t <= nsm ? 4 : (2 * t <= nsm ? 2 : 1);
+    const long long t = tiles64(V);
+    int best = 1;
+    double cost = 1e30;
+    for (int C = 1; C <= 4; C *= 2) {
+        const double f = (double)((t * C + nsm - 1) / nsm) / C * (C == 1 ? 1.0 : C == 2 ? 1.08 : 1.16);
+        if (f < cost) {
+            cost = f;
+            best = C;
+        }
+    }
+    return best;
 }
 
 // out = scale g5out (diag in' - 1/2 sum hops(in')), in' = g5in ? g5 in : in, one

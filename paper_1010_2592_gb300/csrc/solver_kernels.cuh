@@ -1230,12 +1230,13 @@ template <int C, bool DOT>
 __global__ void __launch_bounds__(hop64_threads<C>(), hop64_min_blocks<C>())
 k_hop64(Geom g, const double2* __restrict__ U, const double2* in, double2* out, Op64 op, const double2* dotv,
         double2* partials, const int* done, const SolverDev* __restrict__ ds, ScalarStep step) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<double>(FA_TK_HOP1, DOT));
     if (done != nullptr && *done) return;
     __shared__ Smem64<C> sm;
     const int tile = blockIdx.x / C, rank = blockIdx.x % C;
     hop64_tile<C, true, DOT>(g, U, internal64(in, g.V), internal64(out, g.V), op, tile, rank, sm);
+    dep_launch();
     if (DOT && rank == 0) {
         const double2 v = dot64_tile<C>(internal64(dotv, g.V), g.V, tile, sm);
         if (threadIdx.x == 0) partials[tile] = v;
@@ -1248,7 +1249,7 @@ template <bool DOT>
 __global__ void __launch_bounds__(hop64_threads<1>(), hop64_min_blocks<1>())
 k_hop64_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel, int out_j, int second, int pass2,
             ScalarStep step, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<double>(FA_TK_HOP_SYS, DOT));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -1258,6 +1259,7 @@ k_hop64_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel,
     const Op64 op{sc * d.diag, -0.5 * sc, d.ef, d.eb, d.bc, 0, 1};
     hop64_tile<1, true, DOT>(d.g, d.links64, internal64(select_vec<double>(d, in_sel, in_j), d.V),
                              internal64(select_vec<double>(d, out_sel, out_j), d.V), op, w.bx, 0, sm);
+    dep_launch();
     if (DOT) {
         const double2 v = dot64_tile<1>(internal64(d.rt64, d.V), d.V, w.bx, sm);
         if (threadIdx.x == 0) d.part[w.bx] = v;

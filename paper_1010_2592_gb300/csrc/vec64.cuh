@@ -55,7 +55,7 @@ __device__ __forceinline__ double warp_sum(double a) {
 // u_i <- r_i - beta u_i, i = 0..j
 __global__ void __launch_bounds__(kFlat)
 k_update_u64(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<double>(FA_TK_UPDATE_U));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -75,7 +75,7 @@ k_update_u64(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab
 template <bool ACC, bool SHIFTS, bool XS>
 __global__ void __launch_bounds__(kFlat)
 k_update_r64(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<double>(FA_TK_UPDATE_R, XS));
     const Where w = where<XS>(tab);
     const SolverDev& d = ds[w.sys];
@@ -145,7 +145,7 @@ template <int L> constexpr int gram64_warps() { return L == 1 ? 4 : L == 2 ? 9 :
 template <int L>
 __global__ void __launch_bounds__(32 * gram64_warps<L>())
 k_gram64(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<double>(FA_TK_GRAM));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -188,6 +188,7 @@ k_gram64(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
             if (L <= 2 && !im && i == k) p[1] = 0.0;
         }
     }
+    dep_launch();
     const int lb = last_block(d.st, w.ntk);
     if (lb == LB_LAST) {
         sc_mr_seed<L, false>(d, w.nbx, false);
@@ -206,7 +207,7 @@ template <int L, bool ACC, bool SHIFTS, bool DOT, bool XS, int C>
 __global__ void __launch_bounds__(kMrThreads)
 k_mr64(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const int4* tab) {
     static_assert(C == 1 || (SHIFTS && !XS), "clusters split the shifts");
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<double>(FA_TK_MR, XS));
     Where w = where<XS>(tab);
     int rank = 0;
@@ -304,6 +305,7 @@ k_mr64(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const int4*
         }
     }
     if (DOT) {
+        dep_launch();
         if (rank != 0) return;
         if (q < 3) {
             acc = warp_sum(acc);
