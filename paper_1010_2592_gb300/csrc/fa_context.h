@@ -89,7 +89,7 @@ struct fa_ctx {
     fa::DevBuf snap64, snap32;           // seed state at the first unstored outer iteration
     fa::DevBuf descbuf, flagbuf;         // batch descriptors and done flags (first context of a batch)
     fa::DevBuf tabbuf;                   // batch work tables and lattice groups (first context of a batch)
-    int mrhs_rpb = 0, mrhs_mb = 0;       // multi-RHS FP32 sweep shape of batches led by this context (0: default)
+    int mrhs_rpb = 0, mrhs_mb = 0;       // multi-RHS FP32 sweep shape of batches led by this context (0: not tuned)
     fa::DevBuf xrel, brel, snapx;        // reliable updates: seed solution, packed source, snapshot
     fa::DevBuf defl;                     // deflated sign: partial sums, coefficients, projected source
     fa::DevBuf eig;                      // eigensolver: Krylov basis, work spinors, partials

@@ -844,6 +844,22 @@ static int read_states(Batch& B, std::vector<DevState>& hs) {
     return FA_OK;
 }
 
+// Right-hand sides per block of the multi-RHS sweep of a batch that was not
+// tuned: as many as share a tile's links with profit (4), while at least six
+// blocks per SM remain (four are resident).  Measured on GB300, us per sweep
+// with 1 / 2 / 4 / all right-hand sides per block (4 blocks per SM): 12 on 388
+// tiles 51 / 49 / 49 / 57, 5 on 388 tiles 22.6 / 22.6 / 24.6 / 24.6, 12 on 74
+// tiles 12.4 / 12.3 / 16.4 / 33, 12 on 17 tiles 6.3 / 8.3 / 14.3 / 33, 12 on 1189
+// tiles 142 / 132 / 131 / 132.
+static int default_rhs_per_block(const std::vector<GroupDev>& groups) {
+    for (int rpb = 4; rpb > 1; --rpb) {
+        long long items = 0;
+        for (const GroupDev& g : groups) items += (long long)g.ntile * ((g.nsys + rpb - 1) / rpb);
+        if (items >= 6LL * sms()) return rpb;
+    }
+    return 1;
+}
+
 // Work tables and lattice groups of a batch of several systems, in one device
 // buffer of the first context.  Shift blocks come first in their tables (they
 // run the per-shift FP64 recurrences, the longest blocks of a launch).
@@ -903,13 +919,15 @@ static int build_tables(Batch& B) {
             }
             groups[gi].sys[groups[gi].nsys++] = i;
         }
-        const int rpb = c0->mrhs_rpb > 0 ? c0->mrhs_rpb : kMaxRhs;
+        const int rpb = c0->mrhs_rpb > 0 ? c0->mrhs_rpb : default_rhs_per_block(groups);
         for (size_t g = 0; g < groups.size(); ++g)
             for (int tile = 0; tile < groups[g].ntile; ++tile)
                 for (int r0 = 0; r0 < groups[g].nsys; r0 += rpb)
                     items.push_back(make_int4((int)g, tile, r0, std::min(r0 + rpb, groups[g].nsys)));
         B.rhs_per_block = rpb;
-        B.mrhs_min_blocks = c0->mrhs_mb == 4 ? 4 : kHopNarrowBlocks;
+        // not tuned: 4 blocks per SM (128 registers); at 7 the sweep spills and takes 1.5
+        // to 2 times as long on every batch measured
+        B.mrhs_min_blocks = c0->mrhs_mb == kHopNarrowBlocks ? kHopNarrowBlocks : 4;
     }
     size_t off[TB_KINDS + 2], bytes = 0;
     for (int k = 0; k < TB_KINDS; ++k) {
