@@ -124,10 +124,11 @@ inline const float4* linksdf_of(const fa_ctx* c) {
 }
 // operator application on internal layouts (used by the C-ABI and the solver)
 int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g5in, bool g5out, bool dagger_mu);
-int hop_f32(fa_ctx* c, const float4* in, float4* out, double scale, bool g5in, bool g5out, bool dagger_mu,
-            const float4* dot_with, double2* partials, const int* done);
-int hop_df(fa_ctx* c, const float4* in, float4* out, double scale, bool g5in, bool g5out, bool dagger_mu,
-           const float4* dot_with, double2* partials, const int* done);
+// (result in `out`, or in the canonical field `canon` when that is not null)
+int hop_f32(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
+            bool dagger_mu);
+int hop_df(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
+           bool dagger_mu);
 int solve(fa_ctx* c, const double* b_canon, double* y_canon, double* const* xs_canon,
           const fa_solver_params* p, fa_solver_stats* stats);
 int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* const* y_canon,

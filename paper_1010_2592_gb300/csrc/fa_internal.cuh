@@ -119,6 +119,45 @@ template <> inline df host_cvt<df>(double x) {
     return df(h, (float)(x - (double)h));
 }
 
+// Conversions of field data on the integer pipes.  The F2F conversions between
+// FP64 and FP32 run at the FP64 pipe's rate (measured 0.59 T/s, an 80 us floor
+// for the 24 numbers per site of a 32^3 x 64 spinor); these give the same bits
+// for zeros and in the exponent range given, and take the conversion elsewhere.
+//
+// RN(x): 2^-126 <= |x| < 2^127
+__device__ __forceinline__ float d2f_int(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 897u > 252u) return ((hi << 1) | lo) == 0u ? __uint_as_float(hi) : __double2float_rn(x);
+    const unsigned b = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned up = ((lo & 0x1fffffffu) + 0x0fffffffu + (b & 1u)) >> 29;   // round to nearest even
+    return __uint_as_float((b + up) | (hi & 0x80000000u));
+}
+// (RN(x), RN(x - RN(x))): 2^-74 <= |x| < 2^127.  The remainder is an integer of
+// at most 28 bits in units of x's last place.
+__device__ __forceinline__ float2 d2df_int(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = (hi >> 20) & 0x7ffu;
+    if (e - 949u > 200u) {
+        if (((hi << 1) | lo) == 0u) return make_float2(__uint_as_float(hi), 0.0f);
+        const float h = __double2float_rn(x);
+        return make_float2(h, __double2float_rn(__dsub_rn(x, (double)h)));
+    }
+    const unsigned b = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned low = lo & 0x1fffffffu;
+    const unsigned up = (low + 0x0fffffffu + (b & 1u)) >> 29;
+    int rem = (int)low - (int)(up << 29);
+    if (hi & 0x80000000u) rem = -rem;
+    return make_float2(__uint_as_float((b + up) | (hi & 0x80000000u)),
+                       __fmul_rn(__int2float_rn(rem), __uint_as_float((e - 948u) << 23)));   // 2^(e - 1075)
+}
+// the FP32 number as FP64: zeros and normal numbers
+__device__ __forceinline__ double f2d_int(float x) {
+    const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+    if (e - 1u > 253u) return (u << 1) == 0u ? __hiloint2double((int)u, 0) : (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3)), (int)(u << 29));
+}
+
 template <typename R> __device__ __forceinline__ cx<R> czero() { return {R(0), R(0)}; }
 template <typename R> __device__ __forceinline__ cx<R> cadd(cx<R> a, cx<R> b) { return {addR(a.r, b.r), addR(a.i, b.i)}; }
 template <typename R> __device__ __forceinline__ cx<R> csub(cx<R> a, cx<R> b) { return {subR(a.r, b.r), subR(a.i, b.i)}; }
@@ -407,25 +446,22 @@ inline int launch_status(const char* what) {
 // Hop (one D_w sweep): out = scale * G5OUT * (diag*in' - 1/2 sum hops(in')),
 // in' = G5IN ? gamma_5 in : in, time weights from `mu_sign` * mu (the FP64
 // sweep, launch_hop_f64, is declared in hop64.cuh).
-// When dot_with != nullptr, per-block partials of <dot_with, out> are written
-// to partials[blockIdx] (nblk = ceil(V/kThreads) of them).
+// The result goes to `out` (internal layout) or, when canon is not null, to the
+// canonical field `canon` (out is not written then).
 // shape: 0 narrow when the lattice fits one wave of it, 1 wide (kThreads x
 // FA_HOP_MINB per SM), 2 narrow (kHopNarrowThreads x kHopNarrowBlocks per SM)
-int launch_hop_f32(const Geom& g, const float4* links, const float4* in, float4* out,
+int launch_hop_f32(const Geom& g, const float4* links, const float4* in, float4* out, double* canon,
                    double diag, double ef, double eb, double t_bc, double scale,
-                   bool g5in, bool g5out, const float4* dot_with, double2* partials,
-                   const int* done, cudaStream_t st, int shape = 0);
+                   bool g5in, bool g5out, cudaStream_t st, int shape = 0);
 
-int launch_hop_df(const Geom& g, const float4* links, const float4* in, float4* out,
+int launch_hop_df(const Geom& g, const float4* links, const float4* in, float4* out, double* canon,
                   double diag, double ef, double eb, double t_bc, double scale,
-                  bool g5in, bool g5out, const float4* dot_with, double2* partials,
-                  const int* done, cudaStream_t st);
+                  bool g5in, bool g5out, cudaStream_t st);
 
 // canonical (interleaved complex128 AoS) <-> internal layouts
 int launch_pack_spinor_f64(const Geom& g, const double* canon, double2* out, cudaStream_t st);
 int launch_unpack_spinor_f64(const Geom& g, const double2* in, double* canon, cudaStream_t st);
 int launch_pack_spinor_f32(const Geom& g, const double* canon, float4* out, cudaStream_t st);
-int launch_unpack_spinor_f32(const Geom& g, const float4* in, double* canon, cudaStream_t st);
 int launch_pack_links(const Geom& g, const double* canon, double2* l64, float4* l32, float4* ldf, cudaStream_t st);
 // SMs of the current device; whether an FP32 sweep of V sites uses the narrow
 // launch shape (kHopNarrowThreads x kHopNarrowBlocks per SM, one wave)
@@ -436,7 +472,6 @@ inline bool hop_use_narrow(int shape, int V) { return shape == 2 || (shape == 0 
 int launch_convert_f64_to_f32(const Geom& g, const double2* in, float4* out, cudaStream_t st);
 // double-float spinors: [12][V] float4 = (re.hi, re.lo, im.hi, im.lo)
 int launch_pack_spinor_df(const Geom& g, const double* canon, float4* out, cudaStream_t st);
-int launch_unpack_spinor_df(const Geom& g, const float4* in, double* canon, cudaStream_t st);
 int launch_convert_df_to_f32(const Geom& g, const float4* in, float4* out, cudaStream_t st);
 
 // adjoint link force of <a1, D b1> + <a2, D b2> (a1 enters as gamma_5 a1), scaled by w,

@@ -79,23 +79,23 @@ int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g
     return rc;
 }
 
-int hop_f32(fa_ctx* c, const float4* in, float4* out, double scale, bool g5in, bool g5out, bool dagger_mu,
-            const float4* dot_with, double2* partials, const int* done) {
+int hop_f32(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
+            bool dagger_mu) {
     const double mu = dagger_mu ? -c->mu : c->mu;
-    hop_timing_begin(c, 1 + (dot_with ? 3 : 0));
-    int rc = launch_hop_f32(c->g, links32_of(c), in, out, 4.0 + c->mass, std::exp(mu), std::exp(-mu),
-                            c->t_bc, scale, g5in, g5out, dot_with, partials, done, c->stream, c->hop_shape);
+    hop_timing_begin(c, 1);
+    int rc = launch_hop_f32(c->g, links32_of(c), in, out, canon, 4.0 + c->mass, std::exp(mu), std::exp(-mu), c->t_bc,
+                            scale, g5in, g5out, c->stream, c->hop_shape);
     hop_timing_end(c);
     c->launches++;
     return rc;
 }
 
-int hop_df(fa_ctx* c, const float4* in, float4* out, double scale, bool g5in, bool g5out, bool dagger_mu,
-           const float4* dot_with, double2* partials, const int* done) {
+int hop_df(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
+           bool dagger_mu) {
     const double mu = dagger_mu ? -c->mu : c->mu;
-    hop_timing_begin(c, 2 + (dot_with ? 3 : 0));
-    int rc = launch_hop_df(c->g, linksdf_of(c), in, out, 4.0 + c->mass, std::exp(mu), std::exp(-mu), c->t_bc, scale,
-                           g5in, g5out, dot_with, partials, done, c->stream);
+    hop_timing_begin(c, 2);
+    int rc = launch_hop_df(c->g, linksdf_of(c), in, out, canon, 4.0 + c->mass, std::exp(mu), std::exp(-mu), c->t_bc,
+                           scale, g5in, g5out, c->stream);
     hop_timing_end(c);
     c->launches++;
     return rc;
