@@ -32,22 +32,18 @@ hop_kernel(Geom g, LinkView<float> U, SpinorView<float> in, SpinorView<float> ou
         if (!CANON) out.store(s, p);
     }
     if constexpr (CANON) {
-        __shared__ float2 turn[NT / 32][12][33];
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        if (s < g.V) {
+        if (s >= g.V) return;
+        double2* o = canon + (size_t)s * 12;
+        if ((reinterpret_cast<uintptr_t>(canon) & 31u) == 0) {
 #pragma unroll
-            for (int k = 0; k < 12; ++k) turn[warp][k][lane] = make_float2(p[k].r, p[k].i);
-        }
-        __syncwarp();
-        const int s0 = s - lane, n = min(32, g.V - s0) * 12;
-        double2* o = canon + (size_t)s0 * 12;
-#pragma unroll
-        for (int r = 0; r < 12; ++r) {
-            const int e = r * 32 + lane;
-            if (e < n) {
-                const float2 v = turn[warp][e % 12][e / 12];
-                o[e] = make_double2(f2d_int(v.x), f2d_int(v.y));
+            for (int k = 0; k < 12; k += 2) {
+                double v[4] = {f2d_int(p[k].r), f2d_int(p[k].i), f2d_int(p[k + 1].r), f2d_int(p[k + 1].i)};
+                asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(o + k), "d"(v[0]), "d"(v[1]), "d"(v[2]),
+                             "d"(v[3]) : "memory");
             }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) o[k] = make_double2(f2d_int(p[k].r), f2d_int(p[k].i));
         }
     }
 }
@@ -94,8 +90,8 @@ hop_rows_kernel(Geom g, LinkView<df> U, SpinorView<df> in, SpinorView<df> out, d
         const int s0 = blockIdx.x * kRowSites, n = min(kRowSites, g.V - s0) * 12;
         for (int e = threadIdx.x; e < n; e += kRowThreads) {
             const float4 v = turn[e % 12][e / 12];
-            canon[(size_t)s0 * 12 + e] = make_double2(__dadd_rn(f2d_int(v.x), f2d_int(v.y)),
-                                                      __dadd_rn(f2d_int(v.z), f2d_int(v.w)));
+            __stcs(canon + (size_t)s0 * 12 + e, make_double2(__dadd_rn(f2d_int(v.x), f2d_int(v.y)),
+                                                             __dadd_rn(f2d_int(v.z), f2d_int(v.w))));
         }
     }
 }
@@ -327,7 +323,7 @@ pack_kernel(int V, const double2* __restrict__ canon, typename PackOut<R>::T* __
 #pragma unroll
     for (int r = 0; r < 12 * kPackSites / kThreads; ++r) {
         const int e = r * kThreads + threadIdx.x;
-        if (e < 12 * ns) rec[e / 12][e % 12] = canon[(size_t)s0 * 12 + e];
+        if (e < 12 * ns) rec[e / 12][e % 12] = __ldcs(canon + (size_t)s0 * 12 + e);
     }
     __syncthreads();
     const int i = threadIdx.x % kPackSites;

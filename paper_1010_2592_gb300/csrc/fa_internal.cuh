@@ -104,14 +104,7 @@ __device__ __forceinline__ df operator-(df a, df b) { return subR(a, b); }
 __device__ __forceinline__ df operator*(int s, df a) { return {(float)s * a.hi, (float)s * a.lo}; }
 
 // conversions between the working precisions and FP64
-__device__ __forceinline__ double todbl(float x) { return (double)x; }
 __device__ __forceinline__ double todbl(double x) { return x; }
-__device__ __forceinline__ double todbl(df x) { return __dadd_rn((double)x.hi, (double)x.lo); }
-template <typename R> __device__ __forceinline__ R fromdbl(double x) { return (R)x; }
-template <> __device__ __forceinline__ df fromdbl<df>(double x) {
-    const float h = __double2float_rn(x);
-    return {h, __double2float_rn(__dsub_rn(x, (double)h))};
-}
 // the same conversions on the host (kernel arguments)
 template <typename R> inline R host_cvt(double x) { return (R)x; }
 template <> inline df host_cvt<df>(double x) {
@@ -156,6 +149,16 @@ __device__ __forceinline__ double f2d_int(float x) {
     const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
     if (e - 1u > 253u) return (u << 1) == 0u ? __hiloint2double((int)u, 0) : (double)x;
     return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3)), (int)(u << 29));
+}
+
+__device__ __forceinline__ double todbl(float x) { return f2d_int(x); }
+__device__ __forceinline__ double todbl(df x) { return __dadd_rn(f2d_int(x.hi), f2d_int(x.lo)); }
+template <typename R> __device__ __forceinline__ R fromdbl(double x);
+template <> __device__ __forceinline__ double fromdbl<double>(double x) { return x; }
+template <> __device__ __forceinline__ float fromdbl<float>(double x) { return d2f_int(x); }
+template <> __device__ __forceinline__ df fromdbl<df>(double x) {
+    const float2 t = d2df_int(x);
+    return {t.x, t.y};
 }
 
 template <typename R> __device__ __forceinline__ cx<R> czero() { return {R(0), R(0)}; }

@@ -4,7 +4,8 @@
 // The last sweep of BiCG sub-step l-1 produces r_l = c g5 D tmp; the MR step
 // then needs <r_i, r_k> for 0 <= i <= k <= l.  Instead of a kernel of its own
 // that reads r_0..r_l again, the sweep that holds r_l in registers reads
-// r_0..r_{l-1} at its own sites and stores the per-block partials; its last
+// r_0..r_{l-1} (and u_1..u_{l-1}, for the updates of r that the sub-steps
+// deferred) at its own sites and stores the per-block partials; its last
 // block solves for the MR coefficients gamma (sc_mr_seed).  No stencil read
 // changes, so the sweep keeps its neighbour traffic; one launch and one pass
 // over r_l less per outer iteration.
@@ -29,12 +30,14 @@ struct GramHop {
     float4* out;                     // r_l
     double2* part;                   // reduction partials, n_gram(l) slots of gridDim.x
     const float4* r[kMaxEll];        // r_0 .. r_{l-1}
+    const float4* u[kMaxEll];        // u_1 .. u_{l-1} (deferred updates of r)
     float cdiag, chop, ef, eb, bc;   // the second hop of A: scale c
 };
 
 // r_l = c g5 D tmp and the partials of <r_i, r_k> (i <= k <= L) in the order of
 // the Gram kernel, then the MR coefficients in the last block.
-template <int L, int NT, int MB>
+// DEFER: the updates of r that the sub-steps deferred come first.
+template <int L, bool DEFER, int NT, int MB>
 __global__ void __launch_bounds__(NT, MB)
 k_hop_gram(GramHop A, const SolverDev* __restrict__ ds) {
     dep_sync();
@@ -52,24 +55,34 @@ k_hop_gram(GramHop A, const SolverDev* __restrict__ ds) {
         hop_site<float, false, true>(A.g, A.U, SpinorView<float>{const_cast<float4*>(A.in), V}, s, A.cdiag, A.chop,
                                      A.ef, A.eb, A.bc, p);
         SpinorView<float>{A.out, V}.store(s, p);
+        const StepScalars<float, DEFER ? L : 1> sc(d, d.st->m);
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
-            cx<float> v[L + 1][2];
+            Ch<float> v[L + 1];
+            auto ld = [&](const float4* b) {
+                const float4 x = __ldg(b + (size_t)q * V + s);
+                Ch<float> c;
+                c.c[0] = {x.x, x.y};
+                c.c[1] = {x.z, x.w};
+                return c;
+            };
 #pragma unroll
-            for (int i = 0; i < L; ++i) {
-                const float4 x = __ldg(A.r[i] + (size_t)q * V + s);
-                v[i][0] = {x.x, x.y};
-                v[i][1] = {x.z, x.w};
+            for (int i = 0; i < L; ++i) v[i] = ld(A.r[i]);
+            v[L].c[0] = p[2 * q];
+            v[L].c[1] = p[2 * q + 1];
+            if constexpr (DEFER) {
+                Ch<float> u[L];
+#pragma unroll
+                for (int i = 1; i < L; ++i) u[i] = ld(A.u[i]);
+                deferred_r<float, L>(sc, v, u);
             }
-            v[L][0] = p[2 * q];
-            v[L][1] = p[2 * q + 1];
             int gi = 0;
 #pragma unroll
             for (int i = 0; i <= L; ++i)
 #pragma unroll
                 for (int k = i; k <= L; ++k) {
 #pragma unroll
-                    for (int w = 0; w < 2; ++w) red[gi] = cjfma(v[i][w], v[k][w], red[gi]);
+                    for (int w = 0; w < 2; ++w) red[gi] = cjfma(v[i].c[w], v[k].c[w], red[gi]);
                     ++gi;
                 }
         }

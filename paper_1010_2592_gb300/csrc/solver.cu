@@ -16,7 +16,7 @@
 
 #include "fa_context.h"
 #include "fused_sweep.cuh"
-#include "vec64.cuh"
+#include "vec_tile.cuh"
 
 namespace fa {
 
@@ -210,7 +210,7 @@ static int ensure_workspace(fa_ctx* c, const Layout& Lo) {
     FA_CUDA(c->state.ensure(sizeof(DevState)), "alloc state");
     FA_CUDA(c->shiftbuf.ensure((size_t)kMaxShifts * (2 * sizeof(double) + 2 * sizeof(double2) + 2 * sizeof(int))),
             "alloc shifts");
-    FA_CUDA(c->rec.ensure((size_t)MO * (3 * L + 1) * sizeof(double2)), "alloc record");
+    FA_CUDA(c->rec.ensure((size_t)MO * (3 * L + 1) * (sizeof(double2) + sizeof(float4))), "alloc record");
     FA_CUDA(c->prec.ensure((size_t)ns * MO * ps_stride(L) * sizeof(double2)), "alloc shift record");
     FA_CUDA(c->coef.ensure((size_t)MO * nc_slots(L) * sizeof(double2)), "alloc weights");
     FA_CUDA(c->coef4.ensure((size_t)MO * nc_slots(L) * sizeof(float4)), "alloc weights");
@@ -273,6 +273,10 @@ static SolverDev make_dev(fa_ctx* c, const Layout& Lo) {
     d.rec_alpha = rb;
     d.rec_beta = rb + (size_t)Lo.max_outer * Lo.L;
     d.rec_gamma = rb + (size_t)2 * Lo.max_outer * Lo.L;
+    float4* rb4 = reinterpret_cast<float4*>(rb + (size_t)Lo.max_outer * (3 * Lo.L + 1));
+    d.rec_alpha4 = rb4;
+    d.rec_beta4 = rb4 + (size_t)Lo.max_outer * Lo.L;
+    d.rec_gamma4 = rb4 + (size_t)2 * Lo.max_outer * Lo.L;
     d.prec = c->prec.as<double2>();
     d.coef = c->coef.as<double2>();
     d.coef4 = c->coef4.as<float4>();
@@ -285,6 +289,8 @@ static SolverDev make_dev(fa_ctx* c, const Layout& Lo) {
     d.u32 = c->u32.as<float4>();
     d.rt32 = c->rt32.as<float4>();
     d.tmp32 = c->tmp32.as<float4>();
+    d.rb64 = c->rb64.as<double2>();
+    d.rb32 = c->rb32.as<float4>();
     d.y = c->y64.as<double2>();
     d.xs = Lo.single ? c->xs64.as<double2>() : nullptr;
     d.us = Lo.single ? c->us64.as<double2>() : nullptr;
@@ -303,11 +309,17 @@ static SolverDev make_dev(fa_ctx* c, const Layout& Lo) {
 
 // Work tables of a batch launch (see `where` in solver_kernels.cuh): per kernel
 // kind, one entry (system, block, vector blocks, tickets) per block of the launch.
-// FP64 kernels: tiles of the sweep, pairs of the elementwise updates (and 32 at a
-// time for the shift vectors), tiles of the vector and reduction grids.
+// TB_VEC, TB_RG: blocks of the vector and reduction grids; TB_TV, TB_TR: their
+// 32-site tiles; TB_HOP, TB_ROWS: FP64 and double-float sweeps; TB_FLAT, TB_FLAT32:
+// elementwise updates of 12 V and 6 V elements (TB_ONE, TB_ONE32: one per thread);
+// TB_FLATS: shift vectors.  X: with the system's shift block first.
 enum TabKind {
-    TB_VEC = 0, TB_VECX, TB_RG, TB_RGX, TB_ROWS, TB_HOP, TB_FLAT, TB_FLATX, TB_FLATS, TB_TV, TB_TR, TB_TRX, TB_KINDS
+    TB_VEC = 0, TB_VECX, TB_RG, TB_RGX, TB_ROWS, TB_HOP, TB_FLAT, TB_FLATX, TB_FLAT32, TB_FLAT32X, TB_FLATS, TB_ONE, TB_ONE32,
+    TB_TV, TB_TR, TB_TRX, TB_KINDS
 };
+// elements per thread of the elementwise updates: one until the launch has
+// several waves of blocks, then four (four loads in flight, a quarter of the blocks)
+constexpr int kFlatMany = 4;
 
 // A batch: systems whose kernels share each launch.  One system, or systems of
 // one lattice shape without work tables (grid.y = systems), or systems of any
@@ -323,6 +335,8 @@ struct Batch {
     bool tables = false;                  // launches follow the work tables
     const int4* tab[TB_KINDS] = {};       // device tables
     int tab_n[TB_KINDS] = {};             // their lengths (blocks of the launch)
+    int ept64 = 1, ept32 = 1;             // elements per thread of the elementwise updates
+    double sites = 0.0;                   // of all systems
     const GroupDev* groups = nullptr;     // systems sharing a gauge field (multi-RHS FP32 sweep)
     const int4* items = nullptr;          // (group, tile, first, end) per block of that sweep
     int n_items = 0;
@@ -357,6 +371,20 @@ template <typename R> constexpr int rp_of() {
     return std::is_same<R, double>::value ? RP64 : (std::is_same<R, float>::value ? RP32 : RPDF);
 }
 
+// Whether pass 1 defers the updates i < j of its sub-steps (vec_tile.cuh): always
+// for l > 2 (32^3 x 64, l = 4: the FP32 update kernels of an outer iteration took
+// 2.2 ms of 5.5).  At l = 2 there is one such pair to save per vector, against
+// reading u_1 once more for the Gram matrix; FP32 gains where the vectors leave
+// the 129 MB L2 (batch of 596 thousand sites 51.9 -> 48.6 ms) and not below
+// (16^3 x 32: update kernels 34 -> 28 us, Gram sweep and MR step 40 -> 46 us per
+// outer iteration).
+constexpr double kDeferSites = 250e3;
+template <typename R, int L> static bool defer_updates(const Batch& B) {
+    if (L <= 1 || rp_of<R>() == RP64) return false;
+    if (L > 2) return true;
+    return rp_of<R>() == RP32 && B.sites >= kDeferSites;
+}
+
 // ------------------------------------------------------------------ one outer iteration
 // Pass 1 (pass2 = false): seed recurrence with inner products and the scalar
 // kernels.  Pass 2 (pass2 = true): the same vector kernels with the recorded
@@ -367,34 +395,18 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     fa_ctx* c = B.c0;
     const int n = B.n, rg = B.Lo.red_grid, vg = B.Lo.vgrid;
     const int p2 = pass2 ? 1 : 0;
-    // The vector kernels run vg blocks (one site per thread while the lattice
-    // fits one wave); their XS variants add the shift block, which finishes
-    // early (taking one of the vector blocks for it would give the others 257
-    // sites for 256 threads, a second pass for one thread of every block).
-    // k_gram / k_mr use vg where their register budget gives kVecBlocks
-    // resident blocks per SM, else the reduction grid.
-    dim3 gv(vg, n), gvx(vg + 1, n);
-    const bool gram_vec = gram_min_blocks<L>() >= kVecBlocks, mr_vec = mr_min_blocks<L>() >= kVecBlocks;
-    dim3 gg(gram_vec ? vg : rg, n);
-    const int mg = mr_vec ? vg : rg;
-    dim3 gm(mg, n), gmx(mg + 1, n);
-    // work tables (systems of different lattice shapes in one launch)
-    const int4 *tv = nullptr, *tvx = nullptr, *tg = nullptr, *tm = nullptr, *tmx = nullptr;
-    if (B.tables) {
-        auto T = [&](int k, dim3& g, const int4*& t) {
-            g = dim3(B.tab_n[k]);
-            t = B.tab[k];
-        };
-        T(TB_VEC, gv, tv);
-        T(TB_VECX, gvx, tvx);
-        T(gram_vec ? TB_VEC : TB_RG, gg, tg);
-        T(mr_vec ? TB_VEC : TB_RG, gm, tm);
-        T(mr_vec ? TB_VECX : TB_RGX, gmx, tmx);
-    }
+    // The FP32 kernels with inner products run vg blocks (one site per thread while
+    // the lattice fits one wave); their XS variants add the shift block, which
+    // finishes early.  They use vg where their register budget gives kVecBlocks
+    // resident blocks per SM, else the reduction grid; the tile kernels follow
+    // the same grids (8 tiles per block).
+    dim3 gv(vg, n);
+    const bool gram_vec = L <= 2;
+    const bool mr_vec = rp_of<R>() != RP64 && mr_min_blocks<L>() >= kVecBlocks;
     const SolverDev* ds = B.dev;
     cudaStream_t st = c->stream;
-    // FP64 kernels (vec64.cuh)
-    auto grid64 = [&](int k, int blocks, const int4*& t) {
+    // grid of a kernel and its work table, if the batch has tables
+    auto grid = [&](int k, int blocks, const int4*& t) {
         t = B.tables ? B.tab[k] : nullptr;
         return B.tables ? dim3(B.tab_n[k]) : dim3(blocks, n);
     };
@@ -408,8 +420,8 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     const SolverDev& h0 = B.host[0];
     auto vsel = [&](int sel, int j) -> T* {
         constexpr bool wide = rp_of<R>() != RP32;   // FP64 and double-float use the wide buffers
-        T* base = wide ? (T*)(sel == 0 ? (void*)h0.u64 : sel == 1 ? (void*)h0.r64 : (void*)h0.tmp64)
-                       : (T*)(sel == 0 ? (void*)h0.u32 : sel == 1 ? (void*)h0.r32 : (void*)h0.tmp32);
+        T* base = wide ? (T*)(sel == 0 ? (void*)h0.u64 : sel == 1 ? (void*)h0.r64 : sel == 2 ? (void*)h0.tmp64 : (void*)h0.rb64)
+                       : (T*)(sel == 0 ? (void*)h0.u32 : sel == 1 ? (void*)h0.r32 : sel == 2 ? (void*)h0.tmp32 : (void*)h0.rb32);
         return base + (size_t)j * (size_t)Ch<R>::N * h0.V;
     };
     const ScalarStep none{STEP_NONE, 0};
@@ -526,6 +538,7 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     };
     // FP32 pass 1 of a one-system double-pass solve: the last sweep forms the
     // Gram matrix (fused_sweep.cuh) instead of a kernel of its own
+    const bool defer = defer_updates<R, L>(B);
     const bool gram_hop = rp_of<R>() == RP32 && L <= 4 && B.Lo.gram_hop && n == 1 && !pass2 && !single;
     auto gram_sweep = [&]() -> int {
         if constexpr (rp_of<R>() == RP32 && L <= 4) {
@@ -536,6 +549,7 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
             a.out = h0.r32 + (size_t)L * 6 * h0.V;
             a.part = h0.part;
             for (int i = 0; i < L; ++i) a.r[i] = h0.r32 + (size_t)i * 6 * h0.V;
+            for (int i = 1; i < L; ++i) a.u[i] = h0.u32 + (size_t)i * 6 * h0.V;
             a.cdiag = host_cvt<float>(h0.scale * h0.diag);
             a.chop = host_cvt<float>(-0.5 * h0.scale);
             a.ef = host_cvt<float>(h0.ef);
@@ -544,9 +558,13 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
             if (timing) hop_timing_begin(c, 6);
             if (hop_use_narrow(c->hop_shape, h0.V)) {
                 constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks;
-                launch(pdl, k_hop_gram<L, NT, MB>, dim3((h0.V + NT - 1) / NT), NT, st, a, ds);
+                const dim3 gh((h0.V + NT - 1) / NT);
+                if (defer) launch(pdl, k_hop_gram<L, (L > 1), NT, MB>, gh, NT, st, a, ds);
+                else launch(pdl, k_hop_gram<L, (L > 2), NT, MB>, gh, NT, st, a, ds);
             } else {
-                launch(pdl, k_hop_gram<L, kThreads, FA_HOP_MINB>, dim3(nblocks(h0.V)), kThreads, st, a, ds);
+                const dim3 gh(nblocks(h0.V));
+                if (defer) launch(pdl, k_hop_gram<L, (L > 1), kThreads, FA_HOP_MINB>, gh, kThreads, st, a, ds);
+                else launch(pdl, k_hop_gram<L, (L > 2), kThreads, FA_HOP_MINB>, gh, kThreads, st, a, ds);
             }
             if (timing) hop_timing_end(c);
             FA_LAUNCHED(c, "k_hop_gram");
@@ -558,40 +576,47 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     // after <rt, r_{j+1}>, the MR coefficients after the Gram matrix,
     // convergence after |r_0|^2); the shift parts in block 0 of the next
     // vector kernel (double-pass forms) or with the seed part (single pass).
-    const int V0 = B.Lo.V;
+    constexpr bool F64 = rp_of<R>() == RP64;
+    const int ne = flat_elems<R>(B.Lo.V), ept = rp_of<R>() == RP32 ? B.ept32 : (F64 ? 1 : B.ept64);
+    const int flat = rp_of<R>() == RP32 ? TB_FLAT32 : TB_FLAT, flatx = rp_of<R>() == RP32 ? TB_FLAT32X : TB_FLATX;
+    const int nflat = flat_blocks(ne, kFlat * ept);
+    // FP64 updates take one element per thread in every launch, so that the tables of
+    // a batch with a head serve them too
+    const int4* t;
     for (int j = 0; j < L; ++j) {
-        if constexpr (rp_of<R>() == RP64) {
-            const int4* t;
-            const dim3 g = grid64(TB_FLAT, flat_blocks(V0, kFlat), t);
-            launch(j > 0 && pdl, k_update_u64, g, kFlat, st, ds, j, p2, t);
-        } else {
-            launch(j > 0 && pdl, k_update_u<R>, gv, kThreads, st, ds, j, p2, tv);
-        }
+        const dim3 gu = grid(flat, nflat, t);
+        const int i0 = !F64 && (pass2 || defer) ? j : 0;
+        if (ept == 1) launch(j > 0 && pdl, k_update_u<R, 1>, gu, kFlat, st, ds, i0, j, p2, t);
+        else launch(j > 0 && pdl, k_update_u<R, kFlatMany>, gu, kFlat, st, ds, i0, j, p2, t);
         FA_LAUNCHED(c, "k_update_u");
         FA_TRY(hop(0, j, 2, 0, 0, false, none));                                   // tmp = g5 D u_j
         const ScalarStep alpha{single ? STEP_ALPHA_ALL : STEP_ALPHA, j};
         FA_TRY(hop(2, 0, 0, j + 1, 1, !pass2, pass2 ? none : alpha));              // u_{j+1}
         // pass 1 of the double-pass forms: block 0 runs the shift part of sub-step j
         // beside the vector blocks
-        if constexpr (rp_of<R>() == RP64) {
-            const int4* t;
+        if constexpr (F64) {
             if (pass2) {
-                const dim3 g = grid64(TB_FLAT, flat_blocks(V0, kFlat), t);
+                const dim3 g = grid(flat, nflat, t);
                 launch(pdl, k_update_r64<true, false, false>, g, kFlat, st, ds, j, p2, t);
             } else if (single) {
-                const dim3 g = grid64(TB_FLATS, flat_blocks(V0, kFlatShift), t);
+                const dim3 g = grid(TB_FLATS, flat_blocks(ne, kFlatShift), t);
                 launch(pdl, k_update_r64<false, true, false>, g, kFlat, st, ds, j, p2, t);
             } else {
-                const dim3 g = grid64(TB_FLATX, flat_blocks(V0, kFlat) + 1, t);
+                const dim3 g = grid(flatx, nflat + 1, t);
                 launch(pdl, k_update_r64<false, false, true>, g, kFlat, st, ds, j, p2, t);
             }
         } else if (pass2) {
-            launch(pdl, k_update_r<R, true>, gv, kThreads, st, ds, j, p2, tv);
+            const dim3 g = grid(flat, nflat, t);
+            if (ept == 1) launch(pdl, k_update_r<R, true, false, 1>, g, kFlat, st, ds, i0, j, 0, t);
+            else launch(pdl, k_update_r<R, true, false, kFlatMany>, g, kFlat, st, ds, i0, j, 0, t);
         } else {
-            launch(pdl, k_update_r<R, false, true>, gvx, kThreads, st, ds, j, p2, tvx);
+            const dim3 g = grid(flatx, nflat + 1, t);
+            const int seed_x = defer ? 0 : 1;
+            if (ept == 1) launch(pdl, k_update_r<R, false, true, 1>, g, kFlat, st, ds, i0, j, seed_x, t);
+            else launch(pdl, k_update_r<R, false, true, kFlatMany>, g, kFlat, st, ds, i0, j, seed_x, t);
         }
         FA_LAUNCHED(c, "k_update_r");
-        FA_TRY(hop(1, j, 2, 0, 0, false, none));                                   // tmp = g5 D r_j
+        FA_TRY(hop(!F64 && pass2 ? 3 : 1, j, 2, 0, 0, false, none));               // tmp = g5 D r_j
         const bool next_beta = !pass2 && j < L - 1;
         if (gram_hop && j == L - 1) {
             FA_TRY(gram_sweep());   // r_l and, in the epilogue, the Gram matrix and gamma
@@ -601,37 +626,56 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     }
     const ScalarStep conv = pass2 ? none : ScalarStep{STEP_CONV, head ? 1 : 0};
     const ScalarStep mr_step = reliable ? none : conv;
-    if constexpr (rp_of<R>() == RP64) {
-        const int4* t;
-        if (!pass2) {
-            // l <= 2: the tiles of the vector grid, else of the reduction grid
-            const dim3 g = grid64(L <= 2 ? TB_TV : TB_TR, 8 * (L <= 2 ? vg : rg), t);
-            launch(pdl, k_gram64<L>, g, 32 * gram64_warps<L>(), st, ds, single ? 1 : 0, t);
-            FA_LAUNCHED(c, "k_gram");
-        }
-        if (pass2) {
-            const dim3 g = grid64(TB_TR, 8 * rg, t);
-            launch(pdl, k_mr64<L, true, false, false, false, 1>, g, kMrThreads, st, ds, p2, none, t);
-        } else if (single) {
-            // shift vectors: clusters where each of their blocks gets an SM of its own
-            const int C = (B.tables || n > 1) ? 1 : 64 * rg <= sms() ? 8 : 32 * rg <= sms() ? 4 : 16 * rg <= sms() ? 2 : 1;
-            const dim3 g = grid64(TB_TR, 8 * rg * C, t);
-            if (C == 8) launch_ex(pdl, 8, k_mr64<L, false, true, true, false, 8>, g, kMrThreads, st, ds, p2, mr_step, t);
-            else if (C == 4) launch_ex(pdl, 4, k_mr64<L, false, true, true, false, 4>, g, kMrThreads, st, ds, p2, mr_step, t);
-            else if (C == 2) launch_ex(pdl, 2, k_mr64<L, false, true, true, false, 2>, g, kMrThreads, st, ds, p2, mr_step, t);
-            else launch_ex(pdl, 1, k_mr64<L, false, true, true, false, 1>, g, kMrThreads, st, ds, p2, mr_step, t);
+    if (!pass2 && !gram_hop) {
+        if constexpr (F64) {
+            const dim3 g = grid(gram_vec ? TB_TV : TB_TR, 8 * (gram_vec ? vg : rg), t);
+            launch(pdl, k_gram_tile<L>, g, 32 * kGramWarps, st, ds, single ? 1 : 0, t);
         } else {
-            const dim3 g = grid64(TB_TRX, 8 * rg + 1, t);
-            launch(pdl, k_mr64<L, false, false, true, true, 1>, g, kMrThreads, st, ds, p2, mr_step, t);
+            if constexpr (rp_of<R>() == RPDF && L > 2) {
+                const dim3 g = grid(TB_ONE, flat_blocks(ne, kFlat), t);
+                launch(pdl, k_deferred<L>, g, kFlat, st, ds, t);
+                FA_LAUNCHED(c, "k_deferred");
+            }
+            constexpr bool D1 = rp_of<R>() == RP32 && L > 1, D0 = rp_of<R>() == RP32 && L > 2;
+            dim3 g = grid(gram_vec ? TB_VEC : TB_RG, gram_vec ? vg : rg, t);
+            g.z = gram_groups<R, L>();
+            if (defer) launch(pdl, k_gram<R, L, D1>, g, kThreads, st, ds, t);
+            else launch(pdl, k_gram<R, L, D0>, g, kThreads, st, ds, t);
         }
-    } else {
-        if (!pass2 && !gram_hop) {
-            launch(pdl, k_gram<R, L>, gg, kThreads, st, ds, tg);
-            FA_LAUNCHED(c, "k_gram");
+        FA_LAUNCHED(c, "k_gram");
+    }
+    const int mg = mr_vec ? vg : rg;
+    if (pass2) {
+        if constexpr (F64) {
+            const dim3 g = grid(TB_TR, 8 * mg, t);
+            launch(pdl, k_mr_tile<L, true, false, false, false, 1>, g, kMrThreads, st, ds, p2, none, t);
+        } else {
+            const dim3 g = grid(rp_of<R>() == RP32 ? TB_ONE32 : TB_ONE, flat_blocks(ne, kFlat), t);
+            launch(pdl, k_mr_acc<R, L>, g, kFlat, st, ds, t);
         }
-        // pass 1: block 0 runs the shift part of the MR step beside the vector blocks
-        if (pass2) launch(pdl, k_mr<R, L, true, false>, gm, kThreads, st, ds, p2, none, tm);
-        else launch(pdl, k_mr<R, L, false, true, true>, gmx, kThreads, st, ds, p2, mr_step, tmx);
+    } else if (!single) {
+        // block 0 runs the shift part of the MR step beside the vector blocks
+        if constexpr (F64) {
+            const dim3 g = grid(TB_TRX, 8 * mg + 1, t);
+            launch(pdl, k_mr_tile<L, false, false, true, true, 1>, g, kMrThreads, st, ds, p2, mr_step, t);
+        } else {
+            constexpr bool D1 = rp_of<R>() == RP32 && L > 1, D0 = rp_of<R>() == RP32 && L > 2;
+            const dim3 g = grid(mr_vec ? TB_VECX : TB_RGX, mg + 1, t);
+            if (defer) launch(pdl, k_mr<R, L, D1>, g, kThreads, st, ds, mr_step, t);
+            else launch(pdl, k_mr<R, L, D0>, g, kThreads, st, ds, mr_step, t);
+        }
+    } else if constexpr (F64) {
+        // shift vectors: clusters where each of their blocks gets an SM of its own
+        const int C = (B.tables || n > 1) ? 1 : 64 * rg <= sms() ? 8 : 32 * rg <= sms() ? 4 : 16 * rg <= sms() ? 2 : 1;
+        const dim3 g = grid(TB_TR, 8 * rg * C, t);
+        auto go = [&](auto split) {
+            constexpr int K = decltype(split)::value;
+            launch_ex(pdl, K, k_mr_tile<L, false, true, true, false, K>, g, kMrThreads, st, ds, p2, mr_step, t);
+        };
+        if (C == 8) go(std::integral_constant<int, 8>{});
+        else if (C == 4) go(std::integral_constant<int, 4>{});
+        else if (C == 2) go(std::integral_constant<int, 2>{});
+        else go(std::integral_constant<int, 1>{});
     }
     FA_LAUNCHED(c, "k_mr");
     if (reliable) {
@@ -698,6 +742,7 @@ static std::vector<unsigned long long> graph_signature(const Batch& B) {
     for (int k = 0; k < TB_KINDS; ++k) s.push_back((unsigned long long)B.tab_n[k]);
     s.push_back((unsigned long long)B.n_items);
     s.push_back((unsigned long long)B.mrhs_min_blocks);
+    s.push_back((unsigned long long)(B.ept64 * 16 + B.ept32));
     p(c->io64a.p);
     p(c->io64b.p);
     if (B.n == 1) {
@@ -706,7 +751,7 @@ static std::vector<unsigned long long> graph_signature(const Batch& B) {
                               (const void*)h.links32, (const void*)h.linksdf, (const void*)h.r64,
                               (const void*)h.u64, (const void*)h.rt64, (const void*)h.tmp64, (const void*)h.r32,
                               (const void*)h.u32, (const void*)h.rt32, (const void*)h.tmp32, (const void*)h.x64,
-                              (const void*)h.b64})
+                              (const void*)h.b64, (const void*)h.rb64, (const void*)h.rb32})
             p(v);
         d(h.diag);
         d(h.ef);
@@ -870,13 +915,18 @@ static int build_tables(Batch& B) {
     auto blocks = [&](std::vector<int4>& v, int i, int nb, bool xs) {
         for (int b = 0; b < nb; ++b) v.push_back(make_int4(i, b, nb, nb + (xs ? 1 : 0)));
     };
+    // blocks of a system's elementwise updates (FP64: one element per thread)
+    auto nflat = [&](int i, bool wide) {
+        const int ept = wide ? (B.lo[i].fp64 ? 1 : B.ept64) : B.ept32;
+        return flat_blocks((wide ? 12 : 6) * B.lo[i].V, kFlat * ept);
+    };
     for (int i = 0; i < n; ++i) {
         t[TB_VECX].push_back(make_int4(i, -1, B.lo[i].vgrid, B.lo[i].vgrid + 1));
         t[TB_RGX].push_back(make_int4(i, -1, B.lo[i].red_grid, B.lo[i].red_grid + 1));
-        if (!B.lo[i].fp64) continue;
-        const int nf = flat_blocks(B.lo[i].V, kFlat), nt = 8 * B.lo[i].red_grid;
-        t[TB_FLATX].push_back(make_int4(i, -1, nf, nf + 1));
-        t[TB_TRX].push_back(make_int4(i, -1, nt, nt + 1));
+        auto shift = [&](int k, int nb) { t[k].push_back(make_int4(i, -1, nb, nb + 1)); };
+        if (B.lo[i].need64) shift(TB_FLATX, nflat(i, true));
+        if (B.lo[i].fp64) shift(TB_TRX, 8 * B.lo[i].red_grid);
+        if (B.lo[i].need32) shift(TB_FLAT32X, nflat(i, false));
     }
     for (int i = 0; i < n; ++i) {
         const Layout& lo = B.lo[i];
@@ -884,16 +934,24 @@ static int build_tables(Batch& B) {
         blocks(t[TB_VECX], i, lo.vgrid, true);
         blocks(t[TB_RG], i, lo.red_grid, false);
         blocks(t[TB_RGX], i, lo.red_grid, true);
+        if (lo.fp64) blocks(t[TB_HOP], i, tiles64(lo.V), false);
+        if (lo.single) blocks(t[TB_FLATS], i, flat_blocks(12 * lo.V, kFlatShift), false);
+        if (lo.need64) {
+            blocks(t[TB_ROWS], i, row_blocks(lo.V), false);
+            blocks(t[TB_FLAT], i, nflat(i, true), false);
+            blocks(t[TB_FLATX], i, nflat(i, true), true);
+            blocks(t[TB_ONE], i, flat_blocks(12 * lo.V, kFlat), false);
+        }
         if (lo.fp64) {
-            blocks(t[TB_HOP], i, tiles64(lo.V), false);
-            blocks(t[TB_FLAT], i, flat_blocks(lo.V, kFlat), false);
-            blocks(t[TB_FLATX], i, flat_blocks(lo.V, kFlat), true);
-            if (lo.single) blocks(t[TB_FLATS], i, flat_blocks(lo.V, kFlatShift), false);
             blocks(t[TB_TV], i, 8 * lo.vgrid, false);
             blocks(t[TB_TR], i, 8 * lo.red_grid, false);
             blocks(t[TB_TRX], i, 8 * lo.red_grid, true);
         }
-        blocks(t[TB_ROWS], i, row_blocks(lo.V), false);
+        if (lo.need32) {
+            blocks(t[TB_ONE32], i, flat_blocks(6 * lo.V, kFlat), false);
+            blocks(t[TB_FLAT32], i, nflat(i, false), false);
+            blocks(t[TB_FLAT32X], i, nflat(i, false), true);
+        }
     }
     // lattice groups for the FP32 multi-RHS sweep: systems sharing the packed
     // links and the lattice shape, at most kMaxRhs per group
@@ -1049,6 +1107,12 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
     B.pdl = (p->flags & 16) == 0 && !B.use_graph;
     for (int i = 0; i < n; ++i) B.host.push_back(make_dev(B.sys[i], B.lo[i]));
     for (auto& h : B.host) h.fixed_iters = (p->flags & 8) ? 1 : 0;
+    {
+        for (auto& lo : B.lo) B.sites += lo.V;
+        const double many = 4.0 * 8.0 * kFlat * sms();   // elements in four waves of 8 blocks per SM
+        B.ept64 = 12.0 * B.sites >= many ? kFlatMany : 1;
+        B.ept32 = 6.0 * B.sites >= many ? kFlatMany : 1;
+    }
     // Several systems: every launch serves all of them through work tables (any
     // mix of lattice shapes); FP32 sweeps go by lattice groups (systems that
     // share one gauge field and shape) so that a block's right-hand sides read
@@ -1292,6 +1356,15 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
         }
         const int mstart = Kst;
         if (mstart < M) {
+            // the updated r_j of a sub-step (FP32 and double-float iterations of pass 2)
+            for (int i = 0; i < n && prec != FA_F64; ++i) {
+                fa_ctx* c = B.sys[i];
+                if (prec == FA_MIXED_DF) FA_CUDA(c->rb64.ensure(L * B.lo[i].vs64 * sizeof(double2)), "alloc rb64");
+                FA_CUDA(c->rb32.ensure(L * B.lo[i].vs32 * sizeof(float4)), "alloc rb32");
+                B.host[i].rb64 = c->rb64.as<double2>();
+                B.host[i].rb32 = c->rb32.as<float4>();
+            }
+            if (prec != FA_F64) FA_TRY(upload(B));
             int p2 = prec == FA_F64 ? RP64
                    : (prec == FA_F32 ? RP32 : ((switch_outer < 0 || mstart < switch_outer) ? head_rp : RP32));
             for (int i = 0; i < n; ++i) {

@@ -67,8 +67,9 @@ struct TraceScope {
         sm %= ts.nsm;
         const unsigned p = atomicAdd(ts.pos + sm, 1u);
         if (p < ts.per_sm)
-            ts.rec[(size_t)sm * ts.per_sm + p] = TraceRec{t0, t1, kind, (int)(blockIdx.x + gridDim.x * blockIdx.y),
-                                                          (int)sm, (int)(gridDim.x * gridDim.y)};
+            ts.rec[(size_t)sm * ts.per_sm + p] =
+                TraceRec{t0, t1, kind, (int)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)), (int)sm,
+                         (int)(gridDim.x * gridDim.y * gridDim.z)};
         else
             atomicAdd(ts.dropped, 1u);
     }
