@@ -31,23 +31,21 @@ struct Geom {
 // Programmatic dependent launch.  A kernel launched with programmatic stream
 // serialization may be placed on the SMs while its predecessor in the stream
 // is still running; it must not touch global memory before `griddepcontrol.wait`
-// returns, which happens once the predecessor grid has completed and its writes
-// are visible.  `launch_dependents` then lets the successor start its own launch.
-// For an ordinary launch both instructions return at once.  Every kernel that
-// the solver may launch this way calls one of these first.
+// returns (dep_wait), which happens once the predecessor grid has completed and
+// its writes are visible.  For an ordinary launch both instructions return at
+// once.  Every kernel that the solver may launch this way calls dep_wait first.
 //
-// The FP64 kernels let their successor launch only once their main work is done
-// (dep_launch; leaving the kernel counts too): blocks that arrive earlier are
-// placed on the SMs that have room, several on one SM while others still run
-// their predecessor, and blocks that share an SM share its FP64 pipe.  Measured
-// on 8^4, 16 outer iterations of FP64 double pass: 6.98 ms with the successor
-// launched at once, 5.59 ms without programmatic launch.
+// `launch_dependents` lets the successor start its own launch; leaving the
+// kernel counts too.  Kernels call it (dep_launch) once their main work is done,
+// before the ticket and the last block's scalar step: blocks that arrive earlier
+// take the slots and the pipes that the predecessor still needs, and pile up on
+// the SMs that have room.  Measured on GB300, trigger at entry / after the main
+// work / no programmatic launch, all replayed from graphs: 8^4 FP64 double pass,
+// 16 outer iterations (direct launches) 6.98 / 4.62 / 5.59 ms; pseudo-double-pass
+// with a double-float head, 12^3 x 24 9.18 / 8.32 / 8.67 ms, 8^3 x 16 4.95 / 4.58 /
+// 4.77 ms, 16^3 x 32 12.96 / 13.05 / 13.12 ms.
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void dep_sync() {
-    dep_wait();
-    dep_launch();
-}
 
 // ------------------------------------------------------------------ complex
 template <typename R> struct cx { R r, i; };

@@ -40,7 +40,7 @@ struct GramHop {
 template <int L, bool DEFER, int NT, int MB>
 __global__ void __launch_bounds__(NT, MB)
 k_hop_gram(GramHop A, const SolverDev* __restrict__ ds) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<float>(FA_TK_HOP_GRAM));
     const SolverDev& d = ds[0];
     if (sys_idle(d, 0)) return;

@@ -272,7 +272,7 @@ int launch_hop_f64(const Geom& g, const double2* links, const View64& in, const 
                    double eb, double t_bc, double scale, bool g5in, bool g5out, const int* done, cudaStream_t st);
 
 // Kernel launch with programmatic stream serialization when `pdl` is set (see
-// dep_sync) and in clusters of `cluster` blocks.
+// dep_wait) and in clusters of `cluster` blocks.
 template <typename... KArgs, typename... Args>
 inline void launch_ex(bool pdl, int cluster, void (*k)(KArgs...), dim3 grid, int block, cudaStream_t st, Args... args) {
     cudaLaunchAttribute at[2];

@@ -350,7 +350,7 @@ struct Batch {
 
 
 // Launch inside an outer iteration: with `pdl`, programmatic stream
-// serialization (only for kernels that call dep_sync() first and follow
+// serialization (only for kernels that call dep_wait() first and follow
 // another kernel in the stream).
 template <typename... KArgs, typename... Args>
 static void launch(bool pdl, void (*k)(KArgs...), dim3 grid, int block, cudaStream_t st, Args... args) {
@@ -1102,9 +1102,8 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
     B.flags = c0->flagbuf.as<int>();
     // graphs need a capturable stream (not the legacy default stream)
     B.use_graph = (p->flags & 4) != 0 && c0->stream != nullptr && c0->stream != cudaStreamLegacy;
-    // programmatic dependent launch for direct launches only: under CUDA-graph
-    // replay it measured slower (16^3 x 32 headline: 15.00 against 14.62 ms)
-    B.pdl = (p->flags & 16) == 0 && !B.use_graph;
+    // programmatic dependent launch, in captured outer iterations too (flags bit 4: off)
+    B.pdl = (p->flags & 16) == 0;
     for (int i = 0; i < n; ++i) B.host.push_back(make_dev(B.sys[i], B.lo[i]));
     for (auto& h : B.host) h.fixed_iters = (p->flags & 8) ? 1 : 0;
     {

@@ -448,6 +448,7 @@ __device__ __forceinline__ unsigned sm_count_dev() {
 }
 __device__ __forceinline__ int last_block(DevState* S, int ntickets) {
     __shared__ int is_last;
+    dep_launch();
     __syncthreads();
     if (threadIdx.x == 0) {
         // one or several threads stored the block's partials; the fence is cumulative
@@ -1122,7 +1123,7 @@ __device__ __forceinline__ void gram_rows(const SolverDev& d, const Where& w) {
 template <typename R, int L, bool DEFER>
 __global__ void __launch_bounds__(kThreads, gram_min_blocks<R, L>())
 k_gram(const SolverDev* __restrict__ ds, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_GRAM));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -1187,7 +1188,7 @@ template <int L> constexpr int mr_min_blocks() { return L <= 3 ? 4 : 1; }
 template <typename R, int L, bool DEFER>
 __global__ void __launch_bounds__(kThreads, mr_min_blocks<L>())
 k_mr(const SolverDev* __restrict__ ds, ScalarStep step, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_MR, true));
     const Where w = where<true>(tab);
     const SolverDev& d = ds[w.sys];
@@ -1323,8 +1324,8 @@ k_hop64(Geom g, const double2* __restrict__ U, const double2* in, double2* out, 
     __shared__ Smem64<C> sm;
     const int tile = blockIdx.x / C, rank = blockIdx.x % C;
     hop64_tile<C, true, DOT>(g, U, internal64(in, g.V), internal64(out, g.V), op, tile, rank, sm);
-    dep_launch();
     if (DOT && rank == 0) {
+        dep_launch();
         const double2 v = dot64_tile<C>(internal64(dotv, g.V), g.V, tile, sm);
         if (threadIdx.x == 0) partials[tile] = v;
         run_step<false>(ds[0], step, gridDim.x / C, gridDim.x / C);
@@ -1346,8 +1347,8 @@ k_hop64_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel,
     const Op64 op{sc * d.diag, -0.5 * sc, d.ef, d.eb, d.bc, 0, 1};
     hop64_tile<1, true, DOT>(d.g, d.links64, internal64(select_vec<double>(d, in_sel, in_j), d.V),
                              internal64(select_vec<double>(d, out_sel, out_j), d.V), op, w.bx, 0, sm);
-    dep_launch();
     if (DOT) {
+        dep_launch();
         const double2 v = dot64_tile<1>(internal64(d.rt64, d.V), d.V, w.bx, sm);
         if (threadIdx.x == 0) d.part[w.bx] = v;
         run_step<false>(d, step, w.nbx, w.ntk);
@@ -1382,7 +1383,7 @@ __global__ void __launch_bounds__(kHopNarrowThreads, MB)
 k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups, const int4* __restrict__ items,
            int in_sel, int in_j, int out_sel, int out_j, int second, int pass2, ScalarStep step) {
     constexpr int NT = kHopNarrowThreads, NW = NT / 32;
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<float>(FA_TK_HOP_MRHS, DOT));
     const int4 it = items[blockIdx.x];
     const GroupDev& G = groups[it.x];
@@ -1420,6 +1421,7 @@ k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups
         }
     }
     if constexpr (DOT) {
+        dep_launch();
         const int nr = it.w - it.z;
         __syncthreads();
         // a thread per right-hand side: the warps' sums in the order of the block's shuffle
@@ -1464,7 +1466,7 @@ template <typename R, bool DOT>
 __global__ void __launch_bounds__(kRowThreads, rows_sys_min_blocks<DOT>())
 k_hop_sys_rows(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel, int out_j, int second, int pass2,
                ScalarStep step, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_HOP_SYS_ROWS, DOT));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -1492,7 +1494,7 @@ __global__ void __launch_bounds__(kRowThreads, rows_min_blocks<DOT>())
 k_hop1_rows(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cdiag, R chop, R ef, R eb, R bc,
             SpinorView<R> dotv, double2* partials, const int* done, const SolverDev* __restrict__ ds,
             ScalarStep step) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_HOP1_ROWS, DOT));
     if (done != nullptr && *done) return;
     cx<R> dres[1] = {hop_rows_body<R, false, true, DOT>(g, U, in, out, cdiag, chop, ef, eb, bc, dotv, blockIdx.x)};
@@ -1506,7 +1508,7 @@ template <typename R, bool DOT, int NT = kThreads, int MB = hop_min_blocks<R>()>
 __global__ void __launch_bounds__(NT, MB)
 k_hop1(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cdiag, R chop, R ef, R eb, R bc,
        SpinorView<R> dotv, double2* partials, const int* done, const SolverDev* __restrict__ ds, ScalarStep step) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_HOP1, DOT));
     if (done != nullptr && *done) return;
     const int s = blockIdx.x * NT + threadIdx.x;
@@ -1677,7 +1679,7 @@ k_gather(const SolverDev* __restrict__ ds) {
 
 // pass 2: advance the outer-iteration counter
 __global__ void k_advance(const SolverDev* __restrict__ ds) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(FA_TK_ADVANCE);
     DevState* S = ds[blockIdx.x].st;
     if (S->m < S->n_outer) S->m += 1;

@@ -75,8 +75,7 @@ __device__ __forceinline__ double warp_sum(double a) {
 template <typename R, int EPT>
 __global__ void __launch_bounds__(kFlat)
 k_update_u(const SolverDev* __restrict__ ds, int i0, int j, int pass2, const int4* tab) {
-    if constexpr (std::is_same<R, double>::value) dep_wait();
-    else dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_U));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -114,7 +113,7 @@ k_update_u(const SolverDev* __restrict__ ds, int i0, int j, int pass2, const int
 template <typename R, bool PASS2, bool XS, int EPT>
 __global__ void __launch_bounds__(kFlat)
 k_update_r(const SolverDev* __restrict__ ds, int i0, int j, int seed_x, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_R, XS));
     const Where w = where<XS>(tab);
     const SolverDev& d = ds[w.sys];
@@ -164,7 +163,7 @@ template <int L>
 __global__ void __launch_bounds__(kFlat)
 k_deferred(const SolverDev* __restrict__ ds, const int4* tab) {
     using R = df;
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_R, true));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -191,7 +190,7 @@ k_deferred(const SolverDev* __restrict__ ds, const int4* tab) {
 template <typename R, int L>
 __global__ void __launch_bounds__(kFlat)
 k_mr_acc(const SolverDev* __restrict__ ds, const int4* tab) {
-    dep_sync();
+    dep_wait();
     const TraceScope trace_(trace_kind<R>(FA_TK_MR));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
@@ -343,7 +342,6 @@ k_gram_tile(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
             if (L <= 2 && !im && i == k) p[1] = 0.0;
         }
     }
-    dep_launch();
     if (last_block(d.st, w.ntk) == LB_LAST) {
         sc_mr_seed<L, false>(d, w.nbx, false);
         if (shifts) {
@@ -462,7 +460,6 @@ k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const in
         }
     }
     if (DOT) {
-        dep_launch();
         if (rank != 0) return;
         if (q < 3) {
             acc = warp_sum(acc);
