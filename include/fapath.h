@@ -373,7 +373,8 @@ int fa_hop_timing_reset(fa_ctx* ctx);
  * and the backward sweep), for every context on the current device.  While
  * tracing is on, thread 0 of every block of those kernels reads the GPU's global
  * nanosecond timer when the block enters the kernel and again when it leaves,
- * and appends one record to a ring of its SM.  A launch spans from the earliest
+ * and appends one record to a ring of its SM (none for a block that finds its
+ * system finished).  A launch spans from the earliest
  * entry to the latest exit of its blocks; the latest exit includes the scalar
  * step that the last block of a reduction runs.  No work is inserted between
  * launches, so replayed CUDA graphs are timed as they run.  Cost: one atomic

@@ -343,7 +343,8 @@ template <> struct LinkView<df> {
 // double-float; both then in double-float across warps and stored as an FP32
 // pair per part (float4: re.hi, re.lo, im.hi, im.lo) in the same 16 bytes, so
 // that no FP64 instruction is spent (they are scarce on this part).
-// Deterministic for a fixed launch shape.
+// Deterministic for a fixed launch shape.  NT: threads that hold values (the first
+// of the block).
 __device__ __forceinline__ df shfl_down_df(df a, int o) {
     return df(__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o));
 }
@@ -380,6 +381,7 @@ __device__ __forceinline__ void block_reduce_store(cx<R> (&v)[K], double2* out, 
         }
     } else {
         __shared__ float4 sh[K][NW];
+        if (warp < NW) {   // (a block may have further warps, which only meet the barrier)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             if constexpr (std::is_same<R, float>::value) {
@@ -399,6 +401,7 @@ __device__ __forceinline__ void block_reduce_store(cx<R> (&v)[K], double2* out, 
                 }
                 if (lane == 0) sh[k][warp] = make_float4(a.hi, a.lo, b.hi, b.lo);
             }
+        }
         }
         __syncthreads();
         if (warp == 0) {

@@ -37,23 +37,25 @@ struct GramHop {
 // r_l = c g5 D tmp and the partials of <r_i, r_k> (i <= k <= L) in the order of
 // the Gram kernel, then the MR coefficients in the last block.
 // DEFER: the updates of r that the sub-steps deferred come first.
-template <int L, bool DEFER, int NT, int MB>
-__global__ void __launch_bounds__(NT, MB)
+// S = 2: the sweep of small lattices (two threads per site, NT = 128 sites per block).
+template <int L, bool DEFER, int NT, int MB, int S = 1>
+__global__ void __launch_bounds__(NT * S, MB)
 k_hop_gram(GramHop A, const SolverDev* __restrict__ ds) {
     dep_wait();
-    const TraceScope trace_(trace_kind<float>(FA_TK_HOP_GRAM));
     const SolverDev& d = ds[0];
     if (sys_idle(d, 0)) return;
-    const int s = (int)blockIdx.x * NT + (int)threadIdx.x;
+    const TraceScope trace_(trace_kind<float>(FA_TK_HOP_GRAM));
+    const int s = (int)blockIdx.x * NT + (int)(threadIdx.x % NT);
     const int V = A.g.V;
     constexpr int NG = n_gram(L);
     cx<float> red[NG];
 #pragma unroll
     for (int k = 0; k < NG; ++k) red[k] = czero<float>();
-    if (s < V) {
-        cx<float> p[12];
-        hop_site<float, false, true>(A.g, A.U, SpinorView<float>{const_cast<float4*>(A.in), V}, s, A.cdiag, A.chop,
-                                     A.ef, A.eb, A.bc, p);
+    cx<float> p[12];
+    const SpinorView<float> in{const_cast<float4*>(A.in), V};
+    if constexpr (S > 1) hop_site_split<false, true>(A.g, A.U, in, s, A.cdiag, A.chop, A.ef, A.eb, A.bc, p);
+    else if (s < V) hop_site<float, false, true>(A.g, A.U, in, s, A.cdiag, A.chop, A.ef, A.eb, A.bc, p);
+    if (s < V && threadIdx.x < NT) {
         SpinorView<float>{A.out, V}.store(s, p);
         const StepScalars<float, DEFER ? L : 1> sc(d, d.st->m);
 #pragma unroll

@@ -79,11 +79,10 @@ __device__ __forceinline__ void load_in(const SV& in, int s, cx<R> p[12]) {
     }
 }
 
-// forward hop from site s to neighbour nb: acc += w (1 - g_MU) U_MU(s) psi(nb)
+// forward hop from site s to neighbour nb: the spin rows c of w (1 - g_MU) U_MU(s) psi(nb)
 template <int MU, bool WEIGHT, bool G5IN, typename R, typename SV>
-__device__ __forceinline__ void hop_fwd(cx<R> acc[12], const SV& in, const LinkView<R>& U,
-                                        int s, int nb, R w) {
-    cx<R> p[12], h[6], L[3][3], c[6];
+__device__ __forceinline__ void hop_fwd_rows(cx<R> c[6], const SV& in, const LinkView<R>& U, int s, int nb, R w) {
+    cx<R> p[12], h[6], L[3][3];
     load_in<R, G5IN>(in, nb, p);
     project<MU, +1>(p, h);
     U.load(MU, s, L);
@@ -96,14 +95,12 @@ __device__ __forceinline__ void hop_fwd(cx<R> acc[12], const SV& in, const LinkV
             t = cfma(L[a][2], h[3 * sp + 2], t);
             c[3 * sp + a] = WEIGHT ? cscale(w, t) : t;
         }
-    recon_add<MU, +1>(acc, c);
 }
 
-// backward hop: acc += w (1 + g_MU) U_MU(nb)^H psi(nb), nb = s - MU
+// backward hop: the spin rows of w (1 + g_MU) U_MU(nb)^H psi(nb), nb = s - MU
 template <int MU, bool WEIGHT, bool G5IN, typename R, typename SV>
-__device__ __forceinline__ void hop_bwd(cx<R> acc[12], const SV& in, const LinkView<R>& U,
-                                        int nb, R w) {
-    cx<R> p[12], h[6], L[3][3], c[6];
+__device__ __forceinline__ void hop_bwd_rows(cx<R> c[6], const SV& in, const LinkView<R>& U, int nb, R w) {
+    cx<R> p[12], h[6], L[3][3];
     load_in<R, G5IN>(in, nb, p);
     project<MU, -1>(p, h);
     U.load(MU, nb, L);
@@ -116,6 +113,18 @@ __device__ __forceinline__ void hop_bwd(cx<R> acc[12], const SV& in, const LinkV
             t = cjfma(L[2][a], h[3 * sp + 2], t);
             c[3 * sp + a] = WEIGHT ? cscale(w, t) : t;
         }
+}
+
+template <int MU, bool WEIGHT, bool G5IN, typename R, typename SV>
+__device__ __forceinline__ void hop_fwd(cx<R> acc[12], const SV& in, const LinkView<R>& U, int s, int nb, R w) {
+    cx<R> c[6];
+    hop_fwd_rows<MU, WEIGHT, G5IN>(c, in, U, s, nb, w);
+    recon_add<MU, +1>(acc, c);
+}
+template <int MU, bool WEIGHT, bool G5IN, typename R, typename SV>
+__device__ __forceinline__ void hop_bwd(cx<R> acc[12], const SV& in, const LinkView<R>& U, int nb, R w) {
+    cx<R> c[6];
+    hop_bwd_rows<MU, WEIGHT, G5IN>(c, in, U, nb, w);
     recon_add<MU, -1>(acc, c);
 }
 
@@ -159,6 +168,104 @@ __device__ __forceinline__ void hop_site(const Geom& g, const LinkView<R>& U, co
         cx<R> o = cscale(a, p[k]);
         o = crfma(b, acc[k], o);
         p[k] = o;
+    }
+}
+
+// ------------------------------------------------------------------ FP32 sweep of small lattices
+// The sweep with two threads per site, for lattices that leave most of the
+// chip's warps idle.  One thread walks its eight hops one after the other
+// (registers hold about one hop's loads), so the sweep takes eight trips to L2
+// however small the lattice is.  Here a block of 256 threads has 128 sites:
+// warps 0-3 take the hops x+, x-, y+, y-, warps 4-7 the rest and leave their spin
+// rows in shared memory, which the first half adds in that order, then the
+// diagonal term, as one thread would: the same bits.  The first half's threads
+// hold the result.  Used while the lattice is one wave of such blocks (three per
+// SM).  Measured on GB300, us per FP32 outer iteration (l = 2, graph) with 1 / 2 /
+// 4 / 8 threads per site: 512 sites 100.5 / 92.3 / 94.6 / 98.0, 8192 sites 101.6 /
+// 92.4 / 94.7 / 98.8, 31104 sites 118 / 109 / 118 / 153, 48384 sites 129 / 126 /
+// 160 / 197, 65856 sites (more than a wave) 145 / 172 / 184 / 250.
+template <int HOP, bool G5IN>
+__device__ __forceinline__ void hop32_rows(cx<float> c[6], const Geom& g, const LinkView<float>& U,
+                                           const SpinorView<float>& in, int s, const int pos[4], float ef, float eb,
+                                           float bc) {
+    constexpr int MU = HOP >> 1;
+    const int ext = MU == 0 ? g.X : MU == 1 ? g.Y : MU == 2 ? g.Z : g.T;
+    const int str = MU == 0 ? 1 : MU == 1 ? g.X : MU == 2 ? g.X * g.Y : g.X * g.Y * g.Z;
+    const int x = pos[MU];
+    if constexpr ((HOP & 1) == 0) {
+        const int nb = x == ext - 1 ? s - (ext - 1) * str : s + str;
+        const float w = MU == 3 ? (x == ext - 1 ? mulR(ef, bc) : ef) : 1.0f;
+        hop_fwd_rows<MU, MU == 3, G5IN>(c, in, U, s, nb, w);
+    } else {
+        const int nb = x == 0 ? s + (ext - 1) * str : s - str;
+        const float w = MU == 3 ? (x == 0 ? mulR(eb, bc) : eb) : 1.0f;
+        hop_bwd_rows<MU, MU == 3, G5IN>(c, in, U, nb, w);
+    }
+}
+template <int HOP> __device__ __forceinline__ void hop32_add(cx<float> acc[12], const cx<float> c[6]) {
+    recon_add<(HOP >> 1), (HOP & 1) ? -1 : 1>(acc, c);
+}
+constexpr int kSplitSites = 128;
+constexpr int kSplitBlocks = 3;   // blocks of 2 kSplitSites threads per SM (80 registers)
+struct SplitRows { float2 h[4][6][kSplitSites]; };
+template <int HOP, int END, bool G5IN>
+__device__ __forceinline__ void split_part(cx<float> acc[12], SplitRows& sm, const Geom& g, const LinkView<float>& U,
+                                           const SpinorView<float>& in, int s, int i, const int pos[4], float ef,
+                                           float eb, float bc) {
+    if constexpr (HOP < END) {
+        cx<float> c[6];
+        hop32_rows<HOP, G5IN>(c, g, U, in, s, pos, ef, eb, bc);
+        if constexpr (HOP < 4) {
+            hop32_add<HOP>(acc, c);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) sm.h[HOP - 4][k][i] = make_float2(c[k].r, c[k].i);
+        }
+        split_part<HOP + 1, END, G5IN>(acc, sm, g, U, in, s, i, pos, ef, eb, bc);
+    }
+}
+template <int HOP> __device__ __forceinline__ void split_sum(cx<float> acc[12], const SplitRows& sm, int i) {
+    if constexpr (HOP < 8) {
+        cx<float> c[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const float2 t = sm.h[HOP - 4][k][i];
+            c[k] = {t.x, t.y};
+        }
+        hop32_add<HOP>(acc, c);
+        split_sum<HOP + 1>(acc, sm, i);
+    }
+}
+// p: out of hop_site at `site` in the first half's threads (every thread of the
+// block calls it); sites past the end compute the last site
+template <bool G5IN, bool G5OUT>
+__device__ __forceinline__ void hop_site_split(const Geom& g, const LinkView<float>& U, const SpinorView<float>& in,
+                                               int site, float cdiag, float chop, float ef, float eb, float bc,
+                                               cx<float> p[12]) {
+    __shared__ SplitRows sm;
+    const int i = threadIdx.x & (kSplitSites - 1);
+    const bool first = threadIdx.x < kSplitSites;
+    const int s = min(site, g.V - 1);
+    const int r1 = s / g.X, r2 = r1 / g.Y;
+    const int pos[4] = {s - r1 * g.X, r1 - r2 * g.Y, r2 % g.Z, r2 / g.Z};
+    cx<float> acc[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = czero<float>();
+    if (first) {
+        split_part<0, 4, G5IN>(acc, sm, g, U, in, s, i, pos, ef, eb, bc);
+        load_in<float, G5IN>(in, s, p);
+    } else {
+        split_part<4, 8, G5IN>(acc, sm, g, U, in, s, i, pos, ef, eb, bc);
+    }
+    __syncthreads();
+    if (!first) return;
+    split_sum<4>(acc, sm, i);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const bool neg = G5OUT && k >= 6;
+        const float a = neg ? -cdiag : cdiag, b = neg ? -chop : chop;
+        cx<float> o = cscale(a, p[k]);
+        p[k] = crfma(b, acc[k], o);
     }
 }
 

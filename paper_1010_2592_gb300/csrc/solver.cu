@@ -363,12 +363,18 @@ static int upload(Batch& B) {
     return FA_OK;
 }
 
-static inline ScalarStep none_step() { return ScalarStep{STEP_NONE, 0}; }
 
 // working precision of a stretch of outer iterations
 enum Rp { RP64 = 0, RP32 = 1, RPDF = 2 };
 template <typename R> constexpr int rp_of() {
     return std::is_same<R, double>::value ? RP64 : (std::is_same<R, float>::value ? RP32 : RPDF);
+}
+
+// Two threads per site in a one-system FP32 sweep (hop_site_split) while the
+// lattice is one wave of its blocks.  The wide shape, where it is asked for, is
+// left alone.
+static bool hop32_split(int shape, int V) {
+    return shape != FA_SHAPE_WIDE && (V + kSplitSites - 1) / kSplitSites <= kSplitBlocks * sms();
 }
 
 // Whether pass 1 defers the updates i < j of its sub-steps (vec_tile.cuh): always
@@ -465,7 +471,15 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
                 else if (split == 2) go(std::integral_constant<int, 2>{});
                 else go(std::integral_constant<int, 4>{});
             } else {
-                if (hop_use_narrow(c->hop_shape, V)) {
+                if (hop32_split(c->hop_shape, V)) {
+                    const int nbh = (V + kSplitSites - 1) / kSplitSites;
+                    if (dot)
+                        launch(pdl, k_hop1_split<true>, nbh, 2 * kSplitSites, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
+                               vdot, h0.part, done, ds, step);
+                    else
+                        launch(pdl, k_hop1_split<false>, nbh, 2 * kSplitSites, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
+                               vdot, nullptr, done, ds, none);
+                } else if (hop_use_narrow(c->hop_shape, V)) {
                     constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks;
                     const int nbh = (V + NT - 1) / NT;
                     if (dot)
@@ -556,7 +570,12 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
             a.eb = host_cvt<float>(h0.eb);
             a.bc = host_cvt<float>(h0.bc);
             if (timing) hop_timing_begin(c, 6);
-            if (hop_use_narrow(c->hop_shape, h0.V)) {
+            if (hop32_split(c->hop_shape, h0.V)) {
+                constexpr int NT = kSplitSites, MB = kSplitBlocks;
+                const dim3 gh((h0.V + NT - 1) / NT);
+                if (defer) launch(pdl, k_hop_gram<L, (L > 1), NT, MB, 2>, gh, 2 * NT, st, a, ds);
+                else launch(pdl, k_hop_gram<L, (L > 2), NT, MB, 2>, gh, 2 * NT, st, a, ds);
+            } else if (hop_use_narrow(c->hop_shape, h0.V)) {
                 constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks;
                 const dim3 gh((h0.V + NT - 1) / NT);
                 if (defer) launch(pdl, k_hop_gram<L, (L > 1), NT, MB>, gh, NT, st, a, ds);

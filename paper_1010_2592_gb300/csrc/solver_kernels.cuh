@@ -1189,10 +1189,10 @@ template <typename R, int L, bool DEFER>
 __global__ void __launch_bounds__(kThreads, mr_min_blocks<L>())
 k_mr(const SolverDev* __restrict__ ds, ScalarStep step, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_MR, true));
     const Where w = where<true>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, 0)) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_MR, true));
     const int bx = w.bx, nbx = w.nbx;
     if (bx < 0) {
         sc_mr_shifts<L>(d);
@@ -1319,8 +1319,8 @@ __global__ void __launch_bounds__(hop64_threads<C>(), hop64_min_blocks<C>())
 k_hop64(Geom g, const double2* __restrict__ U, const double2* in, double2* out, Op64 op, const double2* dotv,
         double2* partials, const int* done, const SolverDev* __restrict__ ds, ScalarStep step) {
     dep_wait();
-    const TraceScope trace_(trace_kind<double>(FA_TK_HOP1, DOT));
     if (done != nullptr && *done) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_HOP1, DOT));
     __shared__ Smem64<C> sm;
     const int tile = blockIdx.x / C, rank = blockIdx.x % C;
     hop64_tile<C, true, DOT>(g, U, internal64(in, g.V), internal64(out, g.V), op, tile, rank, sm);
@@ -1338,10 +1338,10 @@ __global__ void __launch_bounds__(hop64_threads<1>(), hop64_min_blocks<1>())
 k_hop64_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel, int out_j, int second, int pass2,
             ScalarStep step, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<double>(FA_TK_HOP_SYS, DOT));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, pass2)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_HOP_SYS, DOT));
     __shared__ Smem64<1> sm;
     const double sc = second ? d.scale : 1.0;
     const Op64 op{sc * d.diag, -0.5 * sc, d.ef, d.eb, d.bc, 0, 1};
@@ -1467,10 +1467,10 @@ __global__ void __launch_bounds__(kRowThreads, rows_sys_min_blocks<DOT>())
 k_hop_sys_rows(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel, int out_j, int second, int pass2,
                ScalarStep step, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_HOP_SYS_ROWS, DOT));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, pass2)) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_HOP_SYS_ROWS, DOT));
     const double sc = second ? d.scale : 1.0;
     const Geom g = d.g;
     const SpinorView<R> in{select_vec<R>(d, in_sel, in_j), d.V}, out{select_vec<R>(d, out_sel, out_j), d.V};
@@ -1495,8 +1495,8 @@ k_hop1_rows(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cdiag,
             SpinorView<R> dotv, double2* partials, const int* done, const SolverDev* __restrict__ ds,
             ScalarStep step) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_HOP1_ROWS, DOT));
     if (done != nullptr && *done) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_HOP1_ROWS, DOT));
     cx<R> dres[1] = {hop_rows_body<R, false, true, DOT>(g, U, in, out, cdiag, chop, ef, eb, bc, dotv, blockIdx.x)};
     if (DOT) {
         block_reduce_store<1, R, kRowThreads>(dres, partials, 0, blockIdx.x);
@@ -1509,8 +1509,8 @@ __global__ void __launch_bounds__(NT, MB)
 k_hop1(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cdiag, R chop, R ef, R eb, R bc,
        SpinorView<R> dotv, double2* partials, const int* done, const SolverDev* __restrict__ ds, ScalarStep step) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_HOP1, DOT));
     if (done != nullptr && *done) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_HOP1, DOT));
     const int s = blockIdx.x * NT + threadIdx.x;
     cx<R> dres[1] = {czero<R>()};
     if (s < g.V) {
@@ -1532,6 +1532,36 @@ k_hop1(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cdiag, R ch
     }
 }
 
+// the FP32 sweep with two threads per site (hop_site_split), 128 sites per block
+template <bool DOT>
+__global__ void __launch_bounds__(2 * kSplitSites, kSplitBlocks)
+k_hop1_split(Geom g, LinkView<float> U, SpinorView<float> in, SpinorView<float> out, float cdiag, float chop, float ef,
+             float eb, float bc, SpinorView<float> dotv, double2* partials, const int* done,
+             const SolverDev* __restrict__ ds, ScalarStep step) {
+    dep_wait();
+    if (done != nullptr && *done) return;
+    const TraceScope trace_(trace_kind<float>(FA_TK_HOP1, DOT));
+    const int s = blockIdx.x * kSplitSites + (threadIdx.x & (kSplitSites - 1));
+    cx<float> dres[1] = {czero<float>()};
+    cx<float> p[12];
+    hop_site_split<false, true>(g, U, in, s, cdiag, chop, ef, eb, bc, p);
+    if (threadIdx.x < kSplitSites && s < g.V) {
+        out.store(s, p);
+        if (DOT) {
+            cx<float> q[12];
+            dotv.load(s, q);
+            cx<float> a = czero<float>();
+#pragma unroll
+            for (int k = 0; k < 12; ++k) a = cjfma(q[k], p[k], a);
+            dres[0] = a;
+        }
+    }
+    if (DOT) {
+        block_reduce_store<1, float, kSplitSites>(dres, partials, 0, blockIdx.x);
+        run_step<true>(ds[0], step, gridDim.x, gridDim.x);
+    }
+}
+
 // ------------------------------------------------------------------ reliable update
 // r_0 <- b - A x with A x (FP64) already in ax; the new r_0 is rounded to R.
 // Rewrites the partials of <rt, r_0> (slot 0) and |r_0|^2 (slot 1) that the
@@ -1539,9 +1569,9 @@ k_hop1(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cdiag, R ch
 template <typename R>
 __global__ void __launch_bounds__(kThreads, kVecBlocks)
 k_reliable(const SolverDev* __restrict__ ds, const double2* ax, int pass2, ScalarStep step) {
-    const TraceScope trace_(trace_kind<R>(FA_TK_RELIABLE));
     const SolverDev& d = ds[blockIdx.y];   // one system (reliable updates are not batched)
     if (sys_idle(d, pass2)) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_RELIABLE));
     typename Ch<R>::T* r0 = Vec<R>::r(d);
     const typename Ch<R>::T* rt = Vec<R>::rt(d);
     cx<R> dots[2] = {czero<R>(), czero<R>()};

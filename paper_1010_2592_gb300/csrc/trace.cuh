@@ -3,7 +3,8 @@
 // While tracing is on, thread 0 of every block of a traced kernel reads the
 // GPU's global nanosecond timer (%globaltimer) when the block enters the kernel
 // body and again when thread 0 leaves it, and appends one record (entry, exit,
-// kernel, block, SM, grid size) to a ring of its SM.  A launch then spans from
+// kernel, block, SM, grid size) to a ring of its SM; a block that finds its
+// system finished (iterations enqueued past convergence) leaves none.  A launch then spans from
 // the earliest entry to the latest exit of its blocks; the exit of the last
 // block includes the scalar step it runs.  Unlike CUDA events, the records need
 // no work between launches, so they time the kernels of a replayed CUDA graph

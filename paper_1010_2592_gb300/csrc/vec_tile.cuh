@@ -76,10 +76,10 @@ template <typename R, int EPT>
 __global__ void __launch_bounds__(kFlat)
 k_update_u(const SolverDev* __restrict__ ds, int i0, int j, int pass2, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_U));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, pass2)) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_U));
     const int n = flat_elems<R>(d.V), e0 = w.bx * (kFlat * EPT) + threadIdx.x;
     const cx<R> nb = nweight<R>(d.rec_beta, d.rec_beta4, d.st->m * d.L + j);
     for (int i = i0; i <= j; ++i) {
@@ -114,10 +114,10 @@ template <typename R, bool PASS2, bool XS, int EPT>
 __global__ void __launch_bounds__(kFlat)
 k_update_r(const SolverDev* __restrict__ ds, int i0, int j, int seed_x, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_R, XS));
     const Where w = where<XS>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, PASS2)) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_R, XS));
     if (XS && w.bx < 0) {
         sc_alpha_shifts(d, j);
         return;
@@ -164,10 +164,10 @@ __global__ void __launch_bounds__(kFlat)
 k_deferred(const SolverDev* __restrict__ ds, const int4* tab) {
     using R = df;
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_R, true));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, 0)) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_UPDATE_R, true));
     const int n = 12 * d.V, e = w.bx * kFlat + threadIdx.x, m = d.st->m;
     if (e >= n) return;
     float4 *rp = Vec<R>::r(d) + e, *up = Vec<R>::u(d) + e;
@@ -191,10 +191,10 @@ template <typename R, int L>
 __global__ void __launch_bounds__(kFlat)
 k_mr_acc(const SolverDev* __restrict__ ds, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_MR));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, 1)) return;
+    const TraceScope trace_(trace_kind<R>(FA_TK_MR));
     const int V = d.V, n = flat_elems<R>(V), e = w.bx * kFlat + threadIdx.x, m = d.st->m;
     if (e >= n) return;
     const int q = e / V, s = e - q * V;
@@ -237,10 +237,10 @@ template <bool ACC, bool SHIFTS, bool XS>
 __global__ void __launch_bounds__(kFlat)
 k_update_r64(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<double>(FA_TK_UPDATE_R, XS));
     const Where w = where<XS>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, pass2)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_UPDATE_R, XS));
     if (XS && w.bx < 0) {
         sc_alpha_shifts(d, j);
         return;
@@ -309,10 +309,10 @@ template <int L>
 __global__ void __launch_bounds__(32 * kGramWarps)
 k_gram_tile(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<double>(FA_TK_GRAM));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, 0)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_GRAM));
     constexpr int NG = n_gram(L), NW = kGramWarps;
     constexpr int NCH = L <= 2 ? 2 * NG - (L + 1) : 2 * NG;
     const int V = d.V, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -363,7 +363,6 @@ __global__ void __launch_bounds__(kMrThreads)
 k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const int4* tab) {
     static_assert(C == 1 || (SHIFTS && !XS), "clusters split the shifts");
     dep_wait();
-    const TraceScope trace_(trace_kind<double>(FA_TK_MR, XS));
     Where w = where<XS>(tab);
     int rank = 0;
     if constexpr (C > 1) {
@@ -374,6 +373,7 @@ k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const in
     }
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, pass2)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_MR, XS));
     if (XS && w.bx < 0) {
         sc_mr_shifts<L>(d);
         __threadfence();   // the new zeta of every thread before the ticket
