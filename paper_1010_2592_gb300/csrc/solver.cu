@@ -657,9 +657,14 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
             }
             constexpr bool D1 = rp_of<R>() == RP32 && L > 1, D0 = rp_of<R>() == RP32 && L > 2;
             dim3 g = grid(gram_vec ? TB_VEC : TB_RG, gram_vec ? vg : rg, t);
-            g.z = gram_groups<R, L>();
-            if (defer) launch(pdl, k_gram<R, L, D1>, g, kThreads, st, ds, t);
-            else launch(pdl, k_gram<R, L, D0>, g, kThreads, st, ds, t);
+            // double-float: the rows of the triangle in groups, at l = 2 while their blocks
+            // are one wave
+            constexpr bool G2 = rp_of<R>() == RPDF && L >= 2, G1 = rp_of<R>() == RPDF && L > 2;
+            const bool groups = L > 2 || (int)(g.x * 2) <= 3 * sms();
+            if (G2 && groups) g.z = gram_groups<R, L>();
+            if (G2 && groups) launch(pdl, k_gram<R, L, false, G2>, g, kThreads, st, ds, t);
+            else if (defer) launch(pdl, k_gram<R, L, D1, G1>, g, kThreads, st, ds, t);
+            else launch(pdl, k_gram<R, L, D0, G1>, g, kThreads, st, ds, t);
         }
         FA_LAUNCHED(c, "k_gram");
     }
@@ -1345,11 +1350,8 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
 
     // ---- backward sweep, gather of the stored prefix, pass 2 for the rest
     if (rc_all == FA_OK && !single) {
-        for (int i = 0; i < n; ++i)
-            FA_CUDA(cudaMemsetAsync(B.host[i].cs, 0, (size_t)B.sys[i]->ns * Lo.max_outer * NC * sizeof(double2), st),
-                    "zero sweep");
         FA_TRY(launch_sweep(B));
-        k_coef_reduce<<<dim3((M * NC + 255) / 256, n), 256, 0, st>>>(B.dev);
+        k_coef_reduce<<<dim3((M * NC + 31) / 32, n), 256, 0, st>>>(B.dev);
         FA_LAUNCHED(c0, "k_coef_reduce");
         if (timing) cudaEventRecord(ev[2], st);
         // the largest lattice of the batch sets the grids (blocks beyond a smaller

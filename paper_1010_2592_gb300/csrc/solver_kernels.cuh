@@ -701,6 +701,26 @@ __device__ __noinline__ void sc_init(const SolverDev& d, int nblk, double tol, d
     }
 }
 
+// beta of BiCG sub-step j >= 1 from rho1 = <rt, r_j>, by one thread
+__device__ __forceinline__ void seed_beta(const SolverDev& d, int j, int m, dcx rho0, dcx alpha, dcx rho1) {
+    DevState* S = d.st;
+    if (zabs2(rho0) == 0.0) { fail(S, FA_EBREAKDOWN); return; }
+    const dcx beta = zmul(zmul(alpha, rho1), zinv(rho0));
+    if (!zfinite(beta)) { fail(S, FA_ENONFINITE); return; }
+    S->rho0 = pk(rho1);
+    put_scalar(d.rec_beta, d.rec_beta4, m * d.L + j, beta);
+}
+// alpha of BiCG sub-step j from den = <rt, u_{j+1}>, by one thread
+__device__ __forceinline__ void seed_alpha(const SolverDev& d, int j, int m, dcx rho0, dcx den) {
+    DevState* S = d.st;
+    if (zabs2(den) == 0.0) { fail(S, FA_EBREAKDOWN); return; }
+    const dcx alpha = zmul(rho0, zinv(den));
+    if (!zfinite(alpha)) { fail(S, FA_ENONFINITE); return; }
+    put_scalar(d.rec_alpha, d.rec_alpha4, m * d.L + j, alpha);
+    S->alpha = pk(alpha);
+    S->alpha_prev = pk(alpha);
+}
+
 // beta of BiCG sub-step j >= 1 from partials of <rt, r_j>
 template <bool DFP>
 __device__ __noinline__ void sc_beta(const SolverDev& d, int j, int nblk, bool dry) {
@@ -1081,10 +1101,14 @@ __device__ __forceinline__ void reduce_store(cx<R> (&v)[K], double2* out, int nb
 // the arithmetic is 0.95 ms.  The component loop is not unrolled whole: its code
 // (85 KB for l = 2) did not stay in the instruction cache.
 template <typename R, int L> constexpr int gram_groups() { return std::is_same<R, float>::value || L == 1 ? 1 : (L + 2) / 2; }
+// l = 2: groups while their blocks are one wave of 3 per SM, else all products in a thread
+// (12^3 x 24: 34 -> 19 us; 16^3 x 32: 43 us, 54 in groups)
 // rows of group z: l even {0}, {1, l}, {2, l - 1}, ...; l odd {0, l}, {1, l - 1}, ...
 template <int L> constexpr int gram_row_a(int z) { return z; }
 template <int L> constexpr int gram_row_b(int z) { return L % 2 ? L - z : (z == 0 ? -1 : L + 1 - z); }
-template <typename R, int L> constexpr int gram_min_blocks() { return std::is_same<R, float>::value ? (L <= 2 ? 4 : 1) : (L <= 4 ? 3 : 2); }
+template <typename R, int L, bool GROUPS> constexpr int gram_min_blocks() {
+    return !GROUPS ? (L <= 2 ? 4 : 1) : (L <= 4 ? 3 : 2);
+}
 template <int L> constexpr int gram_row_slot(int i) { return i * (L + 1) - i * (i - 1) / 2; }
 
 template <typename R, int L, int Z>
@@ -1120,15 +1144,15 @@ __device__ __forceinline__ void gram_rows(const SolverDev& d, const Where& w) {
     if constexpr (NB > 0) block_reduce_store<NB, R>(b, d.part + (size_t)gram_row_slot<L>(B) * w.nbx, w.nbx, w.bx);
 }
 
-template <typename R, int L, bool DEFER>
-__global__ void __launch_bounds__(kThreads, gram_min_blocks<R, L>())
+template <typename R, int L, bool DEFER, bool GROUPS>
+__global__ void __launch_bounds__(kThreads, gram_min_blocks<R, L, GROUPS>())
 k_gram(const SolverDev* __restrict__ ds, const int4* tab) {
     dep_wait();
-    const TraceScope trace_(trace_kind<R>(FA_TK_GRAM));
     const Where w = where<false>(tab);
     const SolverDev& d = ds[w.sys];
     if (sys_idle(d, 0)) return;
-    constexpr int NZ = gram_groups<R, L>();
+    const TraceScope trace_(trace_kind<R>(FA_TK_GRAM));
+    constexpr int NZ = GROUPS ? gram_groups<R, L>() : 1;
     if constexpr (NZ > 1) {
         if (blockIdx.z == 0) gram_rows<R, L, 0>(d, w);
         else if (blockIdx.z == 1) gram_rows<R, L, 1>(d, w);
@@ -1145,27 +1169,33 @@ k_gram(const SolverDev* __restrict__ ds, const int4* tab) {
         for (int k = 0; k < NG; ++k) acc[k] = czero<R>();
         int s0, s1;
         site_range(d.V, w.bx, w.nbx, s0, s1);
-        for (int s = s0 + threadIdx.x; s < s1; s += kThreads) {
+        auto chunk = [&](int q, int s) {
+            Ch<R> v[L + 1];
 #pragma unroll
-            for (int q = 0; q < Ch<R>::N; ++q) {
-                Ch<R> v[L + 1];
+            for (int i = 0; i <= L; ++i) v[i] = Ch<R>::ld(r + i * vs, q, d.V, s);
+            if constexpr (DEFER) {
+                Ch<R> u[L];
 #pragma unroll
-                for (int i = 0; i <= L; ++i) v[i] = Ch<R>::ld(r + i * vs, q, d.V, s);
-                if constexpr (DEFER) {
-                    Ch<R> u[L];
+                for (int i = 1; i < L; ++i) u[i] = Ch<R>::ld(ub + i * vs, q, d.V, s);
+                deferred_r<R, L>(sc, v, u);
+            }
+            int g = 0;
 #pragma unroll
-                    for (int i = 1; i < L; ++i) u[i] = Ch<R>::ld(ub + i * vs, q, d.V, s);
-                    deferred_r<R, L>(sc, v, u);
+            for (int i = 0; i <= L; ++i)
+#pragma unroll
+                for (int k = i; k <= L; ++k) {
+#pragma unroll
+                    for (int w = 0; w < Ch<R>::W; ++w) acc[g] = cjfma(v[i].c[w], v[k].c[w], acc[g]);
+                    ++g;
                 }
-                int g = 0;
+        };
+        for (int s = s0 + threadIdx.x; s < s1; s += kThreads) {
+            if constexpr (std::is_same<R, float>::value) {
 #pragma unroll
-                for (int i = 0; i <= L; ++i)
-#pragma unroll
-                    for (int k = i; k <= L; ++k) {
-#pragma unroll
-                        for (int w = 0; w < Ch<R>::W; ++w) acc[g] = cjfma(v[i].c[w], v[k].c[w], acc[g]);
-                        ++g;
-                    }
+                for (int q = 0; q < Ch<R>::N; ++q) chunk(q, s);
+            } else {
+#pragma unroll 2
+                for (int q = 0; q < Ch<R>::N; ++q) chunk(q, s);
             }
         }
         block_reduce_store<NG, R>(acc, d.part, w.nbx, w.bx);
@@ -1364,6 +1394,59 @@ struct GroupDev {
     int sys[kMaxRhs];      // descriptor index of each system
 };
 
+// The seed steps (beta or alpha) of the systems whose last ticket this block
+// holds: it often is the last for all right-hand sides of its run, so their
+// partials are summed side by side and a thread per system runs the step
+// (reduce_slots, sc_beta and sc_alpha_seed, the same operations in the same
+// order).
+__device__ __noinline__ void mrhs_steps(const SolverDev* __restrict__ ds, const GroupDev& G, int first, int nr,
+                                        const int* lasts, ScalarStep e) {
+    __shared__ float4 qf[4 * kMaxRhs];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nblk = G.ntile, per = (nblk + 3) >> 2;
+    for (int u = warp; u < 4 * nr; u += nw) {
+        if (!lasts[u >> 2]) continue;
+        const float4* pf = reinterpret_cast<const float4*>(ds[G.sys[first + (u >> 2)]].part);
+        const int i0 = (u & 3) * per, i1 = min(nblk, i0 + per);
+        df a(0.0f), b(0.0f);
+        for (int ib = i0 + lane; ib < i1; ib += 32 * 8) {
+            float4 v[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const int i = ib + 32 * t;
+                v[t] = i < i1 ? __ldcg(pf + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                a = addR(a, df(v[t].x, v[t].y));
+                b = addR(b, df(v[t].z, v[t].w));
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a = addR(a, shfl_down_df(a, o));
+            b = addR(b, shfl_down_df(b, o));
+        }
+        if (lane == 0) qf[u] = make_float4(a.hi, a.lo, b.hi, b.lo);
+    }
+    __syncthreads();
+    const int r = threadIdx.x;
+    if (r >= nr || !lasts[r]) return;
+    const SolverDev& d = ds[G.sys[first + r]];
+    DevState* S = d.st;
+    df a(0.0f), b(0.0f);
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+        const float4 t = qf[4 * r + q];
+        a = addR(a, df(t.x, t.y));
+        b = addR(b, df(t.z, t.w));
+    }
+    if (S->done) return;
+    const dcx red = {todbl(a), todbl(b)};
+    if (e.kind == STEP_BETA) seed_beta(d, e.arg, S->m, ld(S->rho0), ld(S->alpha), red);
+    else seed_alpha(d, e.arg, S->m, ld(S->rho0), red);
+}
+
 // FP32 sweep of a batch, several right-hand sides per block.  items[blockIdx.x]
 // = (group, tile, first, end): the block applies the sweep to the systems
 // first..end-1 of the group on the tile's sites, one after the other, so the
@@ -1456,8 +1539,9 @@ k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups
             lasts[threadIdx.x] = last;
         }
         __syncthreads();
-        for (int r = 0; r < nr; ++r)
-            if (lasts[r]) do_step<true>(ds[G.sys[it.z + r]], step, G.ntile, false);
+        int any = 0;
+        for (int r = 0; r < nr; ++r) any |= lasts[r];
+        if (any) mrhs_steps(ds, G, it.z, nr, lasts, step);
     }
 }
 
@@ -1730,8 +1814,30 @@ __global__ void k_flags(const SolverDev* __restrict__ ds, int n, int* out) {
 // One thread per shift walks its recorded linear operations backwards
 // (adjoint of "dst <- sum a src + sum c v_occ"), starting from the adjoint
 // lambda_X = 1 of its final solution; the adjoint of each seed-vector
-// occurrence is that occurrence's weight in x_s.  The weighted sum over shifts
-// is formed by k_coef_reduce.
+// occurrence is that occurrence's weight in x_s.
+//
+// The walk is a serial chain of FP64 instructions in one warp (64 cycles each),
+// so it carries only the adjoints lambda_U of the shift directions and leaves
+// those that the weights need; k_coef_reduce forms the weights from them in
+// parallel over outer iterations, slots and shifts.  The record of the next
+// (earlier) iteration is fetched ahead.  With the weights formed in the walk it
+// took 161 us on the 16^3 x 32 workload (52 outer iterations, l = 2).
+// cs[shift][m]: slot_mr(j) = lambda_U[j+1] before sub-step j, slot_old(j, i) =
+// lambda_U[i] in sub-step j before its scaling by -beta_s.
+template <int L> struct SweepRec {
+    double2 ips, as[L], bs[L], gam[L];
+    __device__ __forceinline__ void load(const SolverDev& d, int sh, int m) {
+        const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L);
+        const double2* G = d.rec_gamma + m * (L + 1);
+        ips = __ldg(P + 5 * L);
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            as[j] = __ldg(P + 5 * j);
+            bs[j] = __ldg(P + 5 * j + 1);
+            gam[j] = __ldg(G + j + 1);
+        }
+    }
+};
 template <int L>
 __global__ void k_sweep(const SolverDev* __restrict__ ds) {
     const TraceScope trace_(FA_TK_SWEEP);
@@ -1740,72 +1846,83 @@ __global__ void k_sweep(const SolverDev* __restrict__ ds) {
     if (sh >= d.ns) return;
     constexpr int NC = nc_slots(L);
     const int Ms = d.iters[sh];
-    const double sg = d.sigma[sh];
-    dcx lX = mk(1.0);
+    const double nsg = -d.sigma[sh];
     dcx lU[L + 1];
 #pragma unroll
     for (int i = 0; i <= L; ++i) lU[i] = mk(0.0);
-    // fused multiply-adds throughout (the sweep is bound by FP64 issue in one warp)
+    SweepRec<L> next;
+    if (Ms > 0) next.load(d, sh, Ms - 1);
     for (int m = Ms - 1; m >= 0; --m) {
-        const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L);
-        const double2* G = d.rec_gamma + m * (L + 1);
-        dcx c[NC];
+        const SweepRec<L> R = next;
+        if (m > 0) next.load(d, sh, m - 1);
+        double2* out = d.cs + ((size_t)sh * d.max_outer + m) * NC;
+        // MR, reversed: u0 <- (u0 - sum gamma_j u_j)/p_s
+        const dcx t = zmul(lU[0], ld(R.ips));
 #pragma unroll
-        for (int k = 0; k < NC; ++k) c[k] = mk(0.0);
-        // MR, reversed: u0 <- (u0 - sum gamma_j u_j)/p_s, then x += sum cx_k r_k
-        {
-            const dcx t = zmul(lU[0], ld(P[5 * L]));
-#pragma unroll
-            for (int jj = 1; jj <= L; ++jj) lU[jj] = zfma(zneg(ld(G[jj])), t, lU[jj]);
-            lU[0] = t;
-#pragma unroll
-            for (int k = 0; k < L; ++k) c[slot_mr(L, k)] = zfma(lX, ld(P[5 * L + 1 + k]), c[slot_mr(L, k)]);
-        }
+        for (int jj = 1; jj <= L; ++jj) lU[jj] = zfma(zneg(ld(R.gam[jj - 1])), t, lU[jj]);
+        lU[0] = t;
 #pragma unroll
         for (int j = L - 1; j >= 0; --j) {
-            const double2* Q = P + 5 * j;
-            // x += alpha_s u_0
-            lU[0] = zfma(ld(Q[0]), lX, lU[0]);
+            // x += alpha_s u_0 with lambda_X = 1
+            lU[0] = {__dadd_rn(R.as[j].x, lU[0].r), __dadd_rn(R.as[j].y, lU[0].i)};
             // u_{j+1} <- r_old_j/(alpha_s zeta) - r_j/(alpha_s zeta_new) - sigma u_j
             const dcx lu = lU[j + 1];
-            c[slot_old(j, j)] = zfma(lu, ld(Q[3]), c[slot_old(j, j)]);
-            const int snew = (j < L - 1) ? slot_old(j + 1, j) : slot_mr(L, L - 1);
-            c[snew] = zfma(lu, zneg(ld(Q[4])), c[snew]);
-            lU[j] = zrfma(-sg, lu, lU[j]);
+            out[slot_mr(L, j)] = pk(lu);
+            lU[j] = zrfma(nsg, lu, lU[j]);
             lU[j + 1] = mk(0.0);
             // u_i <- r_old_i/zeta - beta_s u_i
-            const dcx iz = ld(Q[2]), nbs = zneg(ld(Q[1]));
+            const dcx nbs = zneg(ld(R.bs[j]));
 #pragma unroll
             for (int i = 0; i <= j; ++i) {
-                c[slot_old(j, i)] = zfma(lU[i], iz, c[slot_old(j, i)]);
+                out[slot_old(j, i)] = pk(lU[i]);
                 lU[i] = zmul(nbs, lU[i]);
             }
         }
-        double2* out = d.cs + ((size_t)sh * d.max_outer + m) * NC;
-#pragma unroll
-        for (int k = 0; k < NC; ++k) out[k] = pk(c[k]);
     }
 }
 
-// coef[m][k] = sum_s omega_s cs[s][m][k] for m < M (fixed order over s)
-__global__ void k_coef_reduce(const SolverDev* __restrict__ ds) {
+// coef[m][k] = sum_s omega_s c_s[m][k] for m < M (fixed order over s), c_s the
+// weight of occurrence k in x_s, from the adjoints that the sweep left and the
+// shift's record.  32 (m, k) per block, a warp per eighth of the shifts.
+__global__ void __launch_bounds__(256) k_coef_reduce(const SolverDev* __restrict__ ds) {
     const TraceScope trace_(FA_TK_COEF_REDUCE);
     const SolverDev& d = ds[blockIdx.y];
-    const int M = d.st->n_outer;
-    const int NC = nc_slots(d.L);
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= M * NC) return;
+    const int L = d.L, M = d.st->n_outer, NC = nc_slots(L);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int idx = blockIdx.x * 32 + lane;
+    const bool valid = idx < M * NC;
     const int m = idx / NC, k = idx - m * NC;
+    __shared__ double2 w[kMaxShifts][32];
+    // slot k: (j, i) of a sub-step, or the MR step's vector mr
+    int j = 0;
+    while (j < L && k >= (j + 1) * (j + 2) / 2) ++j;
+    const int i = k - j * (j + 1) / 2, mr = j == L ? i : -1;
+    for (int sh = warp; sh < d.ns; sh += 8) {
+        if (!valid || m >= d.iters[sh]) continue;
+        const double2* T = d.cs + ((size_t)sh * d.max_outer + m) * NC;
+        const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L);
+        dcx c;
+        if (mr >= 0) {
+            c = ld(P[5 * L + 1 + mr]);
+            if (mr == L - 1) c = zfma(ld(T[slot_mr(L, mr)]), zneg(ld(P[5 * mr + 4])), c);
+        } else if (i == j) {
+            c = zfma(ld(T[slot_mr(L, j)]), ld(P[5 * j + 3]), mk(0.0));
+            c = zfma(ld(T[k]), ld(P[5 * j + 2]), c);
+        } else {
+            c = zfma(ld(T[k]), ld(P[5 * j + 2]), mk(0.0));
+            if (i == j - 1) c = zfma(ld(T[slot_mr(L, i)]), zneg(ld(P[5 * i + 4])), c);
+        }
+        w[sh][lane] = pk(d.omega[sh] * c);
+    }
+    __syncthreads();
+    if (warp != 0 || !valid) return;
     dcx a = mk(0.0);
     for (int sh = 0; sh < d.ns; ++sh) {
         if (m >= d.iters[sh]) continue;
-        a = a + d.omega[sh] * ld(d.cs[((size_t)sh * d.max_outer + m) * NC + k]);
+        a = a + ld(w[sh][lane]);
     }
-    d.coef[(size_t)m * NC + k] = pk(a);
-    // the same weight as an FP32 pair per part (hi = FP32 rounding, lo = rest)
-    const float hr = __double2float_rn(a.r), hi = __double2float_rn(a.i);
-    d.coef4[(size_t)m * NC + k] = make_float4(hr, __double2float_rn(__dsub_rn(a.r, (double)hr)),
-                                              hi, __double2float_rn(__dsub_rn(a.i, (double)hi)));
+    // and as an FP32 pair per part (hi = FP32 rounding, lo = rest)
+    put_scalar(d.coef, d.coef4, (size_t)m * NC + k, a);
 }
 
 // single-pass result y = sum_s omega_s x_s (FP64 [12][V]) of each system
