@@ -329,7 +329,7 @@ static int apply_op(fa_ctx* c, const double* in, double* out, int dagger, int pr
             CUDA_OR(c->tmp64.ensure(b), "alloc");
             const View64 t = internal64(c->tmp64.as<double2>(), V);
             TRY(hop_f64(c, canonical64(in), t, 1.0, false, true, dg));
-            TRY(hop_f64(c, t, canonical64(out), c->scale_c, false, true, dg));
+            TRY(hop_f64(c, t, canonical64(out), c->scale_c, false, true, dg, true));
         } else {
             TRY(hop_f64(c, canonical64(in), canonical64(out), 1.0, dg, dg, dg));
         }
@@ -343,10 +343,10 @@ static int apply_op(fa_ctx* c, const double* in, double* out, int dagger, int pr
         if (is_A) {
             CUDA_OR(c->tmp32.ensure(b), "alloc");
             float4* t = c->tmp32.as<float4>();
-            TRY(hop_f32(c, a, t, nullptr, 1.0, false, true, dg));
-            TRY(hop_f32(c, t, nullptr, out, c->scale_c, false, true, dg));
+            TRY(hop_f32(c, a, t, nullptr, 1.0, false, true, dg, true));
+            TRY(hop_f32(c, t, nullptr, out, c->scale_c, false, true, dg, true));
         } else {
-            TRY(hop_f32(c, a, nullptr, out, 1.0, dg, dg, dg));
+            TRY(hop_f32(c, a, nullptr, out, 1.0, dg, dg, dg, true));
         }
     } else if (precision == FA_DF) {
         const size_t b = (size_t)12 * V * sizeof(float4);
@@ -356,10 +356,10 @@ static int apply_op(fa_ctx* c, const double* in, double* out, int dagger, int pr
         if (is_A) {
             CUDA_OR(c->tmp64.ensure(b), "alloc");
             float4* t = c->tmp64.as<float4>();
-            TRY(hop_df(c, a, t, nullptr, 1.0, false, true, dg));
-            TRY(hop_df(c, t, nullptr, out, c->scale_c, false, true, dg));
+            TRY(hop_df(c, a, t, nullptr, 1.0, false, true, dg, true));
+            TRY(hop_df(c, t, nullptr, out, c->scale_c, false, true, dg, true));
         } else {
-            TRY(hop_df(c, a, nullptr, out, 1.0, dg, dg, dg));
+            TRY(hop_df(c, a, nullptr, out, 1.0, dg, dg, dg, true));
         }
     } else {
         return FA_EINVAL;

@@ -25,6 +25,8 @@ template <bool G5IN, bool G5OUT, bool CANON, int NT, int MB>
 __global__ void __launch_bounds__(NT, MB)
 hop_kernel(Geom g, LinkView<float> U, SpinorView<float> in, SpinorView<float> out, double2* canon, float cdiag,
            float chop, float ef, float eb, float bc) {
+    dep_wait();
+    if (g.V <= kEarlySites) dep_launch();
     const int s = blockIdx.x * NT + threadIdx.x;
     cx<float> p[12];
     if (s < g.V) {
@@ -71,6 +73,8 @@ template <bool G5IN, bool G5OUT, bool CANON>
 __global__ void __launch_bounds__(kRowThreads, rows_min_blocks<false>())
 hop_rows_kernel(Geom g, LinkView<df> U, SpinorView<df> in, SpinorView<df> out, double2* canon, df cdiag, df chop, df ef,
                 df eb, df bc) {
+    dep_wait();
+    if (g.V <= kEarlySites) dep_launch();
     const int a = row_of_thread(), s = site_of_thread(blockIdx.x);
     cx<df> o[4];
     hop_site_row_sh<G5IN, G5OUT>(g, U, in, s, a, s < g.V, cdiag, chop, ef, eb, bc, o);
@@ -101,7 +105,9 @@ hop_rows_kernel(Geom g, LinkView<df> U, SpinorView<df> in, SpinorView<df> out, d
 // every 192-byte record, so direct stores would write 8 bytes per 32-byte sector).
 template <int C, bool CANON>
 __global__ void __launch_bounds__(hop64_threads<C>(), hop64_min_blocks<C>())
-hop64_kernel(Geom g, const double2* __restrict__ U, View64 in, View64 out, Op64 op, const int* done) {
+hop64_kernel(Geom g, const double2* __restrict__ U, View64 in, View64 out, Op64 op, const int* done, int early) {
+    dep_wait();
+    if (early) dep_launch();
     if (done != nullptr && *done) return;
     __shared__ Smem64<C> sm;
     const int tile = blockIdx.x / C, rank = blockIdx.x % C;
@@ -111,25 +117,28 @@ hop64_kernel(Geom g, const double2* __restrict__ U, View64 in, View64 out, Op64 
 
 template <int C>
 static int launch_hop64(const Geom& g, const double2* links, const View64& in, const View64& out, const Op64& op,
-                        const int* done, cudaStream_t st) {
+                        const int* done, cudaStream_t st, bool after) {
     const dim3 grid(tiles64(g.V) * C);
-    if (out.ks == 1) launch_ex(false, C, hop64_kernel<C, true>, grid, hop64_threads<C>(), st, g, links, in, out, op, done);
-    else launch_ex(false, C, hop64_kernel<C, false>, grid, hop64_threads<C>(), st, g, links, in, out, op, done);
+    // (the successor's blocks must find SMs of their own: they share an SM's FP64 pipe)
+    const int early = 2 * (int)grid.x <= sm_count() ? 1 : 0;
+    if (out.ks == 1) launch_ex(after, C, hop64_kernel<C, true>, grid, hop64_threads<C>(), st, g, links, in, out, op, done, early);
+    else launch_ex(after, C, hop64_kernel<C, false>, grid, hop64_threads<C>(), st, g, links, in, out, op, done, early);
     return launch_status("FP64 hop kernel");
 }
 
 int launch_hop_f64(const Geom& g, const double2* links, const View64& in, const View64& out, double diag, double ef,
-                   double eb, double t_bc, double scale, bool g5in, bool g5out, const int* done, cudaStream_t st) {
+                   double eb, double t_bc, double scale, bool g5in, bool g5out, const int* done, cudaStream_t st,
+                   bool after) {
     const Op64 op{scale * diag, -0.5 * scale, ef, eb, t_bc, g5in ? 1 : 0, g5out ? 1 : 0};
     switch (hop64_split(g.V, sm_count())) {
-        case 1: return launch_hop64<1>(g, links, in, out, op, done, st);
-        case 2: return launch_hop64<2>(g, links, in, out, op, done, st);
-        default: return launch_hop64<4>(g, links, in, out, op, done, st);
+        case 1: return launch_hop64<1>(g, links, in, out, op, done, st, after);
+        case 2: return launch_hop64<2>(g, links, in, out, op, done, st, after);
+        default: return launch_hop64<4>(g, links, in, out, op, done, st, after);
     }
 }
 
 int launch_hop_df(const Geom& g, const float4* links, const float4* in, float4* out, double* canon, double diag,
-                  double ef, double eb, double t_bc, double scale, bool g5in, bool g5out, cudaStream_t st) {
+                  double ef, double eb, double t_bc, double scale, bool g5in, bool g5out, cudaStream_t st, bool after) {
     LinkView<df> U{links, g.V};
     SpinorView<df> vin{const_cast<float4*>(in), g.V};
     SpinorView<df> vout{out, g.V};
@@ -137,30 +146,28 @@ int launch_hop_df(const Geom& g, const float4* links, const float4* in, float4* 
     const df cdiag = host_cvt<df>(scale * diag), chop = host_cvt<df>(-0.5 * scale);
     const df ref = host_cvt<df>(ef), reb = host_cvt<df>(eb), rbc = host_cvt<df>(t_bc);
     const int nb = row_blocks(g.V);
-#define FA_HOPD(A, B)                                                                                                 \
-    (canon ? hop_rows_kernel<A, B, true><<<nb, kRowThreads, 0, st>>>(g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc) \
-           : hop_rows_kernel<A, B, false><<<nb, kRowThreads, 0, st>>>(g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc))
-    if (!g5in && !g5out) FA_HOPD(false, false);
-    else if (!g5in && g5out) FA_HOPD(false, true);
-    else if (g5in && g5out) FA_HOPD(true, true);
+    auto go = [&](auto kernel) {
+        launch_ex(after, 1, kernel, dim3(nb), kRowThreads, st, g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc);
+    };
+    if (!g5in && !g5out) canon ? go(hop_rows_kernel<false, false, true>) : go(hop_rows_kernel<false, false, false>);
+    else if (!g5in && g5out) canon ? go(hop_rows_kernel<false, true, true>) : go(hop_rows_kernel<false, true, false>);
+    else if (g5in && g5out) canon ? go(hop_rows_kernel<true, true, true>) : go(hop_rows_kernel<true, true, false>);
     else return FA_EINVAL;
-#undef FA_HOPD
     return launch_status("hop kernel");
 }
 
-template <bool G5IN, bool G5OUT>
-static void launch_hop32(bool narrow, bool canon, int nb, cudaStream_t st, const Geom& g, LinkView<float> U,
-                         SpinorView<float> in, SpinorView<float> out, double2* cn, float cdiag, float chop, float ef,
-                         float eb, float bc) {
+template <bool G5IN, bool G5OUT, typename... A>
+static void launch_hop32(bool after, bool narrow, bool canon, int nb, cudaStream_t st, A... args) {
     constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks, WT = kThreads, WB = FA_HOP_MINB;
-    if (narrow && canon) hop_kernel<G5IN, G5OUT, true, NT, MB><<<nb, NT, 0, st>>>(g, U, in, out, cn, cdiag, chop, ef, eb, bc);
-    else if (narrow) hop_kernel<G5IN, G5OUT, false, NT, MB><<<nb, NT, 0, st>>>(g, U, in, out, cn, cdiag, chop, ef, eb, bc);
-    else if (canon) hop_kernel<G5IN, G5OUT, true, WT, WB><<<nb, WT, 0, st>>>(g, U, in, out, cn, cdiag, chop, ef, eb, bc);
-    else hop_kernel<G5IN, G5OUT, false, WT, WB><<<nb, WT, 0, st>>>(g, U, in, out, cn, cdiag, chop, ef, eb, bc);
+    if (narrow && canon) launch_ex(after, 1, hop_kernel<G5IN, G5OUT, true, NT, MB>, dim3(nb), NT, st, args...);
+    else if (narrow) launch_ex(after, 1, hop_kernel<G5IN, G5OUT, false, NT, MB>, dim3(nb), NT, st, args...);
+    else if (canon) launch_ex(after, 1, hop_kernel<G5IN, G5OUT, true, WT, WB>, dim3(nb), WT, st, args...);
+    else launch_ex(after, 1, hop_kernel<G5IN, G5OUT, false, WT, WB>, dim3(nb), WT, st, args...);
 }
 
 int launch_hop_f32(const Geom& g, const float4* links, const float4* in, float4* out, double* canon, double diag,
-                   double ef, double eb, double t_bc, double scale, bool g5in, bool g5out, cudaStream_t st, int shape) {
+                   double ef, double eb, double t_bc, double scale, bool g5in, bool g5out, cudaStream_t st, int shape,
+                   bool after) {
     LinkView<float> U{links, g.V};
     SpinorView<float> vin{const_cast<float4*>(in), g.V};
     SpinorView<float> vout{out, g.V};
@@ -171,11 +178,11 @@ int launch_hop_f32(const Geom& g, const float4* links, const float4* in, float4*
     const int nt = narrow ? kHopNarrowThreads : kThreads;
     const int nb = (g.V + nt - 1) / nt;
     if (!g5in && !g5out)
-        launch_hop32<false, false>(narrow, canon != nullptr, nb, st, g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc);
+        launch_hop32<false, false>(after, narrow, canon != nullptr, nb, st, g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc);
     else if (!g5in && g5out)
-        launch_hop32<false, true>(narrow, canon != nullptr, nb, st, g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc);
+        launch_hop32<false, true>(after, narrow, canon != nullptr, nb, st, g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc);
     else if (g5in && g5out)
-        launch_hop32<true, true>(narrow, canon != nullptr, nb, st, g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc);
+        launch_hop32<true, true>(after, narrow, canon != nullptr, nb, st, g, U, vin, vout, cn, cdiag, chop, ref, reb, rbc);
     else return FA_EINVAL;
     return launch_status("hop kernel");
 }
@@ -319,6 +326,7 @@ template <typename R>
 __global__ void __launch_bounds__(kThreads)
 pack_kernel(int V, const double2* __restrict__ canon, typename PackOut<R>::T* __restrict__ out) {
     __shared__ double2 rec[kPackSites][13];   // odd stride in 16-byte units: no bank conflicts across sites
+    if (V <= kEarlySites) dep_launch();
     const int s0 = blockIdx.x * kPackSites, ns = min(kPackSites, V - s0);
 #pragma unroll
     for (int r = 0; r < 12 * kPackSites / kThreads; ++r) {

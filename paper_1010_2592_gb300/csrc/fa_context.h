@@ -124,12 +124,13 @@ inline const float4* linksdf_of(const fa_ctx* c) {
     return c->links_owner ? c->links_owner->linksdf.as<float4>() : c->linksdf.as<float4>();
 }
 // operator application on internal layouts (used by the C-ABI and the solver)
-int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g5in, bool g5out, bool dagger_mu);
+int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g5in, bool g5out, bool dagger_mu,
+            bool after = false);
 // (result in `out`, or in the canonical field `canon` when that is not null)
 int hop_f32(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
-            bool dagger_mu);
+            bool dagger_mu, bool after = false);
 int hop_df(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
-           bool dagger_mu);
+           bool dagger_mu, bool after = false);
 int solve(fa_ctx* c, const double* b_canon, double* y_canon, double* const* xs_canon,
           const fa_solver_params* p, fa_solver_stats* stats);
 int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* const* y_canon,

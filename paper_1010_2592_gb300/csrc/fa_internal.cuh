@@ -47,6 +47,11 @@ struct Geom {
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Operator calls (pack, sweep, sweep): kernels of at most this many sites let
+// the next kernel of the call launch at once; it waits in dep_wait with its
+// blocks in place.  Larger ones would share their slots with waiting blocks.
+constexpr int kEarlySites = 65536;
+
 // ------------------------------------------------------------------ complex
 template <typename R> struct cx { R r, i; };
 
@@ -450,17 +455,20 @@ inline int launch_status(const char* what) {
 // Hop (one D_w sweep): out = scale * G5OUT * (diag*in' - 1/2 sum hops(in')),
 // in' = G5IN ? gamma_5 in : in, time weights from `mu_sign` * mu (the FP64
 // sweep, launch_hop_f64, is declared in hop64.cuh).
+// after: launched programmatically behind the kernel before it in the stream, which
+// must be one of this library's that calls dep_wait first (or was launched in
+// plain order); see kEarlySites.
 // The result goes to `out` (internal layout) or, when canon is not null, to the
 // canonical field `canon` (out is not written then).
 // shape: 0 narrow when the lattice fits one wave of it, 1 wide (kThreads x
 // FA_HOP_MINB per SM), 2 narrow (kHopNarrowThreads x kHopNarrowBlocks per SM)
 int launch_hop_f32(const Geom& g, const float4* links, const float4* in, float4* out, double* canon,
                    double diag, double ef, double eb, double t_bc, double scale,
-                   bool g5in, bool g5out, cudaStream_t st, int shape = 0);
+                   bool g5in, bool g5out, cudaStream_t st, int shape = 0, bool after = false);
 
 int launch_hop_df(const Geom& g, const float4* links, const float4* in, float4* out, double* canon,
                   double diag, double ef, double eb, double t_bc, double scale,
-                  bool g5in, bool g5out, cudaStream_t st);
+                  bool g5in, bool g5out, cudaStream_t st, bool after = false);
 
 // canonical (interleaved complex128 AoS) <-> internal layouts
 int launch_pack_spinor_f64(const Geom& g, const double* canon, double2* out, cudaStream_t st);

@@ -267,9 +267,11 @@ inline int hop64_split(int V, int nsm) {
 
 // out = scale g5out (diag in' - 1/2 sum hops(in')), in' = g5in ? g5 in : in, one
 // FP64 D_w sweep between fields of either layout.  A block returns at once
-// when *done is set (done may be null).
+// when *done is set (done may be null).  after: launched programmatically behind
+// the kernel before it in the stream (see launch_hop_f32).
 int launch_hop_f64(const Geom& g, const double2* links, const View64& in, const View64& out, double diag, double ef,
-                   double eb, double t_bc, double scale, bool g5in, bool g5out, const int* done, cudaStream_t st);
+                   double eb, double t_bc, double scale, bool g5in, bool g5out, const int* done, cudaStream_t st,
+                   bool after = false);
 
 // Kernel launch with programmatic stream serialization when `pdl` is set (see
 // dep_wait) and in clusters of `cluster` blocks.

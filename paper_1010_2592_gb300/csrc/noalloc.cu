@@ -85,7 +85,7 @@ extern "C" int fa_apply_A_noalloc(fa_ctx* c, const double* in, double* out, int 
                         c->stream);
     if (rc == FA_OK)
         rc = launch_hop_f64(c->g, links64_of(c), t, canonical64(out), diag, ef, eb, c->t_bc, c->scale_c, false, true,
-                            nullptr, c->stream);
+                            nullptr, c->stream, true);
     if (rc != FA_OK) return rc;   // the launch error is recorded for fa_last_error
     c->launches += 2;
     return FA_OK;

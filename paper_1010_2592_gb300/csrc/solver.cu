@@ -69,33 +69,34 @@ static void hop_timing_collect(fa_ctx* c, int m_run = 1 << 30) {
     c->hop_ev_used = 0;
 }
 
-int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g5in, bool g5out, bool dagger_mu) {
+int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g5in, bool g5out, bool dagger_mu,
+            bool after) {
     const double mu = dagger_mu ? -c->mu : c->mu;
     hop_timing_begin(c, 0);
     int rc = launch_hop_f64(c->g, links64_of(c), in, out, 4.0 + c->mass, std::exp(mu), std::exp(-mu), c->t_bc, scale,
-                            g5in, g5out, nullptr, c->stream);
+                            g5in, g5out, nullptr, c->stream, after && !c->hop_timing);
     hop_timing_end(c);
     c->launches++;
     return rc;
 }
 
 int hop_f32(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
-            bool dagger_mu) {
+            bool dagger_mu, bool after) {
     const double mu = dagger_mu ? -c->mu : c->mu;
     hop_timing_begin(c, 1);
     int rc = launch_hop_f32(c->g, links32_of(c), in, out, canon, 4.0 + c->mass, std::exp(mu), std::exp(-mu), c->t_bc,
-                            scale, g5in, g5out, c->stream, c->hop_shape);
+                            scale, g5in, g5out, c->stream, c->hop_shape, after && !c->hop_timing);
     hop_timing_end(c);
     c->launches++;
     return rc;
 }
 
 int hop_df(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
-           bool dagger_mu) {
+           bool dagger_mu, bool after) {
     const double mu = dagger_mu ? -c->mu : c->mu;
     hop_timing_begin(c, 2);
     int rc = launch_hop_df(c->g, linksdf_of(c), in, out, canon, 4.0 + c->mass, std::exp(mu), std::exp(-mu), c->t_bc,
-                           scale, g5in, g5out, c->stream);
+                           scale, g5in, g5out, c->stream, after && !c->hop_timing);
     hop_timing_end(c);
     c->launches++;
     return rc;
@@ -105,13 +106,29 @@ int hop_df(fa_ctx* c, const float4* in, float4* out, double* canon, double scale
 static int apply_A_64(fa_ctx* c, const double2* in, double2* out, double2* tmp, double scale) {
     const int V = c->g.V;
     FA_TRY(hop_f64(c, internal64(in, V), internal64(tmp, V), 1.0, false, true, false));
-    return hop_f64(c, internal64(tmp, V), internal64(out, V), scale, false, true, false);
+    return hop_f64(c, internal64(tmp, V), internal64(out, V), scale, false, true, false, true);
 }
 // ------------------------------------------------------------------ small FP64 kernels
+// |x|^2, partials of warps (the FP64 pipe bounds it: the inner product of
+// k_dot2 beside it took 19 of 25 us on 16^3 x 32)
+__global__ void __launch_bounds__(kThreads) k_norm2(int V, const double2* x, double2* part) {
+    cx<double> n[1] = {czero<double>()};
+    int s0, s1;
+    site_range(V, blockIdx.x, gridDim.x, s0, s1);
+    for (int s = s0 + threadIdx.x; s < s1; s += kThreads) {
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+            const double2 b = x[(size_t)q * V + s];
+            n[0].r = __fma_rn(b.x, b.x, n[0].r);
+            n[0].r = __fma_rn(b.y, b.y, n[0].r);
+        }
+    }
+    reduce_store<1, double>(n, part, gridDim.x, blockIdx.x);
+}
 __global__ void k_sc_invnorm(const double2* part, int nblk, double* out) {
-    __shared__ dcx red[2];
-    reduce_slots<2, false>(part, nblk, 2, red);
-    const dcx v = red[1];
+    __shared__ dcx red[1];
+    reduce_slots<1, false>(part, nblk, 1, red);
+    const dcx v = red[0];
     if (threadIdx.x == 0) {
         out[0] = 1.0 / sqrt(v.r);
         out[1] = sqrt(v.r);
@@ -1799,8 +1816,8 @@ int estimate_scale(fa_ctx* c, const double* v0, int iters, double* scale_out) {
     const int n = 12 * V, g = (n + kThreads - 1) / kThreads;
     FA_TRY(launch_pack_spinor_f64(c->g, v0, v, st));
     auto normalise = [&](double2* x) -> int {
-        k_dot2<double><<<rg, kThreads, 0, st>>>(V, x, x, c->partials.as<double2>());
-        FA_LAUNCHED(c, "k_dot2");
+        k_norm2<<<rg, kThreads, 0, st>>>(V, x, c->partials.as<double2>());
+        FA_LAUNCHED(c, "k_norm2");
         k_sc_invnorm<<<1, kScalarThreads, 0, st>>>(c->partials.as<double2>(), n_partials<double>(rg), sc);
         FA_LAUNCHED(c, "k_sc_invnorm");
         k_scale_f64<<<g, kThreads, 0, st>>>(n, x, sc);
@@ -1814,8 +1831,8 @@ int estimate_scale(fa_ctx* c, const double* v0, int iters, double* scale_out) {
         std::swap(v, w);
     }
     FA_TRY(apply_A_64(c, v, w, c->tmp64.as<double2>(), 1.0));
-    k_dot2<double><<<rg, kThreads, 0, st>>>(V, w, w, c->partials.as<double2>());
-    FA_LAUNCHED(c, "k_dot2");
+    k_norm2<<<rg, kThreads, 0, st>>>(V, w, c->partials.as<double2>());
+    FA_LAUNCHED(c, "k_norm2");
     k_sc_invnorm<<<1, kScalarThreads, 0, st>>>(c->partials.as<double2>(), n_partials<double>(rg), sc);
     FA_LAUNCHED(c, "k_sc_invnorm");
     double h[2];
