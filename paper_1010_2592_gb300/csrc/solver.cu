@@ -494,8 +494,8 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
                         launch(pdl, k_hop1_split<true>, nbh, 2 * kSplitSites, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
                                vdot, h0.part, done, ds, step);
                     else
-                        launch(pdl, k_hop1_split<false>, nbh, 2 * kSplitSites, st, h0.g, U, vin, vout, cdiag, chop, ef, eb, bc,
-                               vdot, nullptr, done, ds, none);
+                        launch(pdl, k_hop1_split<false>, nbh + (step.kind == STEP_SHIFTS ? 1 : 0), 2 * kSplitSites, st, h0.g,
+                               U, vin, vout, cdiag, chop, ef, eb, bc, vdot, nullptr, done, ds, step);
                 } else if (hop_use_narrow(c->hop_shape, V)) {
                     constexpr int NT = kHopNarrowThreads, MB = kHopNarrowBlocks;
                     const int nbh = (V + NT - 1) / NT;
@@ -618,6 +618,9 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     const int nflat = flat_blocks(ne, kFlat * ept);
     // FP64 updates take one element per thread in every launch, so that the tables of
     // a batch with a head serve them too
+    // pass 1: the shift part of sub-step j runs beside the update of r_j, or beside the
+    // sweep of r_j where that has two threads per site (k_hop1_split)
+    const bool shifts_in_sweep = rp_of<R>() == RP32 && !pass2 && n == 1 && ept == 1 && hop32_split(c->hop_shape, h0.V);
     const int4* t;
     for (int j = 0; j < L; ++j) {
         const dim3 gu = grid(flat, nflat, t);
@@ -628,8 +631,6 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
         FA_TRY(hop(0, j, 2, 0, 0, false, none));                                   // tmp = g5 D u_j
         const ScalarStep alpha{single ? STEP_ALPHA_ALL : STEP_ALPHA, j};
         FA_TRY(hop(2, 0, 0, j + 1, 1, !pass2, pass2 ? none : alpha));              // u_{j+1}
-        // pass 1 of the double-pass forms: block 0 runs the shift part of sub-step j
-        // beside the vector blocks
         if constexpr (F64) {
             if (pass2) {
                 const dim3 g = grid(flat, nflat, t);
@@ -646,13 +647,19 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
             if (ept == 1) launch(pdl, k_update_r<R, true, false, 1>, g, kFlat, st, ds, i0, j, 0, t);
             else launch(pdl, k_update_r<R, true, false, kFlatMany>, g, kFlat, st, ds, i0, j, 0, t);
         } else {
-            const dim3 g = grid(flatx, nflat + 1, t);
             const int seed_x = defer ? 0 : 1;
-            if (ept == 1) launch(pdl, k_update_r<R, false, true, 1>, g, kFlat, st, ds, i0, j, seed_x, t);
-            else launch(pdl, k_update_r<R, false, true, kFlatMany>, g, kFlat, st, ds, i0, j, seed_x, t);
+            if (shifts_in_sweep) {
+                const dim3 g = grid(flat, nflat, t);
+                launch(pdl, k_update_r<R, false, false, 1>, g, kFlat, st, ds, i0, j, seed_x, t);
+            } else {
+                const dim3 g = grid(flatx, nflat + 1, t);
+                if (ept == 1) launch(pdl, k_update_r<R, false, true, 1>, g, kFlat, st, ds, i0, j, seed_x, t);
+                else launch(pdl, k_update_r<R, false, true, kFlatMany>, g, kFlat, st, ds, i0, j, seed_x, t);
+            }
         }
         FA_LAUNCHED(c, "k_update_r");
-        FA_TRY(hop(!F64 && pass2 ? 3 : 1, j, 2, 0, 0, false, none));               // tmp = g5 D r_j
+        FA_TRY(hop(!F64 && pass2 ? 3 : 1, j, 2, 0, 0, false,                       // tmp = g5 D r_j
+                   shifts_in_sweep ? ScalarStep{STEP_SHIFTS, j} : none));
         const bool next_beta = !pass2 && j < L - 1;
         if (gram_hop && j == L - 1) {
             FA_TRY(gram_sweep());   // r_l and, in the epilogue, the Gram matrix and gamma

@@ -906,48 +906,58 @@ __device__ __noinline__ void sc_mr_seed(const SolverDev& d, int nblk, bool dry) 
     S->omega = pk(gam[L]);
 }
 
-// Shift part of the MR step: p_s = 1 - sum_j gamma_j (-sigma)^j, the weights
-// 1/p_s and c_k/(zeta p_s) with c_k = sum_{j>k} gamma_j (-sigma)^{j-1-k}, and
-// zeta <- zeta p_s, zeta' <- zeta' p_s.  The powers of -sigma are real.
-template <int L>
-__device__ __noinline__ void sc_mr_shifts(const SolverDev& d) {
+// Shift part of the MR step: p_s = 1 - sum_j gamma_j (-sigma)^j, zeta <- zeta p_s,
+// zeta' <- zeta' p_s, and the weights 1/p_s and c_k/(zeta p_s) with c_k = sum_{j>k}
+// gamma_j (-sigma)^{j-1-k}.  The powers of -sigma are real.  A thread per shift.
+// `between` runs once the new zeta are written, by every thread of the block
+// (the ticket and, if it is the last, the convergence step, which waits for
+// nothing else of this block): the weights' divisions are then off the kernel's
+// longest path.
+template <int L, typename F>
+__device__ __forceinline__ void mr_shifts(const SolverDev& d, F between) {
     DevState* S = d.st;
-    if (S->done) return;
-    const int m = S->m;
-    dcx gam[L + 1];
-#pragma unroll
-    for (int j = 0; j <= L; ++j) gam[j] = ld(d.rec_gamma[m * (L + 1) + j]);
-    for (int sh = threadIdx.x; sh < d.ns; sh += blockDim.x) {
-        if (!d.active[sh]) continue;
+    const int sh = threadIdx.x, m = S->m;
+    const bool act = !S->done && sh < d.ns && d.active[sh];
+    dcx gam[L + 1], ps = mk(1.0), zps = mk(1.0);
+    double pw[L + 1], nps = 1.0, nz = 1.0, ips, izps;
+    if (act) {
         const double ms = -d.sigma[sh];
-        double pw[L + 1];
         pw[0] = 1.0;
 #pragma unroll
-        for (int j = 1; j <= L; ++j) pw[j] = __dmul_rn(pw[j - 1], ms);
-        dcx ps = mk(1.0);
+        for (int j = 1; j <= L; ++j) {
+            gam[j] = ld(d.rec_gamma[m * (L + 1) + j]);
+            pw[j] = __dmul_rn(pw[j - 1], ms);
+        }
 #pragma unroll
         for (int j = 1; j <= L; ++j) ps = zrfma(-pw[j], gam[j], ps);
-        const dcx z = ld(d.zeta[sh]);
-        const dcx zps = zmul(z, ps);
-        const double nps = zabs2(ps);
-        double ips, izps;
-        recip2(nps, zabs2(zps), ips, izps);
-        const dcx inv_ps = zconj_scale(ips, ps);
-        const dcx inv_zps = zconj_scale(izps, zps);
-        double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * L;
-        P[0] = pk(inv_ps);
-#pragma unroll
-        for (int k = 0; k < L; ++k) {
-            dcx c = mk(0.0);
-#pragma unroll
-            for (int j = k + 1; j <= L; ++j) c = zrfma(pw[j - 1 - k], gam[j], c);
-            P[1 + k] = pk(zmul(c, inv_zps));
-        }
-        if (!(nps > 0.0) || !isfinite(ips) || !isfinite(izps) || !zfinite(ps)) fail(S, FA_ENONFINITE);
+        zps = zmul(ld(d.zeta[sh]), ps);
         d.zeta[sh] = pk(zps);
         d.zeta_p[sh] = pk(zmul(ld(d.zeta_p[sh]), ps));
+        // a failure has to be on record before the convergence step: within these
+        // bounds the divisions cannot give one
+        nps = zabs2(ps);
+        nz = zabs2(zps);
+        if (!(nps > 1e-120 && nps < 1e120 && nz > 1e-120 && nz < 1e120)) {
+            recip2(nps, nz, ips, izps);
+            if (!(nps > 0.0) || !isfinite(ips) || !isfinite(izps) || !zfinite(ps)) fail(S, FA_ENONFINITE);
+        }
+    }
+    between();
+    if (!act) return;
+    recip2(nps, nz, ips, izps);
+    const dcx inv_ps = zconj_scale(ips, ps);
+    const dcx inv_zps = zconj_scale(izps, zps);
+    double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * L;
+    P[0] = pk(inv_ps);
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        dcx c = mk(0.0);
+#pragma unroll
+        for (int j = k + 1; j <= L; ++j) c = zrfma(pw[j - 1 - k], gam[j], c);
+        P[1 + k] = pk(zmul(c, inv_zps));
     }
 }
+template <int L> __device__ __noinline__ void sc_mr_shifts(const SolverDev& d) { mr_shifts<L>(d, [] {}); }
 
 // end of an outer iteration: convergence and freezing of shifts, next beta
 template <bool DFP>
@@ -1019,7 +1029,8 @@ enum StepKind : int {
     STEP_BETA = 1,          // beta of sub-step arg
     STEP_ALPHA = 2,         // alpha of sub-step arg (seed part)
     STEP_ALPHA_ALL = 3,     // alpha of sub-step arg, seed and shift parts (single pass)
-    STEP_CONV = 4           // convergence; arg = head flag
+    STEP_CONV = 4,          // convergence; arg = head flag
+    STEP_SHIFTS = 5         // k_hop1_split without inner product: block 0 runs the shift part of sub-step arg
 };
 struct ScalarStep {
     int kind;
@@ -1225,9 +1236,10 @@ k_mr(const SolverDev* __restrict__ ds, ScalarStep step, const int4* tab) {
     const TraceScope trace_(trace_kind<R>(FA_TK_MR, true));
     const int bx = w.bx, nbx = w.nbx;
     if (bx < 0) {
-        sc_mr_shifts<L>(d);
-        __threadfence();   // the new zeta of every thread before the ticket
-        run_step<true>(d, step, nbx, w.ntk);
+        mr_shifts<L>(d, [&] {
+            __threadfence();   // the new zeta of every thread before the ticket
+            run_step<true>(d, step, nbx, w.ntk);
+        });
         return;
     }
     const int m = d.st->m, V = d.V;
@@ -1616,7 +1628,12 @@ k_hop1(Geom g, LinkView<R> U, SpinorView<R> in, SpinorView<R> out, R cdiag, R ch
     }
 }
 
-// the FP32 sweep with two threads per site (hop_site_split), 128 sites per block
+// the FP32 sweep with two threads per site (hop_site_split), 128 sites per block.
+// The sweep of r_j carries the shift part of sub-step j (STEP_SHIFTS), 4 us of FP64
+// in one warp that nothing before the next sub-step needs: beside the update of
+// r_j, which takes 1-2 us on such lattices, it was what that kernel waited for.
+// (12^3 x 24 mixed_df: 7.54 -> 7.47 ms together with mr_shifts' early ticket; the
+// ticket alone, 16^3 x 32: 14.43 -> 14.35 ms.)
 template <bool DOT>
 __global__ void __launch_bounds__(2 * kSplitSites, kSplitBlocks)
 k_hop1_split(Geom g, LinkView<float> U, SpinorView<float> in, SpinorView<float> out, float cdiag, float chop, float ef,
@@ -1625,7 +1642,15 @@ k_hop1_split(Geom g, LinkView<float> U, SpinorView<float> in, SpinorView<float> 
     dep_wait();
     if (done != nullptr && *done) return;
     const TraceScope trace_(trace_kind<float>(FA_TK_HOP1, DOT));
-    const int s = blockIdx.x * kSplitSites + (threadIdx.x & (kSplitSites - 1));
+    int bx = blockIdx.x;
+    if (!DOT && step.kind == STEP_SHIFTS) {
+        if (bx == 0) {
+            sc_alpha_shifts(ds[0], step.arg);
+            return;
+        }
+        --bx;
+    }
+    const int s = bx * kSplitSites + (threadIdx.x & (kSplitSites - 1));
     cx<float> dres[1] = {czero<float>()};
     cx<float> p[12];
     hop_site_split<false, true>(g, U, in, s, cdiag, chop, ef, eb, bc, p);

@@ -375,9 +375,10 @@ k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const in
     if (sys_idle(d, pass2)) return;
     const TraceScope trace_(trace_kind<double>(FA_TK_MR, XS));
     if (XS && w.bx < 0) {
-        sc_mr_shifts<L>(d);
-        __threadfence();   // the new zeta of every thread before the ticket
-        run_step<false>(d, step, w.nbx, w.ntk);
+        mr_shifts<L>(d, [&] {
+            __threadfence();   // the new zeta of every thread before the ticket
+            run_step<false>(d, step, w.nbx, w.ntk);
+        });
         return;
     }
     const int V = d.V, n = 12 * V, m = d.st->m;
