@@ -10,7 +10,8 @@
 // spinor with the DeGrand-Rossi projector (1 -+ g_nu), multiplies the two
 // colour vectors by the link and rebuilds the lower spin components.
 //
-// One thread per site; the nearest-neighbour reuse of spinors and links is
+// FP32: one thread per site; double-float: three, one per colour row; FP64: 32-site
+// tiles, a warp per hop (hop64.cuh).  The nearest-neighbour reuse of spinors and links is
 // left to L1/L2 (the 126 MB L2 holds several time slices of every field even
 // on 32^3 x 64).  Memory traffic floor per site and sweep: one spinor in, one
 // out, four links (FP32: 96 + 96 + 4 * 48 = 384 B).

@@ -522,13 +522,6 @@ __device__ __forceinline__ cx<R> hop_rows_body(const Geom& g, const LinkView<R>&
 #ifndef FA_HOP_MINB
 #define FA_HOP_MINB 3
 #endif
-// double-float: register budget for FA_HOP_MINB_DF resident blocks per SM.  The
-// kernel is bound by dependent FP32 instruction chains; measured on 16^3 x 32:
-// 1 block/SM (160 registers) 0.219 ms, 2 blocks/SM (128 registers, 40 B
-// spilled) 0.169 ms per sweep.
-#ifndef FA_HOP_MINB_DF
-#define FA_HOP_MINB_DF 2
-#endif
 // row-split double-float sweep: resident blocks of kRowThreads per SM.  Measured
 // per sweep (16^3 x 32 / 32^3 x 64) with the first, renormalised row split:
 // 3 blocks/SM 0.099 / 1.416 ms, 4 (80 registers) 0.099 / 1.409 ms, 5 (64
@@ -551,8 +544,5 @@ template <bool DOT> constexpr int rows_sys_min_blocks() { return DOT ? FA_HOP_RO
 #endif
 constexpr int kHopNarrowThreads = 128;
 constexpr int kHopNarrowBlocks = FA_HOP_NARROW_BLOCKS;   // 0: never narrow
-template <typename R> constexpr int hop_min_blocks() {
-    return sizeof(R) == 4 ? FA_HOP_MINB : (std::is_same<R, df>::value ? FA_HOP_MINB_DF : 1);
-}
 
 }  // namespace fa

@@ -315,8 +315,6 @@ static SolverDev make_dev(fa_ctx* c, const Layout& Lo) {
     d.store32 = nullptr;
     d.cap64 = d.cap32 = 0;
     d.m0_32 = -1;
-    d.nblk = Lo.nblk;
-    d.red_grid = Lo.red_grid;
     d.part = c->partials.as<double2>();
     d.x64 = nullptr;
     d.b64 = nullptr;
@@ -709,7 +707,11 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
         } else {
             constexpr bool D1 = rp_of<R>() == RP32 && L > 1, D0 = rp_of<R>() == RP32 && L > 2;
             const dim3 g = grid(mr_vec ? TB_VECX : TB_RGX, mg + 1, t);
-            if (defer) launch(pdl, k_mr<R, L, D1>, g, kThreads, st, ds, mr_step, t);
+            constexpr int G = mr_ahead<L>();
+            const bool ahead = (int)g.x <= 2 * sms();
+            if (ahead && defer) launch(pdl, k_mr<R, L, D1, G>, g, kThreads, st, ds, mr_step, t);
+            else if (ahead) launch(pdl, k_mr<R, L, D0, G>, g, kThreads, st, ds, mr_step, t);
+            else if (defer) launch(pdl, k_mr<R, L, D1>, g, kThreads, st, ds, mr_step, t);
             else launch(pdl, k_mr<R, L, D0>, g, kThreads, st, ds, mr_step, t);
         }
     } else if constexpr (F64) {

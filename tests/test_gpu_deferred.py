@@ -55,3 +55,24 @@ def test_double_float_head_defers(ell, mode, store):
     assert rel(to_host(r.y), y_o) < 1e-8
     r2 = ctx.apply_f(to_dev(w["b"]), reliable_every=4, **kw)
     assert rel(to_host(r2.y), y_o) < 1e-8
+
+
+@pytest.mark.parametrize("ell", [1, 2, 3, 4])
+@pytest.mark.parametrize("precision", ["mixed_df", "f32"])
+@pytest.mark.parametrize("lt", [18, 20])
+def test_mr_step_on_both_sides_of_its_grid_rule(lt, precision, ell):
+    """288 and 320 blocks of the MR step, a little below and above two per SM of a
+    152-SM part: components loaded in groups, and one at a time.  All fixed outer
+    iterations, so that both precisions stop at the same polynomial degree and differ
+    by rounding alone: 24 sub-steps at most, residuals of order 1, FP32 sums of 12 V
+    terms in blocks of 256 and a growth of a few per sub-step stay below 1e-3."""
+    dims = (16, 16, 16, lt)
+    ctx = fa.Context(dims)
+    ctx.set_gauge(to_dev(inputs.su3_exp_gauge(dims, 0.4, 731)))
+    ctx.set_params(-1.8, 0.1, -1, 0.028)
+    ctx.set_poles(*fa.neuberger_poles(6))
+    b = to_dev(inputs.gaussian_spinor(dims, 732))
+    kw = dict(ell=ell, tol=1e-30, mode="double", max_outer=3, fixed_iters=True)
+    y = to_host(ctx.apply_f(b, precision=precision, **kw).y)
+    y64 = to_host(ctx.apply_f(b, precision="f64", **kw).y)
+    assert np.all(np.isfinite(y)) and rel(y, y64) < 1e-3
