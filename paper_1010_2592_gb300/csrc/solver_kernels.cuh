@@ -415,7 +415,8 @@ __device__ __forceinline__ void acc_mr(const SolverDev& d, int m, const Ch<R> (&
 // depend on which block finished last) and runs the step.  The shift part (the
 // zeta recurrences and the per-shift scalars of every BiCG sub-step and MR
 // step) is not needed by the next seed-vector kernel: in the double-pass forms
-// it runs in an extra block 0 of that next kernel, beside its vector blocks.
+// it runs in an extra block 0 of that next kernel, beside its vector blocks, or
+// of the sweep after it (k_hop1_split, STEP_SHIFTS).
 // Single-pass solves consume the shift scalars at once and run both parts in
 // the last block.
 //
@@ -907,7 +908,8 @@ __device__ __noinline__ void sc_mr_seed(const SolverDev& d, int nblk, bool dry) 
 
 // Shift part of the MR step: p_s = 1 - sum_j gamma_j (-sigma)^j, zeta <- zeta p_s,
 // zeta' <- zeta' p_s, and the weights 1/p_s and c_k/(zeta p_s) with c_k = sum_{j>k}
-// gamma_j (-sigma)^{j-1-k}.  The powers of -sigma are real.  A thread per shift.
+// gamma_j (-sigma)^{j-1-k}.  The powers of -sigma are real.  A thread per shift
+// (kMaxShifts <= blockDim.x).
 // `between` runs once the new zeta are written, by every thread of the block
 // (the ticket and, if it is the last, the convergence step, which waits for
 // nothing else of this block): the weights' divisions are then off the kernel's
@@ -1218,7 +1220,7 @@ k_gram(const SolverDev* __restrict__ ds, const int4* tab) {
 // r_j, u_0 -= sum gamma_j u_j, the per-block partials of <rt, r_0> (slot 0) and
 // |r_0|^2 (slot 1), grid-stride, then `step` (convergence) in the last block.
 // DEFER (FP32): the deferred updates first.  Block 0 runs the shift part of the
-// MR step (sc_mr_shifts) and takes a ticket too, so that the convergence step
+// MR step (mr_shifts) and takes a ticket too, so that the convergence step
 // sees the new zeta; blocks 1.. are the vector blocks.
 // l <= 3: registers capped for 4 blocks/SM (64; some bytes spilled), so that a
 // 16^3 x 32 lattice (512 blocks) runs in one wave instead of 1.12 (left alone,
