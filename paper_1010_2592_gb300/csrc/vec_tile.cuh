@@ -354,7 +354,10 @@ k_gram_tile(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
 // MR update of a tile (FP64): warp q takes component q; then three warps form
 // <rt, r_0> (two chains) and |r_0|^2.  SHIFTS (single pass): the C blocks of a
 // cluster take the shifts rank, rank + C, ...; block 0 of the cluster
-// overwrites r_0 and u_0 once all of them hold the old r.  ACC (pass 2): y +=
+// overwrites r_0 and u_0 once all of them hold the old r.  Only block 0 takes a
+// ticket, so the convergence step may run while the others are still at their
+// shifts: whatever it writes (the active flags, the outer iteration) they read
+// before the cluster's barrier, which comes before the ticket.  ACC (pass 2): y +=
 // sum_k coef[m][slot_mr(k)] r_k.
 // Measured on GB300 (tracer, us per launch, one thread per site -> this): l = 2,
 // 8^3 x 16 28 -> 12.8 (pass 1), 30 -> 8.3 (pass 2).
@@ -390,6 +393,12 @@ k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const in
 #pragma unroll
     for (int k = 1; k <= L; ++k) ng[k] = negcx<double>(d.rec_gamma[m * (L + 1) + k]);
     double2* store = pass2 ? nullptr : store_at<double>(d, m);
+    unsigned long long live = 0ull;   // the shifts still active
+    if constexpr (SHIFTS) {
+        static_assert(kMaxShifts == 64, "one bit per shift");
+        live = __ballot_sync(0xffffffffu, lane < d.ns && d.active[lane] != 0);
+        live |= (unsigned long long)__ballot_sync(0xffffffffu, 32 + lane < d.ns && d.active[32 + lane] != 0) << 32;
+    }
     double acc = 0.0;
     // every lane makes the same number of rounds (barriers); its site may lie past the end
     const int first = ts.s - lane;
@@ -432,7 +441,7 @@ k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const in
         }
         if (SHIFTS && valid) {
             for (int sh = rank; sh < d.ns; sh += C) {
-                if (!d.active[sh]) continue;
+                if (!((live >> sh) & 1ull)) continue;
                 const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * L;
                 double2* us = d.us + (size_t)sh * (L + 1) * n + e;
                 double2* xs = d.xs + (size_t)sh * n + e;
