@@ -116,6 +116,19 @@ hop64_kernel(Geom g, const double2* __restrict__ U, View64 in, View64 out, Op64 
     if (CANON && rank == 0) store_canonical<C>(out.p, g.V, tile, sm);
 }
 
+// FP64 between internal fields, a thread per site (rule: hop64_by_site)
+template <bool G5OUT>
+__global__ void __launch_bounds__(kSite64, kSite64Blocks)
+hop64_site_kernel(Geom g, LinkView<double> U, SpinorView<double> in, SpinorView<double> out, Op64 op, const int* done) {
+    dep_wait();
+    if (done != nullptr && *done) return;
+    const int s = blockIdx.x * kSite64 + threadIdx.x;
+    if (s >= g.V) return;
+    cx<double> p[12];
+    hop_site<double, false, G5OUT>(g, U, in, s, op.cdiag, op.chop, op.ef, op.eb, op.bc, p);
+    out.store(s, p);
+}
+
 template <int C>
 static int launch_hop64(const Geom& g, const double2* links, const View64& in, const View64& out, const Op64& op,
                         const int* done, cudaStream_t st, bool after) {
@@ -131,6 +144,14 @@ int launch_hop_f64(const Geom& g, const double2* links, const View64& in, const 
                    double eb, double t_bc, double scale, bool g5in, bool g5out, const int* done, cudaStream_t st,
                    bool after) {
     const Op64 op{scale * diag, -0.5 * scale, ef, eb, t_bc, g5in ? 1 : 0, g5out ? 1 : 0};
+    const int nb = site64_blocks(g.V);
+    if (in.ss == 1 && out.ss == 1 && !g5in && hop64_by_site(nb, sm_count())) {
+        const SpinorView<double> vi{in.p, g.V}, vo{out.p, g.V};
+        const LinkView<double> U{links, g.V};
+        if (g5out) launch_ex(after, 1, hop64_site_kernel<true>, dim3(nb), kSite64, st, g, U, vi, vo, op, done);
+        else launch_ex(after, 1, hop64_site_kernel<false>, dim3(nb), kSite64, st, g, U, vi, vo, op, done);
+        return launch_status("FP64 hop kernel");
+    }
     switch (hop64_split(g.V, sm_count())) {
         case 1: return launch_hop64<1>(g, links, in, out, op, done, st, after);
         case 2: return launch_hop64<2>(g, links, in, out, op, done, st, after);

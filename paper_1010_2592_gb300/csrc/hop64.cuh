@@ -1,12 +1,13 @@
 // The FP64 Wilson-Dirac sweep, split over the eight hops of a site.
 //
-// What bounds it: GB300 issues one FP64 warp instruction per sub-partition in
-// about 64 cycles (a probe of independent FMA chains: 0.50 T thread
-// instructions/s), and a sweep takes 912 FP64 instructions per site, so its
-// floor is 234 us on 16^3 x 32 whatever the memory does (126 MB there: 19 us),
-// and one warp that walks a whole site takes 28 us even on an idle chip.  One
-// thread per site in 256-thread blocks put a 4^3 x 8 lattice on 2 of 152 SMs
-// (50-60 us per sweep) and left 3.4 waves of one block per SM on 16^3 x 32
+// What bounds it: the FP64 pipe.  A GB300 SM takes one FP64 warp instruction every 19
+// cycles while its four sub-partitions all ask (add, multiply or FMA, dependent or not:
+// 76 cycles per sub-partition, 0.53 T thread instructions/s at 2.06 GHz); a
+// sub-partition alone gets one every 64.  A sweep takes 912 FP64 instructions per
+// site, so that rate makes 227 us on 16^3 x 32 whatever the memory does (126 MB
+// there: 19 us), and one warp that walks a whole site takes 28 us even on an idle
+// chip.  One thread per site in 256-thread blocks put a 4^3 x 8 lattice on 2 of 152
+// SMs (50-60 us per sweep) and left 3.4 waves of one block per SM on 16^3 x 32
 // (270 us).
 //
 // So a tile is 32 consecutive sites and its work is spread over the warps of a
@@ -27,6 +28,8 @@
 // template parameter: eight copies of the code would be fetched cold by every
 // short launch, and the integer work hides under the FP64 pipe.
 #pragma once
+
+#include <cmath>
 
 #include "fa_internal.cuh"
 
@@ -249,7 +252,7 @@ __device__ __forceinline__ void store_canonical(double2* out, int V, int tile, c
 // 4: 512 sites 4.5 / 3.7 / 3.3, 2160 sites 4.6 / 3.7 / 3.8, 3456 sites 4.7 / 4.9 /
 // 4.4, 4096 sites 4.6 / 4.9 / 4.9, 6144 sites 6.9 / 6.3 / 6.3, 16000 sites 12.1 /
 // 11.7 / 11.7, 41472 sites 25.2 / 26.4 / 26.2; one sweep on 16^3 x 32 234 / 239 /
-// 246 us (its FP64 issue floor; one thread per site: 270).
+// 246 us.
 inline int hop64_split(int V, int nsm) {
     if (nsm < 1) nsm = 152;
     const long long t = tiles64(V);
@@ -264,6 +267,25 @@ inline int hop64_split(int V, int nsm) {
     }
     return best;
 }
+
+// A thread per site instead (hop_site in hop_device.cuh; the same bits), in blocks of
+// 128 threads at 255 registers: 912 FP64 instructions per site too, but the SM's
+// FP64 pipe takes one of its warp instructions every 17.5 cycles, of the tile form's
+// every 19.1 (a probe: 19.0 when all four sub-partitions ask at once, 16 would be its
+// best), and a wave of one block per SM (19,456 sites) takes 31.2 us however few
+// of its blocks there are, where the tile form takes 1.75 ns per site.  So it is
+// used where the last wave is full enough (the busiest SM's blocks against the
+// mean).  Measured on GB300, us per sweep, tiles / a thread per site: 32^3 x 64
+// 3649 / 3348, 16^3 x 32 230 / 219, 155,648 sites (8.0 waves) 273 / 251, 98,304 (5.05)
+// 179 / 187, 41,472 (2.1) 77 / 94, 16,384 33 / 32; with the inner product 32^3 x 64
+// 4045 / 3643.
+constexpr int kSite64 = 128, kSite64Blocks = 2;
+inline int site64_blocks(int V) { return (V + kSite64 - 1) / kSite64; }
+inline bool full_waves(double blocks, int nsm) {
+    const double x = blocks / (nsm > 0 ? nsm : 152);
+    return 0.93 * std::ceil(x) <= x;
+}
+inline bool hop64_by_site(long long blocks, int nsm) { return full_waves((double)blocks, nsm); }
 
 // out = scale g5out (diag in' - 1/2 sum hops(in')), in' = g5in ? g5 in : in, one
 // FP64 D_w sweep between fields of either layout.  A block returns at once

@@ -327,10 +327,10 @@ static SolverDev make_dev(fa_ctx* c, const Layout& Lo) {
 // TB_VEC, TB_RG: blocks of the vector and reduction grids; TB_TV, TB_TR: their
 // 32-site tiles; TB_HOP, TB_ROWS: FP64 and double-float sweeps; TB_FLAT, TB_FLAT32:
 // elementwise updates of 12 V and 6 V elements (TB_ONE, TB_ONE32: one per thread);
-// TB_FLATS: shift vectors.  X: with the system's shift block first.
+// TB_FLATS: shift vectors; TB_SITE: the FP64 sweep with a thread per site.  X: with the system's shift block first.
 enum TabKind {
     TB_VEC = 0, TB_VECX, TB_RG, TB_RGX, TB_ROWS, TB_HOP, TB_FLAT, TB_FLATX, TB_FLAT32, TB_FLAT32X, TB_FLATS, TB_ONE, TB_ONE32,
-    TB_TV, TB_TR, TB_TRX, TB_KINDS
+    TB_TV, TB_TR, TB_TRX, TB_SITE, TB_KINDS
 };
 // elements per thread of the elementwise updates: one until the launch has
 // several waves of blocks, then four (four loads in flight, a quarter of the blocks)
@@ -352,6 +352,9 @@ struct Batch {
     int tab_n[TB_KINDS] = {};             // their lengths (blocks of the launch)
     int ept64 = 1, ept32 = 1;             // elements per thread of the elementwise updates
     double sites = 0.0;                   // of all systems
+    // FP64 kernels with a thread per site (else 32-site tiles): the sweep; the Gram matrix and
+    // the MR step of a double pass; the updates and the MR step with shift vectors
+    bool site64 = false, site64_vec = false, site64_shifts = false, site64_mr_shifts = false;
     const GroupDev* groups = nullptr;     // systems sharing a gauge field (multi-RHS FP32 sweep)
     const int4* items = nullptr;          // (group, tile, first, end) per block of that sweep
     int n_items = 0;
@@ -404,6 +407,22 @@ template <typename R, int L> static bool defer_updates(const Batch& B) {
     if (L <= 1 || rp_of<R>() == RP64) return false;
     if (L > 2) return true;
     return rp_of<R>() == RP32 && B.sites >= kDeferSites;
+}
+
+// Which FP64 kernels take a thread per site: the sweep by the fill of its last wave
+// (hop64_by_site), the others by the sites per SM (vec_tile.cuh).
+static void set_forms64(Batch& B) {
+    if (!B.Lo.fp64) return;
+    long long blocks = 0;
+    int ns = 0;
+    for (int i = 0; i < B.n; ++i) {
+        blocks += site64_blocks(B.lo[i].V);
+        ns = std::max(ns, B.sys[i]->ns);
+    }
+    B.site64 = hop64_by_site(blocks, sms());
+    B.site64_vec = B.sites >= (double)kSite64Min * sms();
+    B.site64_shifts = B.site64_vec && ns <= kFewShifts;
+    B.site64_mr_shifts = B.site64_shifts && B.sites >= 3.0 * kThreads * sms() && full_waves(B.sites / kThreads, sms());
 }
 
 // ------------------------------------------------------------------ one outer iteration
@@ -482,7 +501,14 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
                                   (const double2*)nullptr, (double2*)nullptr, done, ds, none);
                 };
                 const int split = hop64_split(V, sms());
-                if (split == 1) go(std::integral_constant<int, 1>{});
+                if (B.site64) {
+                    if (dot)
+                        launch(pdl, k_hop64_site<true>, site64_blocks(V), kSite64, st, h0.g, U, vin, vout, op, vdot, h0.part,
+                               done, ds, step);
+                    else
+                        launch(pdl, k_hop64_site<false>, site64_blocks(V), kSite64, st, h0.g, U, vin, vout, op, vdot,
+                               nullptr, done, ds, none);
+                } else if (split == 1) go(std::integral_constant<int, 1>{});
                 else if (split == 2) go(std::integral_constant<int, 2>{});
                 else go(std::integral_constant<int, 4>{});
             } else {
@@ -556,7 +582,14 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
                 gh = dim3(B.tab_n[TB_HOP]);
                 th = B.tab[TB_HOP];
             }
-            if (dot) launch(pdl, k_hop64_sys<true>, gh, hop64_threads<1>(), st, ds, in_sel, in_j, out_sel, out_j, second,
+            if (B.site64) {
+                const int4* ts = nullptr;
+                const dim3 gs = grid(TB_SITE, site64_blocks(h0.V), ts);
+                if (dot) launch(pdl, k_hop64_site_sys<true>, gs, kSite64, st, ds, in_sel, in_j, out_sel, out_j, second, p2,
+                                step, ts);
+                else launch(pdl, k_hop64_site_sys<false>, gs, kSite64, st, ds, in_sel, in_j, out_sel, out_j, second, p2,
+                            none, ts);
+            } else if (dot) launch(pdl, k_hop64_sys<true>, gh, hop64_threads<1>(), st, ds, in_sel, in_j, out_sel, out_j, second,
                             p2, step, th);
             else launch(pdl, k_hop64_sys<false>, gh, hop64_threads<1>(), st, ds, in_sel, in_j, out_sel, out_j, second, p2,
                         none, th);
@@ -632,13 +665,16 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
         if constexpr (F64) {
             if (pass2) {
                 const dim3 g = grid(flat, nflat, t);
-                launch(pdl, k_update_r64<true, false, false>, g, kFlat, st, ds, j, p2, t);
+                launch(pdl, k_update_r64<true, false>, g, kFlat, st, ds, j, p2, t);
+            } else if (single && B.site64_shifts) {
+                const dim3 g = grid(TB_FLAT, flat_blocks(ne, kFlat), t);
+                launch(pdl, k_update_shifts64<kFlat>, g, kFlat, st, ds, j, t);
             } else if (single) {
                 const dim3 g = grid(TB_FLATS, flat_blocks(ne, kFlatShift), t);
-                launch(pdl, k_update_r64<false, true, false>, g, kFlat, st, ds, j, p2, t);
+                launch(pdl, k_update_shifts64<kFlatShift>, g, kFlat, st, ds, j, t);
             } else {
                 const dim3 g = grid(flatx, nflat + 1, t);
-                launch(pdl, k_update_r64<false, false, true>, g, kFlat, st, ds, j, p2, t);
+                launch(pdl, k_update_r64<false, true>, g, kFlat, st, ds, j, p2, t);
             }
         } else if (pass2) {
             const dim3 g = grid(flat, nflat, t);
@@ -669,8 +705,13 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     const ScalarStep mr_step = reliable ? none : conv;
     if (!pass2 && !gram_hop) {
         if constexpr (F64) {
-            const dim3 g = grid(gram_vec ? TB_TV : TB_TR, 8 * (gram_vec ? vg : rg), t);
-            launch(pdl, k_gram_tile<L>, g, 32 * kGramWarps, st, ds, single ? 1 : 0, t);
+            if (B.site64_vec) {
+                const dim3 g = grid(gram_vec ? TB_VEC : TB_RG, gram_vec ? vg : rg, t);
+                launch(pdl, k_gram_site<L>, g, kThreads, st, ds, single ? 1 : 0, t);
+            } else {
+                const dim3 g = grid(gram_vec ? TB_TV : TB_TR, 8 * (gram_vec ? vg : rg), t);
+                launch(pdl, k_gram_tile<L>, g, 32 * kGramWarps, st, ds, single ? 1 : 0, t);
+            }
         } else {
             if constexpr (rp_of<R>() == RPDF && L > 2) {
                 const dim3 g = grid(TB_ONE, flat_blocks(ne, kFlat), t);
@@ -702,8 +743,13 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     } else if (!single) {
         // block 0 runs the shift part of the MR step beside the vector blocks
         if constexpr (F64) {
-            const dim3 g = grid(TB_TRX, 8 * mg + 1, t);
-            launch(pdl, k_mr_tile<L, false, false, true, true, 1>, g, kMrThreads, st, ds, p2, mr_step, t);
+            if (B.site64_vec) {
+                const dim3 g = grid(TB_RGX, mg + 1, t);
+                launch(pdl, k_mr_site<L, false, true>, g, kThreads, st, ds, mr_step, t);
+            } else {
+                const dim3 g = grid(TB_TRX, 8 * mg + 1, t);
+                launch(pdl, k_mr_tile<L, false, false, true, true, 1>, g, kMrThreads, st, ds, p2, mr_step, t);
+            }
         } else {
             constexpr bool D1 = rp_of<R>() == RP32 && L > 1, D0 = rp_of<R>() == RP32 && L > 2;
             const dim3 g = grid(mr_vec ? TB_VECX : TB_RGX, mg + 1, t);
@@ -722,7 +768,10 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
             constexpr int K = decltype(split)::value;
             launch_ex(pdl, K, k_mr_tile<L, false, true, true, false, K>, g, kMrThreads, st, ds, p2, mr_step, t);
         };
-        if (C == 8) go(std::integral_constant<int, 8>{});
+        if (B.site64_mr_shifts) {
+            const dim3 gs = grid(TB_RG, rg, t);
+            launch(pdl, k_mr_site<L, true, false>, gs, kThreads, st, ds, mr_step, t);
+        } else if (C == 8) go(std::integral_constant<int, 8>{});
         else if (C == 4) go(std::integral_constant<int, 4>{});
         else if (C == 2) go(std::integral_constant<int, 2>{});
         else go(std::integral_constant<int, 1>{});
@@ -793,6 +842,8 @@ static std::vector<unsigned long long> graph_signature(const Batch& B) {
     s.push_back((unsigned long long)B.n_items);
     s.push_back((unsigned long long)B.mrhs_min_blocks);
     s.push_back((unsigned long long)(B.ept64 * 16 + B.ept32));
+    // the FP64 forms (the number of poles is in their rule)
+    s.push_back((unsigned long long)(B.site64 | B.site64_vec << 1 | B.site64_shifts << 2 | B.site64_mr_shifts << 3));
     p(c->io64a.p);
     p(c->io64b.p);
     if (B.n == 1) {
@@ -984,7 +1035,8 @@ static int build_tables(Batch& B) {
         blocks(t[TB_VECX], i, lo.vgrid, true);
         blocks(t[TB_RG], i, lo.red_grid, false);
         blocks(t[TB_RGX], i, lo.red_grid, true);
-        if (lo.fp64) blocks(t[TB_HOP], i, tiles64(lo.V), false);
+        if (lo.fp64 && !B.site64) blocks(t[TB_HOP], i, tiles64(lo.V), false);
+        if (lo.fp64 && B.site64) blocks(t[TB_SITE], i, site64_blocks(lo.V), false);
         if (lo.single) blocks(t[TB_FLATS], i, flat_blocks(12 * lo.V, kFlatShift), false);
         if (lo.need64) {
             blocks(t[TB_ROWS], i, row_blocks(lo.V), false);
@@ -1161,6 +1213,7 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
         const double many = 4.0 * 8.0 * kFlat * sms();   // elements in four waves of 8 blocks per SM
         B.ept64 = 12.0 * B.sites >= many ? kFlatMany : 1;
         B.ept32 = 6.0 * B.sites >= many ? kFlatMany : 1;
+        set_forms64(B);
     }
     // Several systems: every launch serves all of them through work tables (any
     // mix of lattice shapes); FP32 sweeps go by lattice groups (systems that

@@ -1370,6 +1370,35 @@ __device__ __forceinline__ typename Ch<R>::T* select_vec(const SolverDev& d, int
     return base + (size_t)j * vstride<R>(d);
 }
 
+// A block of the FP64 sweep with a thread per site; DOT: the site's term of <dotv, out>
+template <bool DOT>
+__device__ __forceinline__ cx<double> hop64_site_body(const Geom& g, const LinkView<double>& U,
+                                                      const SpinorView<double>& in, const SpinorView<double>& out,
+                                                      const Op64& op, const SpinorView<double>& dotv, int bx) {
+    const int s = bx * kSite64 + (int)threadIdx.x;
+    cx<double> a = czero<double>();
+    if (s < g.V) {
+        cx<double> p[12];
+        hop_site<double, false, true>(g, U, in, s, op.cdiag, op.chop, op.ef, op.eb, op.bc, p);
+        out.store(s, p);
+        if (DOT) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) a = cjfma(dotv.ld1(s, k), p[k], a);
+        }
+    }
+    return a;
+}
+// the partials of the block's 32-site tiles, as dot64_tile leaves them
+__device__ __forceinline__ void store_tile_dot(cx<double> v, double2* part, int V, int bx) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        v.r = __dadd_rn(v.r, __shfl_down_sync(0xffffffffu, v.r, o));
+        v.i = __dadd_rn(v.i, __shfl_down_sync(0xffffffffu, v.i, o));
+    }
+    const int tile = bx * (kSite64 / 32) + (int)(threadIdx.x >> 5);
+    if ((threadIdx.x & 31) == 0 && tile < tiles64(V)) part[tile] = make_double2(v.r, v.i);
+}
+
 // FP64, one system, pointers as kernel parameters: C blocks per tile (hop64.cuh)
 template <int C, bool DOT>
 __global__ void __launch_bounds__(hop64_threads<C>(), hop64_min_blocks<C>())
@@ -1409,6 +1438,43 @@ k_hop64_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel,
         const double2 v = dot64_tile<1>(internal64(d.rt64, d.V), d.V, w.bx, sm);
         if (threadIdx.x == 0) d.part[w.bx] = v;
         run_step<false>(d, step, w.nbx, w.ntk);
+    }
+}
+
+// FP64, a thread per site (launch rule: hop64_by_site), one system
+template <bool DOT>
+__global__ void __launch_bounds__(kSite64, kSite64Blocks)
+k_hop64_site(Geom g, LinkView<double> U, SpinorView<double> in, SpinorView<double> out, Op64 op,
+             SpinorView<double> dotv, double2* partials, const int* done, const SolverDev* __restrict__ ds,
+             ScalarStep step) {
+    dep_wait();
+    if (done != nullptr && *done) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_HOP1, DOT));
+    const cx<double> v = hop64_site_body<DOT>(g, U, in, out, op, dotv, blockIdx.x);
+    if (DOT) {
+        store_tile_dot(v, partials, g.V, blockIdx.x);
+        run_step<false>(ds[0], step, tiles64(g.V), gridDim.x);
+    }
+}
+// and a batch
+template <bool DOT>
+__global__ void __launch_bounds__(kSite64, kSite64Blocks)
+k_hop64_site_sys(const SolverDev* __restrict__ ds, int in_sel, int in_j, int out_sel, int out_j, int second, int pass2,
+                 ScalarStep step, const int4* tab) {
+    dep_wait();
+    const Where w = where<false>(tab);
+    const SolverDev& d = ds[w.sys];
+    if (sys_idle(d, pass2)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_HOP_SYS, DOT));
+    const double sc = second ? d.scale : 1.0;
+    const Op64 op{sc * d.diag, -0.5 * sc, d.ef, d.eb, d.bc, 0, 1};
+    const cx<double> v = hop64_site_body<DOT>(d.g, LinkView<double>{d.links64, d.V},
+                                              SpinorView<double>{select_vec<double>(d, in_sel, in_j), d.V},
+                                              SpinorView<double>{select_vec<double>(d, out_sel, out_j), d.V}, op,
+                                              SpinorView<double>{d.rt64, d.V}, w.bx);
+    if (DOT) {
+        store_tile_dot(v, d.part, d.V, w.bx);
+        run_step<false>(d, step, tiles64(d.V), w.ntk);
     }
 }
 

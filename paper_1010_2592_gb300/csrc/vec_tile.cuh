@@ -17,7 +17,7 @@
 // operations in the same order as without.
 //
 // Spread over components and chains (FP64).  On small and medium lattices the
-// FP64 kernels are bound by the FP64 pipe (64 cycles per warp instruction and
+// FP64 kernels are bound by the FP64 pipe (76 cycles per warp instruction and
 // sub-partition), not by memory: one thread per site in 256-thread blocks used
 // 2 SMs on 4^3 x 8 and 32 on 8^3 x 16.  Here
 //   * elementwise updates take one thread per 16 bytes of a vector, the shift
@@ -230,10 +230,12 @@ k_mr_acc(const SolverDev* __restrict__ ds, const int4* tab) {
 }
 
 // FP64: r_i <- r_i - alpha u_{i+1}, i = 0..j.  ACC (pass 2): y += sum_i
-// coef[m][slot_old(j,i)] r_i (before the update).  SHIFTS (single pass): the
-// block's 32 pairs of r before the update stay in shared memory, and warp w
-// updates the vectors of the shifts w, w + 8, ...
-template <bool ACC, bool SHIFTS, bool XS>
+// coef[m][slot_old(j,i)] r_i (before the update).  Bound by the FP64 pipe in pass 2 (14
+// instructions per element on average at l = 2).  Measured on GB300, 32^3 x 64, l = 2, pass 2, us per
+// launch with 1 / 4 elements per thread: 630 / 709; a loop that returns early past
+// the end, 64 registers instead of 54: 800; the next pair loaded ahead: 753.
+constexpr int kUpdateElems64 = 1;
+template <bool ACC, bool XS>
 __global__ void __launch_bounds__(kFlat)
 k_update_r64(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab) {
     dep_wait();
@@ -246,37 +248,81 @@ k_update_r64(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab
         return;
     }
     const int n = 12 * d.V, m = d.st->m, L = d.L;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int e = SHIFTS ? w.bx * kFlatShift + lane : w.bx * kFlat + (int)threadIdx.x;
-    __shared__ double2 old[SHIFTS ? kMaxEll : 1][32], now[32];
-    if (e < n && (!SHIFTS || warp == 0)) {
-        double2* store = pass2 ? nullptr : store_at<double>(d, m);
-        const double2 al = d.rec_alpha[m * L + j];
-        const cx<double> na = negcx<double>(al);
-        cx<double> t = czero<double>();
-        for (int i = 0; i <= j; ++i) {
-            double2* ri = d.r64 + (size_t)i * n + e;
-            const cx<double> a = ldc(ri), b = ldc(d.u64 + (size_t)(i + 1) * n + e);
-            if (store != nullptr) __stcs(store + (size_t)slot_old(j, i) * n + e, make_double2(a.r, a.i));
-            if (ACC) t = cfma(tocx<double>(d.coef[(size_t)m * nc_slots(L) + slot_old(j, i)]), a, t);
-            const cx<double> v = cfma(na, b, a);
-            stc(ri, v);
-            if (SHIFTS) {
-                old[i][lane] = make_double2(a.r, a.i);
-                if (i == j) now[lane] = make_double2(v.r, v.i);
+    const double2 al = d.rec_alpha[m * L + j];
+    const cx<double> na = negcx<double>(al);
+    double2* store = pass2 ? nullptr : store_at<double>(d, m);
+    constexpr int EPT = kUpdateElems64;
+    const int e0 = w.bx * (kFlat * EPT) + (int)threadIdx.x;
+    cx<double> t[EPT];
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) t[k] = czero<double>();
+    for (int i = 0; i <= j; ++i) {
+        double2* r = d.r64 + (size_t)i * n;
+        const double2* u = d.u64 + (size_t)(i + 1) * n;
+        const cx<double> cf = ACC ? tocx<double>(d.coef[(size_t)m * nc_slots(L) + slot_old(j, i)]) : czero<double>();
+        cx<double> a[EPT], b[EPT];
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+            const int e = e0 + k * kFlat;
+            if (e < n) {
+                a[k] = ldc(r + e);
+                b[k] = ldc(u + e);
             }
         }
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+            const int e = e0 + k * kFlat;
+            if (e >= n) continue;
+            if (store != nullptr) __stcs(store + (size_t)slot_old(j, i) * n + e, make_double2(a[k].r, a[k].i));
+            if (ACC) t[k] = cfma(cf, a[k], t[k]);
+            stc(r + e, cfma(na, b[k], a[k]));
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) {
+        const int e = e0 + k * kFlat;
+        if (e >= n) continue;
         if (ACC) {
             const double2 y = d.y[e];
-            d.y[e] = make_double2(__dadd_rn(y.x, t.r), __dadd_rn(y.y, t.i));
+            d.y[e] = make_double2(__dadd_rn(y.x, t[k].r), __dadd_rn(y.y, t[k].i));
         }
         if (d.x64 != nullptr) acc_x1(d.x64 + e, al, ldc(d.u64 + e));
     }
-    if (!SHIFTS) return;
-    __syncthreads();
+}
+
+// The same with shift vectors (single pass), W pairs per block.  W = 32: warp 0
+// updates r, and warp w the vectors of the shifts w, w + 8, ...  W = 256: a thread
+// takes a pair through all shifts (rule: k_update_shifts64's launch).  The r before
+// the update stay in shared memory.
+template <int W>
+__global__ void __launch_bounds__(kFlat)
+k_update_shifts64(const SolverDev* __restrict__ ds, int j, const int4* tab) {
+    dep_wait();
+    const Where w = where<false>(tab);
+    const SolverDev& d = ds[w.sys];
+    if (sys_idle(d, 0)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_UPDATE_R));
+    const int n = 12 * d.V, m = d.st->m, L = d.L;
+    const int lane = threadIdx.x % W, part = threadIdx.x / W;
+    const int e = w.bx * W + lane;
+    __shared__ double2 old[kMaxEll][W], now[W];
+    if (e < n && part == 0) {
+        const double2 al = d.rec_alpha[m * L + j];
+        const cx<double> na = negcx<double>(al);
+        for (int i = 0; i <= j; ++i) {
+            double2* ri = d.r64 + (size_t)i * n + e;
+            const cx<double> a = ldc(ri), b = ldc(d.u64 + (size_t)(i + 1) * n + e);
+            const cx<double> v = cfma(na, b, a);
+            stc(ri, v);
+            old[i][lane] = make_double2(a.r, a.i);
+            if (i == j) now[lane] = make_double2(v.r, v.i);
+        }
+        if (d.x64 != nullptr) acc_x1(d.x64 + e, al, ldc(d.u64 + e));
+    }
+    if (W < kFlat) __syncthreads();
     if (e >= n) return;
     const cx<double> rj = ldc(&old[j][lane]), rn = ldc(&now[lane]);
-    for (int sh = warp; sh < d.ns; sh += kFlat / 32) {
+    for (int sh = part; sh < d.ns; sh += kFlat / W) {
         if (!d.active[sh]) continue;
         const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * j;
         const cx<double> as = tocx<double>(P[0]), bs = negcx<double>(P[1]), iz = tocx<double>(P[2]);
@@ -481,6 +527,142 @@ k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const in
         }
         run_step<false>(d, step, w.nbx, w.ntk);
     }
+}
+
+// ------------------------------------------------------------------ FP64, a thread per site
+// From kSite64Min sites per SM on (a wave and a quarter of 256-thread blocks) there is
+// FP64 work for every SM without a split by component and chain, and the tile
+// kernels lose to their barriers, to products formed from vectors loaded once per
+// chain, and to the few blocks that 148 registers x 384 threads leave.  The same
+// chains in the same order: the same bits.  Measured on GB300 (tracer, us per launch,
+// l = 2, tiles / a thread per site): Gram matrix 32^3 x 64 1522 / 776, 16^3 x 32 196 /
+// 92, 41,472 sites 69 / 50, 16,384 32 / 29; MR step of a double pass 1851 / 1136,
+// 158 / 101, 55 / 53, 24 / 29; k_update_shifts64 with 8 shifts (W = 32 / 256) 10444 /
+// 9183, 628 / 585, 198 / 187, 78 / 87.  At l = 8 and 41,472 sites they draw (507 / 511,
+// 119 / 126).  With many shifts a warp per shift is even or better (16^3 x 32, 24
+// shifts: 1661 / 1692), as is the tile form of the single-pass MR step (1386 / 1627),
+// whose site form takes whole waves of one block per SM (8 shifts: 155,648 sites, 4.0
+// waves, 660 / 616; 196,608, 5.05, 832 / 892; 32^3 x 64 8568 / 7940).
+constexpr int kSite64Min = 320;
+constexpr int kFewShifts = 16;
+
+// the Gram matrix
+template <int L>
+__global__ void __launch_bounds__(kThreads, L <= 2 ? 4 : 1)
+k_gram_site(const SolverDev* __restrict__ ds, int shifts, const int4* tab) {
+    dep_wait();
+    const Where w = where<false>(tab);
+    const SolverDev& d = ds[w.sys];
+    if (sys_idle(d, 0)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_GRAM));
+    constexpr int NG = n_gram(L);
+    const int V = d.V, n = 12 * V;
+    cx<double> acc[NG];
+#pragma unroll
+    for (int k = 0; k < NG; ++k) acc[k] = czero<double>();
+    int s0, s1;
+    site_range(V, w.bx, w.nbx, s0, s1);
+    for (int s = s0 + threadIdx.x; s < s1; s += kThreads) {
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+            cx<double> v[L + 1];
+#pragma unroll
+            for (int i = 0; i <= L; ++i) v[i] = ldc(d.r64 + (size_t)i * n + (size_t)q * V + s);
+            int g = 0;
+#pragma unroll
+            for (int i = 0; i <= L; ++i)
+#pragma unroll
+                for (int k = i; k <= L; ++k, ++g) {
+                    if (L <= 2 && i == k) {
+                        acc[g].r = __fma_rn(v[i].r, v[i].r, acc[g].r);
+                        acc[g].r = __fma_rn(v[i].i, v[i].i, acc[g].r);
+                    } else {
+                        acc[g] = cjfma(v[i], v[k], acc[g]);
+                    }
+                }
+        }
+    }
+    reduce_store<NG, double>(acc, d.part, w.nbx, w.bx);
+    if (last_block(d.st, w.ntk) == LB_LAST) {
+        sc_mr_seed<L, false>(d, n_partials<double>(w.nbx), false);
+        if (shifts) {
+            __syncthreads();
+            sc_mr_shifts<L>(d);
+        }
+    }
+}
+
+// the MR update of pass 1
+template <int L, bool SHIFTS, bool XS>
+__global__ void __launch_bounds__(kThreads)
+k_mr_site(const SolverDev* __restrict__ ds, ScalarStep step, const int4* tab) {
+    dep_wait();
+    const Where w = where<XS>(tab);
+    const SolverDev& d = ds[w.sys];
+    if (sys_idle(d, 0)) return;
+    const TraceScope trace_(trace_kind<double>(FA_TK_MR, XS));
+    if (XS && w.bx < 0) {
+        mr_shifts<L>(d, [&] {
+            __threadfence();   // the new zeta of every thread before the ticket
+            run_step<false>(d, step, n_partials<double>(w.nbx), w.ntk);
+        });
+        return;
+    }
+    const int V = d.V, n = 12 * V, m = d.st->m;
+    cx<double> ng[L + 1];
+    ng[0] = czero<double>();
+#pragma unroll
+    for (int k = 1; k <= L; ++k) ng[k] = negcx<double>(d.rec_gamma[m * (L + 1) + k]);
+    double2* store = store_at<double>(d, m);
+    cx<double> dots[2] = {czero<double>(), czero<double>()};
+    int s0, s1;
+    site_range(V, w.bx, w.nbx, s0, s1);
+    for (int s = s0 + threadIdx.x; s < s1; s += kThreads) {
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+            const size_t e = (size_t)q * V + s;
+            cx<double> rv[L + 1];
+#pragma unroll
+            for (int i = 0; i <= L; ++i) rv[i] = ldc(d.r64 + (size_t)i * n + e);
+            if (store != nullptr) {
+#pragma unroll
+                for (int k = 0; k < L; ++k) __stcs(store + (size_t)slot_mr(L, k) * n + e, make_double2(rv[k].r, rv[k].i));
+            }
+            if (SHIFTS) {
+                for (int sh = 0; sh < d.ns; ++sh) {
+                    if (!d.active[sh]) continue;
+                    const double2* P = d.prec + ((size_t)sh * d.max_outer + m) * ps_stride(L) + 5 * L;
+                    double2* us = d.us + (size_t)sh * (L + 1) * n + e;
+                    double2* xs = d.xs + (size_t)sh * n + e;
+                    cx<double> xv = ldc(xs), u0 = ldc(us);
+#pragma unroll
+                    for (int k = 0; k < L; ++k) xv = cfma(tocx<double>(P[1 + k]), rv[k], xv);
+#pragma unroll
+                    for (int k = 1; k <= L; ++k) u0 = cfma(ng[k], ldc(us + (size_t)k * n), u0);
+                    stc(xs, xv);
+                    stc(us, cmul(tocx<double>(P[0]), u0));
+                }
+            }
+            if (d.x64 != nullptr) {
+#pragma unroll
+                for (int k = 1; k <= L; ++k) acc_x1(d.x64 + e, d.rec_gamma[m * (L + 1) + k], rv[k - 1]);
+            }
+            cx<double> r0 = rv[0], u0 = ldc(d.u64 + e);
+#pragma unroll
+            for (int k = 1; k <= L; ++k) {
+                r0 = cfma(ng[k], rv[k], r0);
+                u0 = cfma(ng[k], ldc(d.u64 + (size_t)k * n + e), u0);
+            }
+            stc(d.r64 + e, r0);
+            stc(d.u64 + e, u0);
+            const cx<double> t = ldc(d.rt64 + e);
+            dots[0] = cjfma(t, r0, dots[0]);
+            dots[1].r = __fma_rn(r0.r, r0.r, dots[1].r);
+            dots[1].r = __fma_rn(r0.i, r0.i, dots[1].r);
+        }
+    }
+    reduce_store<2, double>(dots, d.part, w.nbx, w.bx);
+    run_step<false>(d, step, n_partials<double>(w.nbx), w.ntk);
 }
 
 }  // namespace fa
