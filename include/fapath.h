@@ -54,7 +54,9 @@ typedef enum {
 } fa_status;
 
 /* FA_SINGLE: shift vectors updated alongside the seed (Sec. 3 "1-pass").
- * FA_DOUBLE: Sec. 2 option 1, pass 2 regenerates the seed vectors.
+ * FA_DOUBLE: Sec. 2 option 1, pass 2 regenerates the seed vectors.  Pass 2 takes
+ *            no memory that pass 1 does not hold; with FA_F32 and l > 2 a solve
+ *            holds l - 2 spinors (l - 1 with reliable updates) besides its 2 l + 4.
  * FA_PSEUDO: Sec. 2 option 2, pass 1 stores the seed-vector occurrences of as
  *            many outer iterations as store_gb allows (a contiguous prefix);
  *            the rest, if any, is regenerated by a pass 2 from a snapshot. */

@@ -521,7 +521,7 @@ int fa_device_bytes(const fa_ctx* c, unsigned long long* field_bytes, unsigned l
     // lattice-sized buffers: links, spinors, stores, staging, reduction partials
     const fa::DevBuf* field[] = {&c->links64, &c->links32, &c->linksdf, &c->io64a, &c->io64b, &c->io32a,
                                  &c->io32b, &c->tmp64, &c->tmp32, &c->partials, &c->r64, &c->u64, &c->rt64,
-                                 &c->r32, &c->u32, &c->rt32, &c->rb64, &c->rb32, &c->y64, &c->xs64, &c->us64, &c->bhost_dev,
+                                 &c->ru32, &c->rt32, &c->y64, &c->xs64, &c->us64, &c->bhost_dev,
                                  &c->yhost_dev, &c->gx, &c->gpart, &c->store64, &c->store32, &c->snap64,
                                  &c->snap32, &c->xrel, &c->brel, &c->snapx, &c->defl, &c->eig};
     // scalars: solver state, shifts, records, pass-2 weights, batch descriptors

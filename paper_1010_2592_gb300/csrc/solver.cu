@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(kThreads) k_lincomb_canon(int n, int k, const 
 struct Layout {
     int L, ns, max_outer, V;
     bool need64, need32, single;
+    bool pseudo, reliable;     // FA_PSEUDO; reliable updates
     bool fp64;                 // FP64 outer iterations (the whole solve or its head)
     bool gram_hop;             // FP32 pass 1: the Gram matrix in the last sweep's epilogue (one system, l <= 4)
     size_t vs64, vs32;         // one spinor in elements of double2 / float4
@@ -213,6 +214,26 @@ static int sms() {
     return n > 0 ? n : 152;
 }
 static int red_grid_for(int V) { return std::min(nblocks(V), 8 * sms()); }
+
+// Where pass 2 keeps rb_0..rb_{l-2} (solver_kernels.cuh), so that a solve holds
+// no more than its pass 1 does and takes nothing after it: the double-float
+// head in the FP32 vectors, which the switch fills later (2 (l + 1) FP32 spinors
+// hold l + 1 wide ones); an FP32 tail in the head's r vectors; an FP32 solve of
+// its own in the snapshot, once restored, or, with option 1, from the shadow
+// vector on, which only a reliable update reads in pass 2.  The last two need
+// room past it: FP32 option 1 holds l - 2 more spinors for l > 2 (l - 1 with
+// reliable updates).
+static size_t rt32_spinors(const Layout& Lo) {
+    if (Lo.need64 || Lo.single || Lo.pseudo) return 1;
+    return std::max(1, Lo.L - 1 + (Lo.reliable ? 1 : 0));
+}
+static size_t snap32_spinors(const Layout& Lo) { return Lo.need64 ? 3 : std::max(3, Lo.L - 1); }
+static void place_rb(const fa_ctx* c, const Layout& Lo, SolverDev& d) {
+    d.rb64 = Lo.need64 && Lo.need32 ? c->ru32.as<double2>() : nullptr;
+    d.rb32 = Lo.need64 ? c->r64.as<float4>()
+           : Lo.pseudo ? c->snap32.as<float4>()
+                       : c->rt32.as<float4>() + (Lo.reliable ? Lo.vs32 : 0);
+}
 
 static int ensure_workspace(fa_ctx* c, const Layout& Lo) {
     const int V = Lo.V, L = Lo.L, ns = c->ns, MO = Lo.max_outer;
@@ -240,14 +261,17 @@ static int ensure_workspace(fa_ctx* c, const Layout& Lo) {
         FA_CUDA(c->tmp64.ensure(s64), "alloc tmp64");
     }
     if (Lo.need32) {
-        FA_CUDA(c->r32.ensure((L + 1) * s32), "alloc r32");
-        FA_CUDA(c->u32.ensure((L + 1) * s32), "alloc u32");
-        FA_CUDA(c->rt32.ensure(s32), "alloc rt32");
+        FA_CUDA(c->ru32.ensure(2 * (L + 1) * s32), "alloc r32, u32");
+        FA_CUDA(c->rt32.ensure(rt32_spinors(Lo) * s32), "alloc rt32");
         FA_CUDA(c->tmp32.ensure(s32), "alloc tmp32");
     }
     if (Lo.single) {
         FA_CUDA(c->xs64.ensure((size_t)ns * s64), "alloc shift solutions");
         FA_CUDA(c->us64.ensure((size_t)ns * (L + 1) * s64), "alloc shift directions");
+    }
+    if (Lo.pseudo) {   // (before the stores take their share of the free memory)
+        if (Lo.need64) FA_CUDA(c->snap64.ensure(3 * s64), "alloc snapshot");
+        if (Lo.need32) FA_CUDA(c->snap32.ensure(snap32_spinors(Lo) * s32), "alloc snapshot");
     }
     if (!c->pinned) {
         FA_CUDA(cudaMallocHost(&c->pinned, 4096), "alloc pinned");
@@ -302,12 +326,11 @@ static SolverDev make_dev(fa_ctx* c, const Layout& Lo) {
     d.u64 = c->u64.as<double2>();
     d.rt64 = c->rt64.as<double2>();
     d.tmp64 = c->tmp64.as<double2>();
-    d.r32 = c->r32.as<float4>();
-    d.u32 = c->u32.as<float4>();
+    d.r32 = c->ru32.as<float4>();
+    d.u32 = d.r32 + (size_t)(Lo.L + 1) * Lo.vs32;
     d.rt32 = c->rt32.as<float4>();
     d.tmp32 = c->tmp32.as<float4>();
-    d.rb64 = c->rb64.as<double2>();
-    d.rb32 = c->rb32.as<float4>();
+    place_rb(c, Lo, d);
     d.y = c->y64.as<double2>();
     d.xs = Lo.single ? c->xs64.as<double2>() : nullptr;
     d.us = Lo.single ? c->us64.as<double2>() : nullptr;
@@ -460,6 +483,7 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     const SolverDev& h0 = B.host[0];
     auto vsel = [&](int sel, int j) -> T* {
         constexpr bool wide = rp_of<R>() != RP32;   // FP64 and double-float use the wide buffers
+        if (sel == 3 && j == L - 1) sel = 1, j = L;   // rb_at
         T* base = wide ? (T*)(sel == 0 ? (void*)h0.u64 : sel == 1 ? (void*)h0.r64 : sel == 2 ? (void*)h0.tmp64 : (void*)h0.rb64)
                        : (T*)(sel == 0 ? (void*)h0.u32 : sel == 1 ? (void*)h0.r32 : sel == 2 ? (void*)h0.tmp32 : (void*)h0.rb32);
         return base + (size_t)j * (size_t)Ch<R>::N * h0.V;
@@ -937,10 +961,10 @@ static int load_source(Batch& B, int i, const double* b, int rp) {
                 "copy rt");
         FA_CUDA(cudaMemsetAsync(c->u64.p, 0, (size_t)12 * V * sizeof(double2), st), "zero u");
     } else {
-        FA_TRY(launch_pack_spinor_f32(c->g, b, c->r32.as<float4>(), st));
-        FA_CUDA(cudaMemcpyAsync(c->rt32.p, c->r32.p, (size_t)6 * V * sizeof(float4), cudaMemcpyDeviceToDevice, st),
-                "copy rt");
-        FA_CUDA(cudaMemsetAsync(c->u32.p, 0, (size_t)6 * V * sizeof(float4), st), "zero u");
+        const SolverDev& d = B.host[i];
+        FA_TRY(launch_pack_spinor_f32(c->g, b, d.r32, st));
+        FA_CUDA(cudaMemcpyAsync(d.rt32, d.r32, (size_t)6 * V * sizeof(float4), cudaMemcpyDeviceToDevice, st), "copy rt");
+        FA_CUDA(cudaMemsetAsync(d.u32, 0, (size_t)6 * V * sizeof(float4), st), "zero u");
     }
     B.c0->launches += 1;
     return FA_OK;
@@ -952,10 +976,10 @@ static int switch_to_f32(Batch& B, int i, int from) {
     fa_ctx* c = B.sys[i];
     cudaStream_t st = B.c0->stream;
     DevBuf* src[3] = {&c->r64, &c->u64, &c->rt64};
-    DevBuf* dst[3] = {&c->r32, &c->u32, &c->rt32};
+    float4* dst[3] = {B.host[i].r32, B.host[i].u32, B.host[i].rt32};
     for (int k = 0; k < 3; ++k) {
-        if (from == RPDF) FA_TRY(launch_convert_df_to_f32(c->g, src[k]->as<float4>(), dst[k]->as<float4>(), st));
-        else FA_TRY(launch_convert_f64_to_f32(c->g, src[k]->as<double2>(), dst[k]->as<float4>(), st));
+        if (from == RPDF) FA_TRY(launch_convert_df_to_f32(c->g, src[k]->as<float4>(), dst[k], st));
+        else FA_TRY(launch_convert_f64_to_f32(c->g, src[k]->as<double2>(), dst[k], st));
     }
     B.c0->launches += 3;
     return FA_OK;
@@ -966,7 +990,8 @@ static int snapshot(Batch& B, int i, bool f64, bool restore) {
     fa_ctx* c = B.sys[i];
     const size_t sb = f64 ? B.lo[i].vs64 * sizeof(double2) : B.lo[i].vs32 * sizeof(float4);
     char* snap = f64 ? c->snap64.as<char>() : c->snap32.as<char>();
-    void* v[3] = {f64 ? c->r64.p : c->r32.p, f64 ? c->u64.p : c->u32.p, f64 ? c->rt64.p : c->rt32.p};
+    const SolverDev& d = B.host[i];
+    void* v[3] = {f64 ? (void*)d.r64 : (void*)d.r32, f64 ? (void*)d.u64 : (void*)d.u32, f64 ? (void*)d.rt64 : (void*)d.rt32};
     for (int k = 0; k < 3; ++k) {
         void* dst = restore ? v[k] : (void*)(snap + k * sb);
         const void* src = restore ? (const void*)(snap + k * sb) : v[k];
@@ -1169,6 +1194,8 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
         Lo.max_outer = p->max_outer;
         Lo.V = c->g.V;
         Lo.single = single;
+        Lo.pseudo = pseudo;
+        Lo.reliable = rel_every > 0;
         Lo.need64 = prec != FA_F32;
         Lo.fp64 = prec == FA_F64 || prec == FA_MIXED;
         Lo.need32 = prec != FA_F64;
@@ -1265,8 +1292,6 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
             const size_t s64i = B.lo[i].vs64 * sizeof(double2), s32i = B.lo[i].vs32 * sizeof(float4);
             if (cap64 > 0) FA_CUDA(c->store64.ensure((size_t)cap64 * NC * s64i), "alloc occurrence store");
             if (cap32 > 0) FA_CUDA(c->store32.ensure((size_t)cap32 * NC * s32i), "alloc occurrence store");
-            if (Lo.need64) FA_CUDA(c->snap64.ensure(3 * s64i), "alloc snapshot");
-            if (Lo.need32) FA_CUDA(c->snap32.ensure(3 * s32i), "alloc snapshot");
             B.host[i].store64 = c->store64.as<char>();
             B.host[i].store32 = c->store32.as<char>();
             B.host[i].cap64 = (int)cap64;
@@ -1455,15 +1480,6 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
         }
         const int mstart = Kst;
         if (mstart < M) {
-            // the updated r_j of a sub-step (FP32 and double-float iterations of pass 2)
-            for (int i = 0; i < n && prec != FA_F64; ++i) {
-                fa_ctx* c = B.sys[i];
-                if (prec == FA_MIXED_DF) FA_CUDA(c->rb64.ensure(L * B.lo[i].vs64 * sizeof(double2)), "alloc rb64");
-                FA_CUDA(c->rb32.ensure(L * B.lo[i].vs32 * sizeof(float4)), "alloc rb32");
-                B.host[i].rb64 = c->rb64.as<double2>();
-                B.host[i].rb32 = c->rb32.as<float4>();
-            }
-            if (prec != FA_F64) FA_TRY(upload(B));
             int p2 = prec == FA_F64 ? RP64
                    : (prec == FA_F32 ? RP32 : ((switch_outer < 0 || mstart < switch_outer) ? head_rp : RP32));
             for (int i = 0; i < n; ++i) {
@@ -1591,7 +1607,7 @@ int autotune_batch(fa_ctx* const* ctxs, int n, int reps, int* rpb_out, int* mb_o
     for (int i = 0; i < n; ++i) {
         B.host.push_back(make_dev(ctxs[i], B.lo[i]));
         FA_CUDA(cudaMemsetAsync(B.host[i].st, 0, sizeof(DevState), st), "clear state");
-        FA_CUDA(cudaMemsetAsync(ctxs[i]->r32.p, 0, B.lo[i].vs32 * sizeof(float4), st), "clear r");
+        FA_CUDA(cudaMemsetAsync(ctxs[i]->ru32.p, 0, B.lo[i].vs32 * sizeof(float4), st), "clear r");
     }
     FA_TRY(upload(B));
     const int rpbs[] = {1, 2, 3, 4, 6, 12, kMaxRhs};

@@ -88,8 +88,9 @@ struct SolverDev {
     // seed vectors: r_0..r_l and u_0..u_l contiguous, the shadow vector, scratch
     double2 *r64, *u64, *rt64, *tmp64;
     float4 *r32, *u32, *rt32, *tmp32;
-    // pass 2, FP32 and double-float: r_j after sub-step j's update (l vectors; r_j itself keeps
-    // the value before it for the MR step)
+    // pass 2, FP32 and double-float: r_j after sub-step j's update, j < l - 1 (r_j itself
+    // keeps the value before it for the MR step; the last one goes to r_l, which the
+    // sub-step's second hop overwrites).  In memory that pass 2 does not use: place_rb
     double2* rb64;
     float4* rb32;
     double2* y;            // FP64 [12][V] result
@@ -230,6 +231,10 @@ template <> struct Ch<float> {
 
 template <typename R> __device__ __forceinline__ size_t vstride(const SolverDev& d) {
     return (size_t)Ch<R>::N * d.V;
+}
+// pass 2: r_j after its own update
+template <typename R> __device__ __forceinline__ typename Ch<R>::T* rb_at(const SolverDev& d, int j) {
+    return j == d.L - 1 ? Vec<R>::r(d) + (size_t)d.L * vstride<R>(d) : Vec<R>::rb(d) + (size_t)j * vstride<R>(d);
 }
 
 // store slots of outer iteration m, or nullptr when m is not stored
@@ -387,7 +392,7 @@ __device__ __forceinline__ void deferred_acc(const SolverDev& d, int m, const St
         for (int i = 0; i < j; ++i) defer_r(sc.na[j], r, u, i);
         // r_j after its own update: rb_j, formed again where u_{j+1} is still what the sweep left
         if (j == L - 1) defer_r(sc.na[j], r, u, j);
-        else r[j] = Ch<R>::ld(Vec<R>::rb(d) + j * vs, q, d.V, s);
+        else r[j] = Ch<R>::ld(rb_at<R>(d, j), q, d.V, s);
     }
 }
 // the MR step's occurrences r_0..r_{L-1}
@@ -1366,7 +1371,8 @@ k_dot2_sys(const SolverDev* __restrict__ ds, double tol, double theta, const int
 // partials of <rt, out> into the system's partial buffer.
 template <typename R>
 __device__ __forceinline__ typename Ch<R>::T* select_vec(const SolverDev& d, int sel, int j) {
-    typename Ch<R>::T* base = sel == 0 ? Vec<R>::u(d) : sel == 1 ? Vec<R>::r(d) : sel == 2 ? Vec<R>::tmp(d) : Vec<R>::rb(d);
+    if (sel == 3) return rb_at<R>(d, j);
+    typename Ch<R>::T* base = sel == 0 ? Vec<R>::u(d) : sel == 1 ? Vec<R>::r(d) : Vec<R>::tmp(d);
     return base + (size_t)j * vstride<R>(d);
 }
 

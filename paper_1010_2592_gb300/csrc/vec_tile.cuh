@@ -11,8 +11,8 @@
 // kernel before the Gram matrix (k_deferred).  Each vector is then read and
 // written once per outer iteration instead of once per sub-step: per site 2 l
 // instead of l (l + 1) updates of 3 spinors.  Where it is done: defer_updates
-// in solver.cu.  In pass 2 (always) the updated r_j goes to a vector of its own
-// (rb_j), so that the MR step still has every occurrence of the weighted sum and
+// in solver.cu.  In pass 2 (always) the updated r_j goes to another vector
+// (rb_j, rb_at), so that the MR step still has every occurrence of the weighted sum and
 // adds to y once instead of l + 1 times.  Every number is formed by the same
 // operations in the same order as without.
 //
@@ -129,7 +129,7 @@ k_update_r(const SolverDev* __restrict__ ds, int i0, int j, int seed_x, const in
     for (int i = i0; i <= j; ++i) {
         T* r = Vec<R>::r(d) + (size_t)i * n;
         const T* u = Vec<R>::u(d) + (size_t)(i + 1) * n;
-        T* out = PASS2 ? Vec<R>::rb(d) + (size_t)i * n : r;
+        T* out = PASS2 ? rb_at<R>(d, i) : r;
         Ch<R> a[EPT], b[EPT];
 #pragma unroll
         for (int k = 0; k < EPT; ++k) {
