@@ -412,7 +412,10 @@ int fa_trace_stop(fa_trace_record* records, long long capacity, long long* n, lo
  * thread-block size and residency for the stencil kernel).
  *   FA_SHAPE_WIDE    256-thread blocks, 3 per SM (80 registers)
  *   FA_SHAPE_NARROW  128-thread blocks, 7 per SM (72 registers)
- *   FA_SHAPE_AUTO    narrow when the lattice fits one wave of it (the default) */
+ *   FA_SHAPE_AUTO    narrow when the lattice fits one wave of it (the default)
+ * One-system solves on lattices of up to three 128-site blocks per SM run the sweep
+ * with two threads per site (256-thread blocks of 128 sites, 3 per SM) unless the
+ * shape is WIDE; fa_apply_dw and fa_apply_A take the shapes as listed. */
 typedef enum { FA_SHAPE_AUTO = 0, FA_SHAPE_WIDE = 1, FA_SHAPE_NARROW = 2 } fa_hop_shape;
 
 /* Set / read the FP32 sweep launch shape of ctx; it applies to fa_apply_dw,
@@ -422,8 +425,8 @@ typedef enum { FA_SHAPE_AUTO = 0, FA_SHAPE_WIDE = 1, FA_SHAPE_NARROW = 2 } fa_ho
 int fa_set_hop_shape(fa_ctx* ctx, int shape);
 int fa_get_hop_shape(const fa_ctx* ctx);
 
-/* Autotuner: time every FP32 sweep launch shape on ctx's lattice (chains of
- * `reps` sweeps, each reading the previous one's output, on scratch spinors
+/* Autotuner: time every FP32 sweep launch shape on ctx's lattice, as a one-system
+ * solve with that shape runs it (chains of `reps` sweeps, each reading the previous one's output, on scratch spinors
  * owned by ctx, between CUDA events on ctx's stream; replayed from a CUDA graph,
  * as the solver replays its outer iterations, unless ctx's stream is the legacy
  * or per-thread default stream, where they are launched directly; three

@@ -540,12 +540,13 @@ class Context:
         """Pick the fastest FP32 sweep launch shape for this lattice (fa_autotune).
 
         With `cache` (a JSON file path), a choice stored for the same lattice
-        dimensions and GPU is applied without timing, and a new timing is stored.
+        dimensions and GPU is applied without timing, and a new timing is stored.  A
+        choice among other sweeps than today's (TUNE_SWEEPS) is timed again.
         Returns {"shape": k, "times_ms": [wide, narrow] or None, "cached": bool}."""
         key = tune_key(self.dims, _device_name())
         if cache is not None:
             entry = load_tune_cache(cache).get(key)
-            if entry is not None:
+            if entry is not None and entry.get("sweeps") == TUNE_SWEEPS:
                 self.set_hop_shape(int(entry["shape"]))
                 return {"shape": int(entry["shape"]), "times_ms": entry.get("times_ms"), "cached": True}
         times = (ctypes.c_double * SHAPE_NARROW)()
@@ -554,11 +555,16 @@ class Context:
             _check(rc, "fa_autotune")
         result = {"shape": int(rc), "times_ms": [float(t) for t in times], "cached": False}
         if cache is not None:
-            store_tune_cache(cache, key, {"shape": result["shape"], "times_ms": result["times_ms"]})
+            store_tune_cache(cache, key, {"shape": result["shape"], "times_ms": result["times_ms"], "sweeps": TUNE_SWEEPS})
         return result
 
 
 # ------------------------------------------------------------------ autotuner cache
+# The sweeps that the shapes of a cache entry stand for: 2, small lattices are timed
+# with two threads per site, as the solver runs them (entries without the field: one)
+TUNE_SWEEPS = 2
+
+
 def _device_name():
     import torch
     return torch.cuda.get_device_name(torch.cuda.current_device()) if torch.cuda.is_available() else "none"

@@ -579,8 +579,9 @@ int fa_set_hop_shape(fa_ctx* c, int shape) {
 
 int fa_get_hop_shape(const fa_ctx* c) { return c ? c->hop_shape : FA_EINVAL; }
 
-// Time each FP32 sweep launch shape on the context's lattice: chains of sweeps
-// g5 D_w(mu) that read the previous sweep's output (as in a solve), `reps`
+// Time each FP32 sweep launch shape on the context's lattice, as a solve with that
+// shape runs it (small lattices other than WIDE: two threads per site): chains of
+// sweeps g5 D_w(mu) that read the previous sweep's output (as in a solve), `reps`
 // launches between two CUDA events on the context's stream, three rounds with
 // the shapes interleaved, the best round per shape.  The automatic choice is
 // kept unless the other shape is faster by more than 3 % (single-launch timings
@@ -606,7 +607,7 @@ int fa_autotune(fa_ctx* c, int reps, double* times_ms) {
     c->hop_timing = false;
     auto chain = [&](int n) {
         for (int k = 0; k < n && rc == FA_OK; ++k)
-            rc = hop_f32(c, buf[k & 1], buf[(k + 1) & 1], nullptr, 1.0, false, true, false);
+            rc = hop_f32_solve(c, buf[k & 1], buf[(k + 1) & 1]);
     };
     // The solver replays its outer iterations from CUDA graphs, so the chains are
     // timed the same way where the stream can be captured (not the legacy or

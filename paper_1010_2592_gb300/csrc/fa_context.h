@@ -128,6 +128,9 @@ int hop_f64(fa_ctx* c, const View64& in, const View64& out, double scale, bool g
 // (result in `out`, or in the canonical field `canon` when that is not null)
 int hop_f32(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
             bool dagger_mu, bool after = false);
+// the plain FP32 sweep that a one-system solve with launch shape c->hop_shape runs, as an
+// ordinary launch (autotuner)
+int hop_f32_solve(fa_ctx* c, const float4* in, float4* out);
 int hop_df(fa_ctx* c, const float4* in, float4* out, double* canon, double scale, bool g5in, bool g5out,
            bool dagger_mu, bool after = false);
 int solve(fa_ctx* c, const double* b_canon, double* y_canon, double* const* xs_canon,

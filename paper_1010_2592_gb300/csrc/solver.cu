@@ -418,6 +418,19 @@ static bool hop32_split(int shape, int V) {
     return shape != FA_SHAPE_WIDE && (V + kSplitSites - 1) / kSplitSites <= kSplitBlocks * sms();
 }
 
+int hop_f32_solve(fa_ctx* c, const float4* in, float4* out) {
+    const int V = c->g.V;
+    if (!hop32_split(c->hop_shape, V)) return hop_f32(c, in, out, nullptr, 1.0, false, true, false);
+    const SpinorView<float> vin{const_cast<float4*>(in), V}, vout{out, V};
+    const SpinorView<float> none{nullptr, V};
+    launch_ex(false, 1, k_hop1_split<false>, dim3((V + kSplitSites - 1) / kSplitSites), 2 * kSplitSites, c->stream, c->g,
+              LinkView<float>{links32_of(c), V}, vin, vout, (float)(4.0 + c->mass), -0.5f, (float)std::exp(c->mu),
+              (float)std::exp(-c->mu), (float)c->t_bc, none, (double2*)nullptr, (const int*)nullptr,
+              (const SolverDev*)nullptr, ScalarStep{STEP_NONE, 0});
+    c->launches++;
+    return launch_status("k_hop1_split");
+}
+
 // Whether pass 1 defers the updates i < j of its sub-steps (vec_tile.cuh): always
 // for l > 2 (32^3 x 64, l = 4: the FP32 update kernels of an outer iteration took
 // 2.2 ms of 5.5).  At l = 2 there is one such pair to save per vector, against
