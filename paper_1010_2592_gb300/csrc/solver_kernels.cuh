@@ -443,7 +443,9 @@ __device__ __forceinline__ void acc_mr(const SolverDev& d, int m, const Ch<R> (&
 // writes nothing outside its own shared memory.  Only in launches of at most
 // about one wave (8 blocks per SM): in a longer launch a block that lingers
 // for its dry run holds back the blocks still waiting for a slot (the
-// 72-system batch, one launch for all systems, measured 3-10 % slower).
+// 72-system batch, one launch for all systems, measured 3-10 % slower; the
+// double-float Gram matrix with its row groups, us with / without: 16^3 x 32,
+// l = 8, 5 x 512 blocks 601 / 405, 32^3 x 64, l = 4, 3 x 1216 1002 / 995).
 constexpr unsigned kWarmTickets = 1024, kWarmSkip = 32;
 enum { LB_NONE = 0, LB_WARM = 1, LB_LAST = 2 };
 __device__ __forceinline__ unsigned sm_count_dev() {
@@ -464,7 +466,7 @@ __device__ __forceinline__ int last_block(DevState* S, int ntickets) {
         const unsigned t = atomicAdd(&S->ticket, 1u);
         // (the last kWarmSkip before the last block run no dry run: they would
         // end after it on an SM whose code is still cold)
-        const bool one_wave = gridDim.x * gridDim.y <= 8u * sm_count_dev();
+        const bool one_wave = (unsigned long long)gridDim.x * gridDim.y * gridDim.z <= 8u * sm_count_dev();
         is_last = t == (unsigned)ntickets - 1u ? LB_LAST
                   : (one_wave && t + kWarmTickets >= (unsigned)ntickets && t + 1u + kWarmSkip < (unsigned)ntickets
                          ? LB_WARM
