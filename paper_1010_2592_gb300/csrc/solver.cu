@@ -456,8 +456,8 @@ static void set_forms64(Batch& B) {
         ns = std::max(ns, B.sys[i]->ns);
     }
     B.site64 = hop64_by_site(blocks, sms());
-    B.site64_vec = B.sites >= (double)kSite64Min * sms();
-    B.site64_shifts = B.site64_vec && ns <= kFewShifts;
+    B.site64_vec = B.sites >= (double)site64_min(B.Lo.L) * sms();
+    B.site64_shifts = B.sites >= 1.25 * kThreads * sms() && ns <= kFewShifts;
     B.site64_mr_shifts = B.site64_shifts && B.sites >= 3.0 * kThreads * sms() && full_waves(B.sites / kThreads, sms());
 }
 

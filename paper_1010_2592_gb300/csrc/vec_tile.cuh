@@ -530,20 +530,20 @@ k_mr_tile(const SolverDev* __restrict__ ds, int pass2, ScalarStep step, const in
 }
 
 // ------------------------------------------------------------------ FP64, a thread per site
-// From kSite64Min sites per SM on (a wave and a quarter of 256-thread blocks) there is
-// FP64 work for every SM without a split by component and chain, and the tile
+// From site64_min sites per SM on (a wave and a quarter of 256-thread blocks, half of
+// that for the few products of l <= 2) there is FP64 work for every SM without a split by component and chain, and the tile
 // kernels lose to their barriers, to products formed from vectors loaded once per
 // chain, and to the few blocks that 148 registers x 384 threads leave.  The same
 // chains in the same order: the same bits.  Measured on GB300 (tracer, us per launch,
 // l = 2, tiles / a thread per site): Gram matrix 32^3 x 64 1522 / 776, 16^3 x 32 196 /
-// 92, 41,472 sites 69 / 50, 16,384 32 / 29; MR step of a double pass 1851 / 1136,
-// 158 / 101, 55 / 53, 24 / 29; k_update_shifts64 with 8 shifts (W = 32 / 256) 10444 /
+// 92, 41,472 sites 69 / 50, 24,576 44 / 29, 16,384 32 / 29; MR step of a double pass 1851 /
+// 1136, 158 / 101, 55 / 53, 34 / 30, 24 / 29 (l = 4 at 24,576 sites: 52 / 69); k_update_shifts64 with 8 shifts (W = 32 / 256) 10444 /
 // 9183, 628 / 585, 198 / 187, 78 / 87.  At l = 8 and 41,472 sites they draw (507 / 511,
 // 119 / 126).  With many shifts a warp per shift is even or better (16^3 x 32, 24
 // shifts: 1661 / 1692), as is the tile form of the single-pass MR step (1386 / 1627),
 // whose site form takes whole waves of one block per SM (8 shifts: 155,648 sites, 4.0
 // waves, 660 / 616; 196,608, 5.05, 832 / 892; 32^3 x 64 8568 / 7940).
-constexpr int kSite64Min = 320;
+constexpr int site64_min(int L) { return L <= 2 ? 160 : 320; }
 constexpr int kFewShifts = 16;
 
 // the Gram matrix

@@ -12,9 +12,9 @@ pytestmark = pytest.mark.gpu
 
 
 # on a 152-SM part: two systems of 74 blocks of 128 sites (148 of 152 SMs; ragged tile and
-# block): the sweep; two of 26,364 sites: the Gram matrix, the MR step of a double pass and
-# the updates with shifts; four of 37,349 (3.84 waves of 256 sites): the MR step with shifts
-@pytest.mark.parametrize("dims,nsys", [((13, 13, 7, 8), 2), ((13, 13, 13, 12), 2), ((13, 17, 13, 13), 4)])
+# block): the sweep; two of 13,520 (l <= 2) and of 26,364 sites: the Gram matrix and the MR step of
+# a double pass, at 26,364 the updates with shifts; four of 37,349 (3.84 waves of 256 sites): the MR step with shifts
+@pytest.mark.parametrize("dims,nsys", [((13, 13, 7, 8), 2), ((13, 13, 8, 10), 2), ((13, 13, 13, 12), 2), ((13, 17, 13, 13), 4)])
 @pytest.mark.parametrize("mode,ell,ns", [("double", 1, 4), ("double", 2, 4), ("pseudo", 4, 4), ("double", 8, 2),
                                          ("single", 1, 16), ("single", 2, 3), ("single", 2, 17), ("single", 4, 2)])
 def test_site_forms_equal_tile_forms(dims, nsys, mode, ell, ns):
