@@ -388,7 +388,7 @@ int fa_hop_timing_reset(fa_ctx* ctx);
 typedef struct {
     unsigned long long t_start_ns, t_end_ns;   /* %globaltimer at block entry / exit */
     int kernel;
-    int block;                                 /* blockIdx.x + gridDim.x * blockIdx.y */
+    int block;                                 /* blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) */
     int sm;
     int grid;                                  /* blocks of the launch */
 } fa_trace_record;

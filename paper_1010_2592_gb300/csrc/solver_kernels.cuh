@@ -1568,7 +1568,8 @@ k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups
            int in_sel, int in_j, int out_sel, int out_j, int second, int pass2, ScalarStep step) {
     constexpr int NT = kHopNarrowThreads, NW = NT / 32;
     dep_wait();
-    const TraceScope trace_(trace_kind<float>(FA_TK_HOP_MRHS, DOT));
+    TraceScope trace_(trace_kind<float>(FA_TK_HOP_MRHS, DOT));
+    bool ran = false;
     const int4 it = items[blockIdx.x];
     const GroupDev& G = groups[it.x];
     const int tile = it.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1577,6 +1578,7 @@ k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups
     for (int r = it.z; r < it.w; ++r) {
         const SolverDev& d = ds[G.sys[r]];
         if (sys_idle(d, pass2)) continue;   // the same for every thread of the block
+        ran = true;
         const int s = tile * NT + (int)threadIdx.x;
         cx<float> dres = czero<float>();
         if (s < d.V) {
@@ -1604,6 +1606,7 @@ k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups
             if (lane == 0) sums[r - it.z][warp] = make_float2(a, b);
         }
     }
+    if (!ran) trace_.drop();
     if constexpr (DOT) {
         dep_launch();
         const int nr = it.w - it.z;

@@ -58,8 +58,10 @@ struct TraceScope {
     __device__ __forceinline__ explicit TraceScope(int k) : t0(0ull), kind(k) {
         if (threadIdx.x == 0) t0 = global_ns();
     }
+    // leave no record (the block found nothing to do)
+    __device__ __forceinline__ void drop() { kind = -1; }
     __device__ __forceinline__ ~TraceScope() {
-        if (threadIdx.x != 0) return;
+        if (threadIdx.x != 0 || kind < 0) return;
         const TraceState ts = g_trace;
         if (ts.rec == nullptr) return;
         const unsigned long long t1 = global_ns();
