@@ -314,7 +314,8 @@ int fa_estimate_scale(fa_ctx* c, const double* v0, int iters, double* scale_out)
     return estimate_scale(c, v0, iters, scale_out);
 }
 
-// canonical in -> internal (FP64 or FP32), one or two hops, -> canonical out
+// One or two hops between canonical fields: FP64 reads `in` itself, FP32 and
+// double-float a packed copy; the last sweep writes `out`.
 static int apply_op(fa_ctx* c, const double* in, double* out, int dagger, int precision, bool is_A) {
     if (!c || !in || !out || in == out) return FA_EINVAL;
     if (!c->have_gauge || !c->have_params) return FA_ESTATE;
@@ -330,6 +331,13 @@ static int apply_op(fa_ctx* c, const double* in, double* out, int dagger, int pr
             const View64 t = internal64(c->tmp64.as<double2>(), V);
             TRY(hop_f64(c, canonical64(in), t, 1.0, false, true, dg));
             TRY(hop_f64(c, t, canonical64(out), c->scale_c, false, true, dg, true));
+        } else if (in < out + 24 * (size_t)V && out < in + 24 * (size_t)V) {
+            // fields that overlap: the sweep reads neighbours of what it writes, so from a copy
+            CUDA_OR(c->io64a.ensure(b), "alloc");
+            double2* a = c->io64a.as<double2>();
+            TRY(launch_pack_spinor_f64(c->g, in, a, st));
+            c->launches += 1;
+            TRY(hop_f64(c, internal64(a, V), canonical64(out), 1.0, dg, dg, dg));
         } else {
             TRY(hop_f64(c, canonical64(in), canonical64(out), 1.0, dg, dg, dg));
         }
