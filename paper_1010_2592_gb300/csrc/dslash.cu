@@ -11,7 +11,7 @@
 // colour vectors by the link and rebuilds the lower spin components.
 //
 // FP32: one thread per site; double-float: three, one per colour row; FP64: 32-site
-// tiles, a warp per hop (hop64.cuh).  The nearest-neighbour reuse of spinors and links is
+// tiles, a warp per hop, or one thread per site (hop64.cuh).  The nearest-neighbour reuse of spinors and links is
 // left to L1/L2 (the 126 MB L2 holds several time slices of every field even
 // on 32^3 x 64).  Memory traffic floor per site and sweep: one spinor in, one
 // out, four links (FP32: 96 + 96 + 4 * 48 = 384 B).
@@ -21,7 +21,8 @@
 namespace fa {
 
 // FP32.  CANON: the result is written to the canonical field `canon` instead of
-// `out`, each warp turning its 32 records of 192 bytes round in shared memory.
+// `out`: each thread stores its record of 192 bytes itself, 32 bytes at a time
+// where the field is 32-byte aligned, else 16.
 template <bool G5IN, bool G5OUT, bool CANON, int NT, int MB>
 __global__ void __launch_bounds__(NT, MB)
 hop_kernel(Geom g, LinkView<float> U, SpinorView<float> in, SpinorView<float> out, double2* canon, float cdiag,

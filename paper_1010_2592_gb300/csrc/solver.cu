@@ -1158,7 +1158,7 @@ static int build_tables(Batch& B) {
     return FA_OK;
 }
 
-// ------------------------------------------------------------------ the solve (a batch of n systems)// ------------------------------------------------------------------ the solve (a batch of n systems)
+// ------------------------------------------------------------------ the solve (a batch of n systems)
 int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* const* y_canon, double* const* xs_canon,
                 const fa_solver_params* p, fa_solver_stats* stats) {
     if (n < 1 || !ctxs || !b || !p) return FA_EINVAL;
@@ -1168,11 +1168,6 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
         if (!c || !b[i]) return FA_EINVAL;
         if (!c->have_gauge || !c->have_params || !c->have_poles) return FA_ESTATE;
         if (c->device != c0->device) return FA_EINVAL;
-    }
-    bool same_shape = true;
-    for (int i = 0; i < n; ++i) {
-        const Geom& g = ctxs[i]->g;
-        same_shape = same_shape && g.X == c0->g.X && g.Y == c0->g.Y && g.Z == c0->g.Z && g.T == c0->g.T;
     }
     const int L = p->ell;
     if (!(L == 1 || L == 2 || L == 3 || L == 4 || L == 8)) return FA_EINVAL;
@@ -1260,7 +1255,6 @@ int solve_batch(fa_ctx* const* ctxs, int n, const double* const* b, double* cons
     // share one gauge field and shape) so that a block's right-hand sides read
     // its tile's links once.
     if (n > 1) FA_TRY(build_tables(B));
-    (void)same_shape;
     cudaStream_t st = c0->stream;
     const bool timing = (p->flags & 1) != 0;
     c0->hop_timing = (p->flags & 2) != 0;

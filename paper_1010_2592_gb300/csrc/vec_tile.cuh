@@ -292,7 +292,7 @@ k_update_r64(const SolverDev* __restrict__ ds, int j, int pass2, const int4* tab
 
 // The same with shift vectors (single pass), W pairs per block.  W = 32: warp 0
 // updates r, and warp w the vectors of the shifts w, w + 8, ...  W = 256: a thread
-// takes a pair through all shifts (rule: k_update_shifts64's launch).  The r before
+// takes a pair through all shifts (rule: set_forms64 in solver.cu).  The r before
 // the update stay in shared memory.
 template <int W>
 __global__ void __launch_bounds__(kFlat)
@@ -349,7 +349,8 @@ k_update_shifts64(const SolverDev* __restrict__ ds, int j, const int4* tab) {
 // imaginary part of one product); l <= 2 needs no imaginary part of the
 // diagonal.  Last block: the MR coefficients, and with `shifts` their shift part.
 // Measured on GB300 (tracer, us per launch, one thread per site with all
-// products -> this): l = 2, 8^3 x 16 30 -> 8.7.
+// products -> this): l = 2, 8^3 x 16 30 -> 8.7.  (Nine warps and two blocks per SM, 113
+// registers instead of 148: 32^3 x 64 1522 -> 1347, 8^3 x 16 11 -> 21.)
 constexpr int kGramWarps = 12;
 template <int L>
 __global__ void __launch_bounds__(32 * kGramWarps)
