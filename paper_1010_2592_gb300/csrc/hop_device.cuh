@@ -143,12 +143,11 @@ __device__ __forceinline__ void hop_site(const Geom& g, const LinkView<R>& U, co
     const int t = r2 / Z;
     const int sY = X, sZ = X * Y, sT = X * Y * Z;
     cx<R> acc[12];
-    const int xp = (x == X - 1) ? s - (X - 1) : s + 1;
     if constexpr (std::is_same<R, double>::value) {
         // the first term set, not added to zero: 24 of 936 FP64 instructions less, and the
         // sign of a zero as the tile form has it (hop64.cuh)
         cx<R> c[6];
-        hop_fwd_rows<0, false, G5IN>(c, in, U, s, xp, R(1));
+        hop_fwd_rows<0, false, G5IN>(c, in, U, s, (x == X - 1) ? s - (X - 1) : s + 1, R(1));
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             acc[k] = c[k];
@@ -159,7 +158,7 @@ __device__ __forceinline__ void hop_site(const Geom& g, const LinkView<R>& U, co
     } else {
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[k] = czero<R>();
-        hop_fwd<0, false, G5IN>(acc, in, U, s, xp, R(1));
+        hop_fwd<0, false, G5IN>(acc, in, U, s, (x == X - 1) ? s - (X - 1) : s + 1, R(1));
     }
     hop_bwd<0, false, G5IN>(acc, in, U, (x == 0) ? s + (X - 1) : s - 1, R(1));
     hop_fwd<1, false, G5IN>(acc, in, U, s, (y == Y - 1) ? s - (Y - 1) * sY : s + sY, R(1));

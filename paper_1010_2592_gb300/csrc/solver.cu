@@ -496,13 +496,13 @@ static int enqueue_outer(Batch& B, bool pass2, bool single, bool head, bool reli
     const SolverDev& h0 = B.host[0];
     auto vsel = [&](int sel, int j) -> T* {
         constexpr bool wide = rp_of<R>() != RP32;   // FP64 and double-float use the wide buffers
-        if (sel == 3 && j == L - 1) sel = 1, j = L;   // rb_at
         T* base = wide ? (T*)(sel == 0 ? (void*)h0.u64 : sel == 1 ? (void*)h0.r64 : sel == 2 ? (void*)h0.tmp64 : (void*)h0.rb64)
                        : (T*)(sel == 0 ? (void*)h0.u32 : sel == 1 ? (void*)h0.r32 : sel == 2 ? (void*)h0.tmp32 : (void*)h0.rb32);
         return base + (size_t)j * (size_t)Ch<R>::N * h0.V;
     };
     const ScalarStep none{STEP_NONE, 0};
     auto hop = [&](int in_sel, int in_j, int out_sel, int out_j, int second, bool dot, ScalarStep step) -> int {
+        if (in_sel == 3 && in_j == L - 1) in_sel = 1, in_j = L;   // rb_{l-1} is in r_l (rb_at)
         if (timing) hop_timing_begin(c, kind + (dot ? 3 : 0));
         if (n == 1) {
             const T* rt = rp_of<R>() != RP32 ? (const T*)(const void*)h0.rt64 : (const T*)(const void*)h0.rt32;

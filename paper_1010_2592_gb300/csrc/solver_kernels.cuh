@@ -1373,8 +1373,7 @@ k_dot2_sys(const SolverDev* __restrict__ ds, double tol, double theta, const int
 // partials of <rt, out> into the system's partial buffer.
 template <typename R>
 __device__ __forceinline__ typename Ch<R>::T* select_vec(const SolverDev& d, int sel, int j) {
-    if (sel == 3) return rb_at<R>(d, j);
-    typename Ch<R>::T* base = sel == 0 ? Vec<R>::u(d) : sel == 1 ? Vec<R>::r(d) : Vec<R>::tmp(d);
+    typename Ch<R>::T* base = sel == 0 ? Vec<R>::u(d) : sel == 1 ? Vec<R>::r(d) : sel == 2 ? Vec<R>::tmp(d) : Vec<R>::rb(d);
     return base + (size_t)j * vstride<R>(d);
 }
 
@@ -1568,17 +1567,22 @@ k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups
            int in_sel, int in_j, int out_sel, int out_j, int second, int pass2, ScalarStep step) {
     constexpr int NT = kHopNarrowThreads, NW = NT / 32;
     dep_wait();
-    TraceScope trace_(trace_kind<float>(FA_TK_HOP_MRHS, DOT));
-    bool ran = false;
     const int4 it = items[blockIdx.x];
     const GroupDev& G = groups[it.x];
+    // no record of a block that finds all its systems finished (looked up while tracing only:
+    // a flag kept through the loop below cost 20 bytes of spills and 0.8 % of a batch)
+    if (trace_on()) {
+        bool idle = true;
+        for (int r = it.z; r < it.w; ++r) idle = idle && sys_idle(ds[G.sys[r]], pass2);
+        if (idle) return;
+    }
+    const TraceScope trace_(trace_kind<float>(FA_TK_HOP_MRHS, DOT));
     const int tile = it.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ float2 sums[DOT ? kMaxRhs : 1][NW];
     __shared__ int lasts[DOT ? kMaxRhs : 1];
     for (int r = it.z; r < it.w; ++r) {
         const SolverDev& d = ds[G.sys[r]];
         if (sys_idle(d, pass2)) continue;   // the same for every thread of the block
-        ran = true;
         const int s = tile * NT + (int)threadIdx.x;
         cx<float> dres = czero<float>();
         if (s < d.V) {
@@ -1606,7 +1610,6 @@ k_hop_mrhs(const SolverDev* __restrict__ ds, const GroupDev* __restrict__ groups
             if (lane == 0) sums[r - it.z][warp] = make_float2(a, b);
         }
     }
-    if (!ran) trace_.drop();
     if constexpr (DOT) {
         dep_launch();
         const int nr = it.w - it.z;

@@ -52,16 +52,16 @@ template <typename R> constexpr int trace_kind(int id, bool variant = false) {
     return id | (trace_prec<R>() << 8) | ((variant ? 1 : 0) << 10);
 }
 
+__device__ __forceinline__ bool trace_on() { return g_trace.rec != nullptr; }
+
 struct TraceScope {
     unsigned long long t0;
     int kind;
     __device__ __forceinline__ explicit TraceScope(int k) : t0(0ull), kind(k) {
         if (threadIdx.x == 0) t0 = global_ns();
     }
-    // leave no record (the block found nothing to do)
-    __device__ __forceinline__ void drop() { kind = -1; }
     __device__ __forceinline__ ~TraceScope() {
-        if (threadIdx.x != 0 || kind < 0) return;
+        if (threadIdx.x != 0) return;
         const TraceState ts = g_trace;
         if (ts.rec == nullptr) return;
         const unsigned long long t1 = global_ns();
