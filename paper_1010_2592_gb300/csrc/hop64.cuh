@@ -3,8 +3,9 @@
 // What bounds it: the FP64 pipe.  A GB300 SM takes one FP64 warp instruction every 19
 // cycles while its four sub-partitions all ask (add, multiply or FMA, dependent or not:
 // 76 cycles per sub-partition, 0.53 T thread instructions/s at 2.06 GHz); a
-// sub-partition alone gets one every 64.  A sweep takes 912 FP64 instructions per
-// site, so that rate makes 227 us on 16^3 x 32 whatever the memory does (126 MB
+// sub-partition alone gets one every 64.  A sweep takes 992 FP64 warp instructions
+// per 32 sites here (ncu; 914 with a thread per site), so it takes 230 us on 16^3 x 32
+// (17.6 cycles each) whatever the memory does (126 MB
 // there: 19 us), and one warp that walks a whole site takes 28 us even on an idle
 // chip.  One thread per site in 256-thread blocks put a 4^3 x 8 lattice on 2 of 152
 // SMs (50-60 us per sweep) and left 3.4 waves of one block per SM on 16^3 x 32
@@ -269,10 +270,10 @@ inline int hop64_split(int V, int nsm) {
 }
 
 // A thread per site instead (hop_site in hop_device.cuh; the same bits), in blocks of
-// 128 threads at 255 registers: 912 FP64 instructions per site too, but the SM's
-// FP64 pipe takes one of its warp instructions every 17.5 cycles, of the tile form's
-// every 19.1 (a probe: 19.0 when all four sub-partitions ask at once, 16 would be its
-// best), and a wave of one block per SM (19,456 sites) takes 31.2 us however few
+// 128 threads at 255 registers: 914 FP64 warp instructions per 32 sites against the
+// tile form's 992 (ncu), both at about 17.5 cycles of the SM's pipe (a probe: 19.0
+// when all four sub-partitions ask in step, 16 would be its best); but a wave of
+// one block per SM (19,456 sites) takes 31.2 us however few
 // of its blocks there are, where the tile form takes 1.75 ns per site.  So it is
 // used where the last wave is full enough (the busiest SM's blocks against the
 // mean).  Measured on GB300, us per sweep, tiles / a thread per site: 32^3 x 64

@@ -144,7 +144,7 @@ __device__ __forceinline__ void hop_site(const Geom& g, const LinkView<R>& U, co
     const int sY = X, sZ = X * Y, sT = X * Y * Z;
     cx<R> acc[12];
     if constexpr (std::is_same<R, double>::value) {
-        // the first term set, not added to zero: 24 of 936 FP64 instructions less, and the
+        // the first term set, not added to zero: 24 FP64 instructions of 936 less, and the
         // sign of a zero as the tile form has it (hop64.cuh)
         cx<R> c[6];
         hop_fwd_rows<0, false, G5IN>(c, in, U, s, (x == X - 1) ? s - (X - 1) : s + 1, R(1));
